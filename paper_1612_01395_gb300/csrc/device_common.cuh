@@ -6,12 +6,13 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "dots.cuh"
 #include "pbicgstab.h"
 
 namespace pbcg {
 
-constexpr int kTPB = 128;          // threads per block of every kernel here
-constexpr int kMaxGrid = 2048;     // upper bound on thread blocks (sizes the partial-sum slots)
+constexpr int kTPB = 128;          // threads per block of the cluster, batched and mixed-precision kernels
+constexpr int kMaxGrid = 2040;     // upper bound on thread blocks (kPartialBytes holds their slots)
 constexpr int kMaxDots = 8;        // dot products carried by one reduction
 constexpr uint64_t kSyncTimeoutNs = 4000000000ull;   // 4 s per grid-wide wait
 
@@ -45,9 +46,11 @@ struct Control {
 };
 static_assert(sizeof(Control) <= 256, "control block must fit 256 bytes");
 constexpr size_t kControlBytes = 256;
-// 3 rotating buffers of one 8-double slot per block, then 3 rotating 8-double
-// totals; rounded up to 256 bytes so the vectors after it stay 256-byte aligned
-constexpr size_t kPartialBytes = ((3ull * kMaxGrid + 3) * 8 * sizeof(double) + 255) / 256 * 256;
+// 3 rotating buffers of one 8-double slot per block, then 3 rotating records of
+// 16 doubles; a multiple of 256 bytes, so the vectors after it stay 256-byte aligned
+constexpr size_t kPartialBytes = 393472;
+static_assert((3ull * kMaxGrid * 8 + 3 * 16) * sizeof(double) <= kPartialBytes && kPartialBytes % 256 == 0,
+              "slots and records fit");
 
 // n / d for 0 <= n < 2^31 and 1 <= d < 2^31 by one multiply-high: the
 // round-up method of Granlund & Montgomery, "Division by invariant integers
@@ -125,29 +128,50 @@ __device__ __forceinline__ void warp_allsum(double (&v)[K]) {
     }
 }
 
-// Fixed-order block sum; every thread receives the K results. sm: [kMaxDots][32].
-// Warps reduce independently, then lane k of every warp adds value k of the
-// warps in warp order and shuffles it to the other lanes.
-template <int K>
-__device__ __forceinline__ void block_sum(double (&v)[K], double (*sm)[32]) {
-    constexpr int kWarps = kTPB / 32;
-    warp_allsum<K>(v);
-    if (kWarps == 1) return;
+// What the threads of a block share in an exchange. Every field after `part`
+// is the same in all blocks of a solve once an exchange has completed.
+struct alignas(16) Scalars {
+    double alpha, beta, omega, rho, r0s, r0z;   // of the iteration
+    double nr;          // squared norm tested last
+    double nr0, tol, bound;   // ||r_0||, the tolerance, the squared norms it can accept
+    double aux;         // total of an exchange outside the iteration
+    int action, status;   // what the loop does next (kGo, kHalf, kStop); pbcg_status of a stop
+};
+constexpr int kScalarWords = sizeof(Scalars) / 8;
+static_assert(kScalarWords <= 16, "the scalars fit one published record");
+enum { kGo = 0, kHalf = 1, kStop = 2 };
+
+template <int T>   // most threads of the block
+struct Exchange {
+    double part[T / 32][kMaxDots];   // the warps' sums
+    Scalars s;
+    int ok;     // cleared when a wait is abandoned, never set again: a slow thread cannot read a later value
+    int last;
+};
+
+// Fixed-order block sums, returned to every lane of warp 0: the warps reduce
+// independently, then lane k of warp 0 adds value k of the warps in warp order.
+template <int K, int T>
+__device__ __forceinline__ void block_sum(double (&v)[K], Exchange<T> &X) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    warp_allsum<K>(v);
     if (lane == 0) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) sm[k][wid] = v[k];
+        for (int k = 0; k < K; ++k) X.part[wid][k] = v[k];
     }
     __syncthreads();
-    double t = 0.0;
-    if (lane < K) {
-        t = sm[lane][0];
+    if (wid == 0) {
+        double t = 0.0;
+        if (lane < K) {
+            t = X.part[0][lane];
+            const int warps = (int)(blockDim.x >> 5);
 #pragma unroll
-        for (int w = 1; w < kWarps; ++w) t += sm[lane][w];
+            for (int w = 1; w < T / 32; ++w)
+                if (w < warps) t += X.part[w][lane];
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] = __shfl_sync(kFull, t, k);
     }
-#pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = __shfl_sync(kFull, t, k);
-    __syncthreads();
 }
 
 // Grid-wide exchange of a cooperative launch. Each block owns one 64-byte
@@ -157,13 +181,13 @@ __device__ __forceinline__ void block_sum(double (&v)[K], double (*sm)[32]) {
 // __syncthreads, is ordered before the arrival) and adds 1 to the arrival
 // counter. Then, by grid size:
 //  * small grids: thread 0 spins on the counter until all blocks of exchange
-//    e arrived, and every block adds all slots in the same fixed order;
+//    e arrived, every block adds all slots in the same fixed order, and its
+//    warp 0 forms the scalars;
 //  * large grids (at least kLastReduceGrid blocks): the block whose arrival
-//    completes the count adds all slots (same fixed order), publishes the K
-//    totals and raises `ready`; the others spin on `ready` and read the
-//    totals. Every block adding every slot costs each SM (blocks per SM x
-//    blocks x K) FP64 additions per exchange -- about 12 us of its FP64 pipe
-//    at 1216 blocks -- against one extra flag hop.
+//    completes the count adds all slots (same fixed order), forms the scalars,
+//    publishes them and raises `ready`; the others spin on `ready` and read
+//    them. Every block adding every slot costs each SM (blocks per SM x
+//    blocks x K) FP64 additions per exchange against one extra flag hop.
 // One poller per block on one word: polling all slots from every thread
 // congests the L2 and was measured slower. The rotation keeps a slot or a
 // total from being rewritten while a slow block may still read it (exchange
@@ -176,17 +200,19 @@ constexpr int kLastReduceGrid = 512;
 
 struct GridSync {
     Control *ctl;
-    double *slots;      // [3][gridDim.x][kSlotDoubles], then [3][kSlotDoubles] totals
+    double *slots;      // [3][gridDim.x][kSlotDoubles], then [3][16]: the scalars of an exchange
     unsigned epoch;     // exchanges done by this block
     int count;          // exchanges performed (for diagnostics)
+    int step;           // distance between a thread's rows
     uint64_t limit_ns = kSyncTimeoutNs;   // bound on each wait
 };
+__device__ __forceinline__ int row_step(const GridSync &g) { return g.step; }
 
 __device__ __forceinline__ double *slot_ptr(const GridSync &g, unsigned buf, int block) {
     return g.slots + ((size_t)buf * gridDim.x + block) * kSlotDoubles;
 }
 __device__ __forceinline__ double *totals_ptr(const GridSync &g, unsigned buf) {
-    return g.slots + ((size_t)3 * gridDim.x + buf) * kSlotDoubles;
+    return g.slots + (size_t)3 * gridDim.x * kSlotDoubles + (size_t)buf * 16;
 }
 __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -210,46 +236,44 @@ __device__ __forceinline__ bool wait_at_least(GridSync &g, const unsigned *word,
     return true;
 }
 
-// *sflag (shared, set to 1 once at kernel start) only ever goes from 1 to 0:
-// thread 0 clears it when a wait is abandoned, and every thread returns its
-// value after the barrier that follows. Never resetting it keeps a slow thread
-// from reading a later exchange's value.
-
 // Barrier without data.
-__device__ __forceinline__ bool grid_sync(GridSync &g, double (*)[32], int *sflag) {
+template <int T>
+__device__ __forceinline__ bool grid_sync(GridSync &g, Exchange<T> &X) {
     __syncthreads();   // every thread's stores of this phase precede thread 0's fence
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(&g.ctl->arrivals, 1u);
-        if (!wait_at_least(g, &g.ctl->arrivals, (g.epoch + 1u) * gridDim.x)) *sflag = 0;
+        if (!wait_at_least(g, &g.ctl->arrivals, (g.epoch + 1u) * gridDim.x)) X.ok = 0;
         __threadfence();
     }
     __syncthreads();
     g.epoch++;
     g.count++;
-    return *sflag != 0;
+    return X.ok != 0;
 }
 
-// Fixed-order sum over all slots of buffer buf, returned in every thread.
-template <int K>
-__device__ __forceinline__ void sum_slots(const GridSync &g, unsigned buf, double (&v)[K], double (*sm)[32]) {
+// Fixed-order sum over all slots of buffer buf, returned to every lane of warp 0.
+template <int K, int T>
+__device__ __forceinline__ void sum_slots(const GridSync &g, unsigned buf, double (&v)[K], Exchange<T> &X) {
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += kTPB) {
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += (int)blockDim.x) {
         const double *src = slot_ptr(g, buf, b);
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] += __ldcg(src + k);
     }
-    block_sum<K>(v, sm);
+    block_sum(v, X);
 }
 
-// Barrier that also returns, in every thread of every block, the same
-// fixed-order sum over the grid of the K per-thread values v.
-template <int K>
-__device__ __forceinline__ bool grid_sum(GridSync &g, double (&v)[K], double (*sm)[32], int *sflag) {
-    static_assert(K <= kSlotDoubles, "at most 8 values per exchange");
-    __shared__ int last;
-    block_sum<K>(v, sm);   // ends with __syncthreads
+// Barrier that adds the K values v of all threads of the grid in a fixed order
+// and lets `f` turn the totals into the loop's scalars: f(scalars, totals) runs
+// on one warp (all lanes alike) of every block, or of the last block to arrive,
+// and every thread of every block finds the same result in X.s afterwards.
+template <int K, int T, class F>
+__device__ __forceinline__ bool exchange(GridSync &g, double (&v)[K], Exchange<T> &X, F f) {
+    static_assert(K <= kSlotDoubles, "the values fit a slot");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    block_sum(v, X);
     const unsigned buf = g.epoch % 3u;
     const unsigned target = (g.epoch + 1u) * gridDim.x;
     const bool by_last = gridDim.x >= (unsigned)kLastReduceGrid;
@@ -259,38 +283,42 @@ __device__ __forceinline__ bool grid_sum(GridSync &g, double (&v)[K], double (*s
         for (int k = 0; k < K; ++k) out[k] = v[k];
         __threadfence();
         const unsigned before = atomicAdd(&g.ctl->arrivals, 1u);
-        last = before == target - 1u;
+        X.last = before == target - 1u;
         if (!by_last) {
-            if (!wait_at_least(g, &g.ctl->arrivals, target)) *sflag = 0;
+            if (!wait_at_least(g, &g.ctl->arrivals, target)) X.ok = 0;
         }
         __threadfence();
     }
     __syncthreads();
     if (!by_last) {
-        sum_slots<K>(g, buf, v, sm);
-    } else if (last) {
-        sum_slots<K>(g, buf, v, sm);   // every slot is visible: all blocks fenced before arriving
-        if (threadIdx.x == 0) {
+        sum_slots(g, buf, v, X);
+        if (wid == 0) f(X.s, v);
+    } else if (X.last) {   // every slot is visible: all blocks fenced before arriving
+        sum_slots(g, buf, v, X);
+        if (wid == 0) {
+            f(X.s, v);
+            __syncwarp();
             double *tot = totals_ptr(g, buf);
-#pragma unroll
-            for (int k = 0; k < K; ++k) tot[k] = v[k];
-            __threadfence();
-            st_release_u32(&g.ctl->ready, g.epoch + 1u);
+            if (lane < kScalarWords) tot[lane] = reinterpret_cast<const double *>(&X.s)[lane];
+            __syncwarp();
+            if (lane == 0) {
+                __threadfence();
+                st_release_u32(&g.ctl->ready, g.epoch + 1u);
+            }
         }
-    } else {
-        if (threadIdx.x == 0) {
-            if (!wait_at_least(g, &g.ctl->ready, g.epoch + 1u)) *sflag = 0;
+    } else if (wid == 0) {
+        if (lane == 0) {
+            if (!wait_at_least(g, &g.ctl->ready, g.epoch + 1u)) X.ok = 0;
             __threadfence();
         }
-        __syncthreads();
+        __syncwarp();
         const double *tot = totals_ptr(g, buf);
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = __ldcg(tot + k);
+        if (lane < kScalarWords) reinterpret_cast<double *>(&X.s)[lane] = __ldcg(tot + lane);
     }
     g.epoch++;
     g.count++;
-    __syncthreads();   // `last` is rewritten by the next exchange
-    return *sflag != 0;
+    __syncthreads();
+    return X.ok != 0;
 }
 
 // Synchronisation policy of a solve owned by one thread block (batched
@@ -301,17 +329,21 @@ struct BlockSync {
 };
 
 __device__ __forceinline__ bool is_leader(const BlockSync &) { return true; }
+__device__ __forceinline__ int row_step(const BlockSync &) { return kTPB; }
 
-__device__ __forceinline__ bool grid_sync(BlockSync &g, double (*)[32], int *) {
+template <int T>
+__device__ __forceinline__ bool grid_sync(BlockSync &g, Exchange<T> &) {
     __syncthreads();
     g.count++;
     return true;
 }
 
-template <int K>
-__device__ __forceinline__ bool grid_sum(BlockSync &g, double (&v)[K], double (*sm)[32], int *) {
-    block_sum<K>(v, sm);   // its __syncthreads also orders the block's stores of the phase
+template <int K, int T, class F>
+__device__ __forceinline__ bool exchange(BlockSync &g, double (&v)[K], Exchange<T> &X, F f) {
+    block_sum(v, X);   // its barrier also orders the block's stores of the phase
+    if (threadIdx.x < 32) f(X.s, v);
     g.count++;
+    __syncthreads();
     return true;
 }
 
@@ -418,15 +450,13 @@ __device__ __forceinline__ void st_cluster_s32(uint32_t addr, int v) {
 // Synchronisation policy of a solve shared by the `size` CTAs of a cluster:
 // a barrier is the cluster barrier; a reduction pushes each CTA's K block sums
 // into slot [rank] of EVERY CTA's slot array (distributed shared memory,
-// posted stores), crosses the barrier, and then each warp of each CTA adds the
-// `size` slots of its own shared memory with the same fixed-order warp
-// reduction -- the same additions in the same order everywhere, so all CTAs
-// (and all warps) hold identical scalars, with no remote loads on the
-// critical path and no block barrier after the sum. Slot arrays alternate
-// between two buffers: buffer e % 2 is rewritten by exchange e + 2, which a
-// CTA starts only after the barrier of exchange e + 1, which every thread of
-// every CTA reaches only after it has read exchange e. Same interface as
-// GridSync and BlockSync.
+// posted stores), crosses the barrier, and then warp 0 of each CTA adds the
+// `size` slots of its own shared memory and forms the scalars -- the same
+// additions in the same order everywhere, so all CTAs hold identical scalars, with no remote
+// loads on the critical path. Slot arrays alternate between two buffers:
+// buffer e % 2 is rewritten by exchange e + 2, which a CTA starts only after
+// the barrier of exchange e + 1, which every thread of every CTA reaches only
+// after it has read exchange e. Same interface as GridSync and BlockSync.
 struct ClusterSync {
     double (*slots)[kMaxCluster][kSlotDoubles];   // this CTA's shared [2][kMaxCluster][kSlotDoubles]
     unsigned rank, size;
@@ -435,34 +465,34 @@ struct ClusterSync {
 };
 
 __device__ __forceinline__ bool is_leader(const ClusterSync &g) { return g.rank == 0; }
+__device__ __forceinline__ int row_step(const ClusterSync &) { return kTPB; }
 
-__device__ __forceinline__ bool grid_sync(ClusterSync &g, double (*)[32], int *) {
+template <int T>
+__device__ __forceinline__ bool grid_sync(ClusterSync &g, Exchange<T> &) {
     cluster_barrier();
     g.count++;
     return true;
 }
 
-template <int K>
-__device__ __forceinline__ bool grid_sum(ClusterSync &g, double (&v)[K], double (*sm)[32], int *) {
-    block_sum<K>(v, sm);   // ends with __syncthreads; every thread holds the block sums
+template <int K, int T, class F>
+__device__ __forceinline__ bool exchange(ClusterSync &g, double (&v)[K], Exchange<T> &X, F f) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    block_sum(v, X);
     const unsigned buf = g.epoch & 1u;
-    const unsigned t = threadIdx.x;
-    if (t < g.size * K) {
-        const unsigned dst = t / K, k = t - dst * K;
-        double mine = v[0];
+    if (wid == 0 && lane < (int)g.size) {
 #pragma unroll
-        for (int q = 1; q < K; ++q)
-            if ((int)k == q) mine = v[q];
-        st_cluster_f64(cluster_map(&g.slots[buf][g.rank][k], dst), mine);
+        for (int k = 0; k < K; ++k) st_cluster_f64(cluster_map(&g.slots[buf][g.rank][k], (unsigned)lane), v[k]);
     }
     cluster_barrier();
-    // every warp: lane l holds slot l, then a fixed-order warp sum
-    const int lane = threadIdx.x & 31;
+    if (wid == 0) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = lane < (int)g.size ? g.slots[buf][lane][k] : 0.0;
-    warp_allsum<K>(v);
+        for (int k = 0; k < K; ++k) v[k] = lane < (int)g.size ? g.slots[buf][lane][k] : 0.0;
+        warp_allsum<K>(v);
+        f(X.s, v);
+    }
     g.epoch++;
     g.count++;
+    __syncthreads();
     return true;
 }
 

@@ -162,28 +162,39 @@ using StCoef = StCoefT<double>;
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 
-template <typename C>
+template <typename C, bool kAhead = true>
 struct StencilOpT {
     int n, nx, ny, nz;
     int nxy;
     FastDiv dx, dy;
     StCoefT<C> c[7];   // C, W, E, S, N, B, T
 
-    __device__ __forceinline__ C coef(int d, int i, int j, int k) const {
+    // First table (or value) of coefficient d at node (i, j, k).
+    __device__ __forceinline__ C first(int d, int i, int j, int k) const {
         const StCoefT<C> &q = c[d];
-        C v = q.t1 ? __ldg(q.t1 + PBCG_SAFE(i * q.a1 + j * q.b1 + k * q.c1, q.len1)) : q.value;
-        // The second table is rare (a coefficient varying along two separate
-        // directions), and its addition is written as a loop of n2 (0 or 1)
-        // trips so that the compiler jumps over it rather than predicating it:
-        // a DADD whose lanes are all predicated off still occupies the FP64
-        // pipe for a whole warp instruction (64 cycles per sub-partition on
-        // this GPU), which as an if-converted branch cost 6 dead DADDs per row
-        // of a 7-point stencil with one summed coefficient.
+        return q.t1 ? __ldg(q.t1 + PBCG_SAFE(i * q.a1 + j * q.b1 + k * q.c1, q.len1)) : q.value;
+    }
+    // v plus the second table of coefficient d. The second table is rare (a
+    // coefficient varying along two separate directions), and its addition is
+    // written as a loop of n2 (0 or 1) trips so that the compiler jumps over it
+    // rather than predicating it: a DADD whose lanes are all predicated off
+    // still occupies the FP64 pipe for a whole warp instruction (64 cycles per
+    // sub-partition on this GPU), which as an if-converted branch cost 6 dead
+    // DADDs per row of a 7-point stencil with one summed coefficient.
+    __device__ __forceinline__ C second(int d, int i, int j, int k, C v) const {
+        const StCoefT<C> &q = c[d];
 #pragma unroll 1
         for (int m = 0; m < q.n2; ++m) v = add_rn(v, __ldg(q.t2 + PBCG_SAFE(i * q.a2 + j * q.b2 + k * q.c2, q.len2)));
         return v;
     }
+    __device__ __forceinline__ C coef(int d, int i, int j, int k) const { return second(d, i, j, k, first(d, i, j, k)); }
 
+    // kAhead: all neighbour values and first tables are loaded before the sum,
+    // whose chain (about 140 cycles a step, and a loop per second table that
+    // loads are not moved across) would otherwise wait for one load after
+    // another. Algorithm 9 per iteration: 32^3 18.9 -> 16.6 us, 48^3 29.4 ->
+    // 27.0, 128^3 179 -> 174. The mixed-precision kernel, with 56 registers for
+    // its FP32 sweeps, spills more with it and loads one neighbour at a time.
     template <class L>
     __device__ __forceinline__ auto row(int r, const L &u) const -> decltype(u(0)) {
         using T = decltype(u(0));
@@ -191,14 +202,29 @@ struct StencilOpT {
         const int i = r - t * nx;
         const int k = (int)dy.div((uint32_t)t);
         const int j = t - k * ny;
+        const bool in[7] = {true, i > 0, i < nx - 1, j > 0, j < ny - 1, k > 0, k < nz - 1};
+        const int off[7] = {0, -1, 1, -nx, nx, -nxy, nxy};
+        constexpr int order[7] = {PBCG_B, PBCG_S, PBCG_W, PBCG_C, PBCG_E, PBCG_N, PBCG_T};
         T acc = T(0);
-        if (k > 0) acc = fmaT((T)coef(PBCG_B, i, j, k), u(PBCG_SAFE(r - nxy, n)), acc);
-        if (j > 0) acc = fmaT((T)coef(PBCG_S, i, j, k), u(PBCG_SAFE(r - nx, n)), acc);
-        if (i > 0) acc = fmaT((T)coef(PBCG_W, i, j, k), u(PBCG_SAFE(r - 1, n)), acc);
-        acc = fmaT((T)coef(PBCG_C, i, j, k), u(PBCG_SAFE(r, n)), acc);
-        if (i < nx - 1) acc = fmaT((T)coef(PBCG_E, i, j, k), u(PBCG_SAFE(r + 1, n)), acc);
-        if (j < ny - 1) acc = fmaT((T)coef(PBCG_N, i, j, k), u(PBCG_SAFE(r + nx, n)), acc);
-        if (k < nz - 1) acc = fmaT((T)coef(PBCG_T, i, j, k), u(PBCG_SAFE(r + nxy, n)), acc);
+        if constexpr (kAhead) {
+            T uv[7];
+            C cf[7];
+#pragma unroll
+            for (int d = 0; d < 7; ++d) uv[d] = in[d] ? u(PBCG_SAFE(r + off[d], n)) : T(0);
+#pragma unroll
+            for (int d = 0; d < 7; ++d) cf[d] = first(d, i, j, k);
+#pragma unroll
+            for (int m = 0; m < 7; ++m) {
+                const int d = order[m];
+                if (in[d]) acc = fmaT((T)second(d, i, j, k, cf[d]), uv[d], acc);
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < 7; ++m) {
+                const int d = order[m];
+                if (in[d]) acc = fmaT((T)coef(d, i, j, k), u(PBCG_SAFE(r + off[d], n)), acc);
+            }
+        }
         return acc;
     }
 
@@ -307,6 +333,7 @@ struct StencilOpT {
     }
 };
 using StencilOp = StencilOpT<double>;
+using StencilOpLean = StencilOpT<double, false>;   // mixed-precision kernel, FP64 residual
 
 // Operators whose fused sweeps load their vectors through L2 only.
 template <class Op>
@@ -324,7 +351,7 @@ struct HasRow2 {
     static constexpr bool value = false;
 };
 template <>
-struct HasRow2<StencilOpT<float>> {
+struct HasRow2<StencilOpT<float, false>> {
     static constexpr bool value = true;
 };
 

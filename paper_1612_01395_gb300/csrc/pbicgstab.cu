@@ -59,14 +59,13 @@ struct pbicgstab_s {
     char *ws;
     cudaStream_t stream;
     int device, num_sms;
-    int occ_pipe, occ_plain;   // co-resident blocks per SM of each solver kernel
+    int occ[2][2];   // co-resident blocks per SM of the solver kernels: [pipelined][wide dot products]
     pbcg::Vectors V;
     double *b_stage, *x_stage;
     pbcg::Control *ctl;
     double *partials;
     cudaEvent_t ev0, ev1;   // bracket the solver kernel
     int prec;               // pbcg_prec of the handle
-    int occ_pipe_prec, occ_plain_prec;
     double *minv, *rh, *sh, *zh, *qh, *wh;   // Jacobi: M^{-1} and the hat vectors
     long long st_len[7][2];  // stencil: table elements the grid reaches (0: no table)
     long long nnz;           // stored entries (stencil: 7 per row), for the launch shape
@@ -93,19 +92,31 @@ int32_t pbicgstab_size(pbicgstab_t h) { return h ? h->n : -1; }
 
 namespace {
 
+template <class Op, bool Prec, bool Wide>
+const void *solver_kernel(bool pipelined) {
+    return pipelined ? (const void *)pbcg::pbicgstab_kernel<Op, Prec, Wide>
+                     : (const void *)pbcg::bicgstab_kernel<Op, Prec, Wide>;
+}
 template <class Op>
-pbcg_status occupancy(int *pipe, int *plain) {
-    PBCG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(pipe, pbcg::pbicgstab_kernel<Op, false>, pbcg::kTPB, 0));
-    PBCG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(plain, pbcg::bicgstab_kernel<Op, false>, pbcg::kTPB, 0));
-    if (*pipe < 1 || *plain < 1) return fail(PBCG_ERR_CUDA, "solver kernel cannot be resident on an SM");
-    return PBCG_OK;
+const void *solver_kernel(bool pipelined, bool prec, bool wide) {
+    return prec ? (wide ? solver_kernel<Op, true, true>(pipelined) : solver_kernel<Op, true, false>(pipelined))
+                : (wide ? solver_kernel<Op, false, true>(pipelined) : solver_kernel<Op, false, false>(pipelined));
 }
 
+int solver_threads(bool wide) {
+    return wide ? pbcg::SolverBlock<true>::kThreads : pbcg::SolverBlock<false>::kThreads;
+}
+
+// Co-resident blocks per SM of the handle's solver kernels.
 template <class Op>
-pbcg_status occupancy_prec(int *pipe, int *plain) {
-    PBCG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(pipe, pbcg::pbicgstab_kernel<Op, true>, pbcg::kTPB, 0));
-    PBCG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(plain, pbcg::bicgstab_kernel<Op, true>, pbcg::kTPB, 0));
-    if (*pipe < 1 || *plain < 1) return fail(PBCG_ERR_CUDA, "solver kernel cannot be resident on an SM");
+pbcg_status occupancy(pbicgstab_s *h) {
+    for (int pipelined = 0; pipelined < 2; ++pipelined)
+        for (int wide = 0; wide < 2; ++wide) {
+            int *occ = &h->occ[pipelined][wide];
+            PBCG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                occ, solver_kernel<Op>(pipelined, h->prec == PBCG_PREC_JACOBI, wide), solver_threads(wide), 0));
+            if (*occ < 1) return fail(PBCG_ERR_CUDA, "solver kernel cannot be resident on an SM");
+        }
     return PBCG_OK;
 }
 
@@ -166,22 +177,24 @@ long long max_index(const int64_t st[3], int nx, int ny, int nz) {
     return st[0] * (long long)(nx - 1) + st[1] * (long long)(ny - 1) + st[2] * (long long)(nz - 1);
 }
 
+// Work of a sweep: rows x max(1, entries per row / 7).
+double sweep_work(const pbicgstab_s *h) {
+    const double per_row = h->n > 0 ? (double)h->nnz / (double)h->n : 0.0;
+    return (double)h->n * (per_row > 7.0 ? per_row / 7.0 : 1.0);
+}
+
+// Blocks of the mixed-precision kernel (128 threads), occ co-resident per SM.
 int pick_grid(const pbicgstab_s *h, int occ, int req) {
     int max_grid = occ * h->num_sms;
     if (max_grid > pbcg::kMaxGrid) max_grid = pbcg::kMaxGrid;
     if (req > 0) return req < max_grid ? req : max_grid;
     // The time of an iteration is the sweep (rows per thread, one after the
     // other) plus the grid-wide exchanges, whose cost grows with the number of
-    // blocks. Block counts by work, measured on GB300 for both methods (60
-    // iterations; the optimum was flat within a few per cent around these).
-    // Work w = rows x max(1, entries per row / 7): for 5- and 7-point stencils
-    // 128 blocks up to w = 80k, then 2, 3, 4, 5 blocks per SM up to 180k,
-    // 400k, 1.2M, 3M and all co-resident blocks beyond; never fewer than one
-    // row per thread up to that count. Rows of ~21 random entries preferred
-    // one row per thread up to 256 blocks, which the work scaling gives.
-    const long long n = h->n;
-    const double per_row = n > 0 ? (double)h->nnz / (double)n : 0.0;
-    const double w = (double)n * (per_row > 7.0 ? per_row / 7.0 : 1.0);
+    // blocks. Block counts by work, measured on GB300: 128 blocks up to
+    // w = 80k, then 2, 3, 4, 5 blocks per SM up to 180k, 400k, 1.2M, 3M and all
+    // co-resident blocks beyond; never fewer than one row per thread up to that
+    // count.
+    const double w = sweep_work(h);
     long long want;
     if (w <= 80000.0) {
         want = 128;
@@ -189,20 +202,61 @@ int pick_grid(const pbicgstab_s *h, int occ, int req) {
         const int per_sm = w <= 180000.0 ? 2 : w <= 400000.0 ? 3 : w <= 1200000.0 ? 4 : w <= 3000000.0 ? 5 : occ;
         want = (long long)per_sm * h->num_sms;
     }
-    const long long one_row = (n + pbcg::kTPB - 1) / pbcg::kTPB;
+    const long long one_row = ((long long)h->n + pbcg::kTPB - 1) / pbcg::kTPB;
     if (want > one_row) want = one_row;
     if (want < 1) want = 1;
     return (int)(want < max_grid ? want : max_grid);
 }
 
+// Kernel and launch shape of a grid solve. The blocks fill the SMs only where
+// the sweep is long enough to pay for what each block adds to an exchange, and
+// never hold less than one row per thread. Measured per iteration, p-BiCGStab /
+// BiCGStab, us:
+//                          1 x 256     2 x 256     2 x 512 wide  (blocks per SM)
+//    110k, 5-7 entries     22 / 26     26 / 31     -
+//    262k                  36 / 41     36 / 39     39 / 42
+//    490k                  55 / 62     52 / 52     56 / 55
+//    885k                  88 / 91     78 / 72     75 / 69
+//    1.05M, 5 entries      194 / 173   119 / 107   89 / 82
+// Long rows (21 random entries) are bound by their gathers, which the wide
+// sums do not shorten and their shared memory takes L1 from: 200k 91 / 90 at 2
+// x 256 against 126 / 128, 500k 212 / 208 against 264 / 251. Systems of less
+// than a 128-row block per SM take blocks of 128, to use more SMs.
+constexpr long long kOneBlockRows = 180000, kWideRows = 700000, kLongRow = 8;
+struct Shape {
+    bool wide;
+    int grid, block;
+};
+Shape pick_shape(const pbicgstab_s *h, const int occ[2], bool can_wide, int req) {
+    Shape s{false, 0, solver_threads(false)};
+    const int all = occ[0] * h->num_sms;
+    if (req > 0) {   // forced: smaller blocks where the larger ones are not all resident
+        if (req > all) s.block /= 2;
+        const int most = all * solver_threads(false) / s.block;
+        s.grid = req < most ? req : most;
+    } else {
+        const long long n = h->n;
+        const bool long_rows = h->nnz > kLongRow * n;
+        int per_sm = n <= kOneBlockRows && !long_rows ? 1 : 2;
+        if (long_rows && n > kWideRows) per_sm = occ[0];
+        s.wide = can_wide && !long_rows && n > kWideRows;
+        s.block = solver_threads(s.wide);
+        if (n <= (long long)h->num_sms * (s.block / 2)) s.block /= 2;
+        const long long one_row = (n + s.block - 1) / s.block;
+        s.grid = (per_sm < occ[s.wide] ? per_sm : occ[s.wide]) * h->num_sms;
+        if (s.grid > one_row) s.grid = (int)one_row;
+        if (s.grid < 1) s.grid = 1;
+    }
+    if (s.grid > pbcg::kMaxGrid) s.grid = pbcg::kMaxGrid;
+    return s;
+}
+
 template <class Op>
-pbcg_status launch_solver(pbicgstab_s *h, const Op &op, bool pipelined, const pbcg::SolveArgs &args, int grid) {
+pbcg_status launch_solver(pbicgstab_s *h, const Op &op, bool pipelined, const pbcg::SolveArgs &args,
+                          const Shape &shape) {
     void *params[2] = {(void *)&op, (void *)&args};
-    const void *fn = pipelined ? (args.minv ? (const void *)pbcg::pbicgstab_kernel<Op, true>
-                                            : (const void *)pbcg::pbicgstab_kernel<Op, false>)
-                               : (args.minv ? (const void *)pbcg::bicgstab_kernel<Op, true>
-                                            : (const void *)pbcg::bicgstab_kernel<Op, false>);
-    PBCG_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(pbcg::kTPB), params, 0, h->stream));
+    const void *fn = solver_kernel<Op>(pipelined, args.minv != nullptr, shape.wide);
+    PBCG_CUDA(cudaLaunchCooperativeKernel(fn, dim3(shape.grid), dim3(shape.block), params, 0, h->stream));
     return PBCG_OK;
 }
 
@@ -323,8 +377,6 @@ pbcg_status run_solve(pbicgstab_s *h, bool pipelined, const double *d_b, double 
     a.qh = h->qh;
     a.wh = h->wh;
 
-    const int occ = h->prec == PBCG_PREC_JACOBI ? (pipelined ? h->occ_pipe_prec : h->occ_plain_prec)
-                                                : (pipelined ? h->occ_pipe : h->occ_plain);
     // one thread-block cluster for small unpreconditioned systems, else a cooperative grid
     int csize = 0;
     if (h->prec != PBCG_PREC_JACOBI && o.grid == 0 && h->cluster_max > 0) {
@@ -339,7 +391,8 @@ pbcg_status run_solve(pbicgstab_s *h, bool pipelined, const double *d_b, double 
     } else if (o.cluster > 0 && o.grid == 0) {
         return fail(PBCG_ERR_ARG, "cluster solves need an unpreconditioned handle on a device with clusters");
     }
-    const int grid = csize ? csize : pick_grid(h, occ, o.grid);
+    const Shape shape = csize ? Shape{false, csize, pbcg::kTPB}
+                              : pick_shape(h, h->occ[pipelined], pipelined || h->prec || a.variant == 5, o.grid);
     PBCG_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(pbcg::Control), h->stream));
     if (h->ev0) PBCG_CUDA(cudaEventRecord(h->ev0, h->stream));
     if (h->n > 0) {
@@ -349,9 +402,9 @@ pbcg_status run_solve(pbicgstab_s *h, bool pipelined, const double *d_b, double 
                  : h->csr_chunked ? launch_cluster(h, chunked(h->csr), pipelined, a, csize)
                                   : launch_cluster(h, h->csr, pipelined, a, csize);
         else
-            st = h->kind == 1 ? launch_solver(h, h->st, pipelined, a, grid)
-                 : h->csr_chunked ? launch_solver(h, chunked(h->csr), pipelined, a, grid)
-                                  : launch_solver(h, h->csr, pipelined, a, grid);
+            st = h->kind == 1 ? launch_solver(h, h->st, pipelined, a, shape)
+                 : h->csr_chunked ? launch_solver(h, chunked(h->csr), pipelined, a, shape)
+                                  : launch_solver(h, h->csr, pipelined, a, shape);
         if (st != PBCG_OK) return st;
     }
     if (h->ev1) PBCG_CUDA(cudaEventRecord(h->ev1, h->stream));
@@ -377,8 +430,8 @@ pbcg_status run_solve(pbicgstab_s *h, bool pipelined, const double *d_b, double 
         info->nr0 = c.nr0;
         info->rel_res_recursive = c.rel_rec;
         info->rel_res_true = c.rel_true;
-        info->grid = h->n > 0 ? grid : 0;
-        info->block = pbcg::kTPB;
+        info->grid = h->n > 0 ? shape.grid : 0;
+        info->block = shape.block;
         info->cluster = h->n > 0 ? csize : 0;
         info->grid_syncs = c.grid_syncs;
         info->spmvs = c.spmvs;
@@ -427,13 +480,11 @@ pbcg_status pbicgstab_create_csr(int32_t n, int32_t nnz, const int32_t *d_rowptr
         h->nnz = nnz;
         h->csr_chunked = (long long)nnz > pbcg::kChunkedMinAvgRow * (long long)n;
         if (h->csr_chunked) {
-            st = occupancy<pbcg::CsrOpChunked>(&h->occ_pipe, &h->occ_plain);
+            st = occupancy<pbcg::CsrOpChunked>(h);
             h->cluster_max = cluster_max_for<pbcg::CsrOpChunked>();
-            if (st == PBCG_OK) st = occupancy_prec<pbcg::CsrOpChunked>(&h->occ_pipe_prec, &h->occ_plain_prec);
         } else {
-            st = occupancy<pbcg::CsrOpScalar>(&h->occ_pipe, &h->occ_plain);
+            st = occupancy<pbcg::CsrOpScalar>(h);
             h->cluster_max = cluster_max_for<pbcg::CsrOpScalar>();
-            if (st == PBCG_OK) st = occupancy_prec<pbcg::CsrOpScalar>(&h->occ_pipe_prec, &h->occ_plain_prec);
         }
     }
     if (st == PBCG_OK) st = check_csr(h, n, nnz, d_rowptr, d_col);
@@ -503,9 +554,8 @@ pbcg_status pbicgstab_create_stencil(const pbcg_stencil *desc, pbcg_prec prec, v
             h->st_len[d][0] = c.data ? max_index(c.stride, nx, ny, nz) + 1 : 0;
             h->st_len[d][1] = c.data2 ? max_index(c.stride2, nx, ny, nz) + 1 : 0;
         }
-        st = occupancy<pbcg::StencilOp>(&h->occ_pipe, &h->occ_plain);
+        st = occupancy<pbcg::StencilOp>(h);
         h->cluster_max = cluster_max_for<pbcg::StencilOp>();
-        if (st == PBCG_OK) st = occupancy_prec<pbcg::StencilOp>(&h->occ_pipe_prec, &h->occ_plain_prec);
     }
     if (st == PBCG_OK && prec == PBCG_PREC_JACOBI)
         st = setup_jacobi(h, [&](int blocks, int *flag) {
@@ -656,8 +706,17 @@ extern "C" pbcg_status pbicgstab_solve_mixed(pbicgstab_t h, const void *d_val_lo
         // The coefficient tables rounded to FP32, in the part of the FP64
         // vector area the 12 float vectors and the best iterate leave free
         // (10 * s floats).
-        pbcg::StencilOpT<float> a32;
-        const pbcg::StencilOp &a64 = h->st;
+        pbcg::StencilOpT<float, false> a32;
+        const pbcg::StencilOp &st64 = h->st;
+        pbcg::StencilOpLean a64;
+        a64.n = st64.n;
+        a64.nx = st64.nx;
+        a64.ny = st64.ny;
+        a64.nz = st64.nz;
+        a64.nxy = st64.nxy;
+        a64.dx = st64.dx;
+        a64.dy = st64.dy;
+        for (int d = 0; d < 7; ++d) a64.c[d] = st64.c[d];
         a32.n = a64.n;
         a32.nx = a64.nx;
         a32.ny = a64.ny;
@@ -1057,8 +1116,7 @@ extern "C" pbcg_status pbicgstab_solve_csr_noalloc(int32_t n, int32_t nnz, const
         h.csr = pbcg::CsrOpScalar{n, d_rowptr, d_col, d_val, nnz};
         h.nnz = nnz;
         h.csr_chunked = (long long)nnz > pbcg::kChunkedMinAvgRow * (long long)n;
-        st = h.csr_chunked ? occupancy<pbcg::CsrOpChunked>(&h.occ_pipe, &h.occ_plain)
-                           : occupancy<pbcg::CsrOpScalar>(&h.occ_pipe, &h.occ_plain);
+        st = h.csr_chunked ? occupancy<pbcg::CsrOpChunked>(&h) : occupancy<pbcg::CsrOpScalar>(&h);
         h.cluster_max = h.csr_chunked ? cluster_max_for<pbcg::CsrOpChunked>() : cluster_max_for<pbcg::CsrOpScalar>();
     }
     if (st == PBCG_OK) st = check_csr(&h, n, nnz, d_rowptr, d_col);

@@ -1,12 +1,17 @@
 // Persistent cooperative solver kernels: one launch runs a whole solve.
 //
-// Rows are split into gridDim.x contiguous ranges, one per thread block, and a
-// thread owns the rows lo + threadIdx.x + m * kTPB of its block's range in
-// every phase. A phase is one sweep over the rows that fuses an SpMV, the
-// AXPY recurrences that consume it and the partial dot products of a
-// reduction; phases are separated by grid_sum / grid_sync. Every block then
-// holds the same reduced scalars (alpha, beta, omega, rho), so the scalars
-// never leave the GPU and the host is not involved between iterations.
+// A thread owns the rows lo + threadIdx.x + m * row_step below hi in every
+// phase. On a grid lo is the block's first row and row_step the threads of the
+// grid, so all blocks sweep through the rows together and a row's neighbours a
+// plane away were read moments before by another block and are still in L2
+// (contiguous ranges per block read them again from DRAM: 256^3 CSR rows, 413
+// bytes a row and iteration against 360, 1212 against 1073 us); a block or
+// cluster that solves alone owns a contiguous range. A phase is one sweep over
+// the rows that fuses an SpMV, the AXPY recurrences that consume it and the
+// partial dot products of a reduction; phases are separated by exchange /
+// grid_sync. An exchange also forms the scalars (alpha, beta, omega, rho), the
+// same in every block, so they never leave the GPU and the host is not involved
+// between iterations.
 //
 // Pipelined BiCGStab (Algorithm 9) takes 2 grid-wide synchronisations per
 // iteration: on one GPU the SpMV of each phase needs its input vector complete
@@ -17,6 +22,7 @@
 // the SpMV) or 5 (variant 5: p and q are written first, fewer FP64 operations).
 #pragma once
 
+#include "dots.cuh"
 #include "operators.cuh"
 
 namespace pbcg {
@@ -49,25 +55,15 @@ struct SolveArgsT {
 };
 using SolveArgs = SolveArgsT<double>;
 
-// Resident blocks per SM the solver kernels are compiled for (register cap
-// 65536 / (kTPB * kMinBlocks) = 64 at 8): the large-n sweeps are limited by
-// the FP64 pipe, which needs many warps in flight to cover memory latency. At
-// 256^3 the stencil kernels take 1.25 (p-BiCGStab) and 1.27 ms (BiCGStab) per
-// iteration with 6 blocks per SM and 1.14 and 1.08 ms with 8. With 9 (56
-// registers), p-BiCGStab slows to 1.20 ms while BiCGStab, whose sweeps hold
-// fewer values, speeds up to 1.05 ms; 10 is slower for both. Each method's
-// stencil kernel takes its own best.
-template <class Op>
-struct Tune {
-    static constexpr int kMinBlocks = 8;
-};
-template <class Op>
-struct TunePlain {
-    static constexpr int kMinBlocks = Tune<Op>::kMinBlocks;
-};
-template <>
-struct TunePlain<StencilOp> {
-    static constexpr int kMinBlocks = 9;
+// Threads per block of a grid solver kernel; both kinds fill an SM with 1024
+// threads at 64 registers. Every block repeats an exchange's arrival, polling
+// and slot sums, so large blocks are cheaper: at 1216 blocks of 128 threads an
+// exchange cost about 15 us, at 304 of 512 about 5. Per iteration of Algorithm
+// 9 (stencil): 110k unknowns 28.7 us with 304 blocks of 128 threads, 22.1 with
+// 152 of 256; 2.1M 178 and 143 us; 16.8M 1177 and 960 us (with the wide sums).
+template <bool Wide>
+struct SolverBlock {
+    static constexpr int kThreads = Wide ? 512 : 256;
 };
 
 struct Outcome {
@@ -75,93 +71,115 @@ struct Outcome {
     double nr0, nr;   // nr: squared norm of the last recursive residual (or of q after a half step)
 };
 
+#define PBCG_ROWS(i) for (int i = lo + (int)threadIdx.x; i < hi; i += row_step(g))
+
+// Tests on scalars that need no FP64 instruction (64 cycles of a sub-partition's
+// FP64 pipe, about 140 to its result): finite and zero from the bits, and the
+// order of non-negative numbers as the order of their bits.
+__device__ __forceinline__ bool is_finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
 template <int K>
 __device__ __forceinline__ bool all_finite(const double (&v)[K]) {
     bool ok = true;
 #pragma unroll
-    for (int i = 0; i < K; ++i) ok = ok && isfinite(v[i]);
+    for (int i = 0; i < K; ++i) ok = ok && is_finite(v[i]);
     return ok;
 }
 
-#define PBCG_ROWS(i) for (int i = lo + (int)threadIdx.x; i < hi; i += kTPB)
-
-// Stopping tests compare squared norms first, so that the square root (about
-// ten FP64 instructions, ~700 cycles per warp on this GPU) stays off the
-// critical path: sqrt(a) <= tol implies a <= 2 tol^2, and the exact test
-// sqrt(a) <= tol is then evaluated only in that rare case.
-__device__ __forceinline__ bool norm_below(double sq, double tol, double tol2) {
-    return (sq <= 2.0 * tol2 || !(tol2 >= 2.2250738585072014e-308)) && sqrt(sq) <= tol;
+// sqrt(sq) <= tol for a finite sq >= 0. The root (about ten FP64 instructions)
+// is taken only where it decides: sqrt(sq) <= tol implies sq <= 2 tol^2 unless
+// tol^2 underflows. bound: 2 tol^2, or infinity where tol^2 is below the normal
+// range.
+__device__ __forceinline__ bool norm_below(double sq, double tol, double bound) {
+    return __double_as_longlong(sq) <= __double_as_longlong(bound) && sqrt(sq) <= tol;
+}
+__device__ __forceinline__ double norm_bound(double tol) {
+    const double t2 = __dmul_rn(tol, tol);
+    return t2 >= 2.2250738585072014e-308 ? 2.0 * t2 : __longlong_as_double(0x7ff0000000000000ll);
 }
 
-// The divisions of an iteration's scalar updates are evaluated once per block,
-// by one warp each, and shared through shared memory. An FP64 warp
-// instruction occupies its sub-partition's FP64 pipe for 64 cycles whether
-// one warp or all four compute the same scalar, so with several resident
-// blocks per SM the redundant copies queued on the same pipes, on the
-// critical path between two sweeps. The warp is rotated by the block index,
-// (blockIdx.x + k) mod 4, so the resident blocks spread their divisions over
-// the four sub-partitions. Every thread receives the same bits as before.
-// sq: a row of 32 shared doubles; slots 0-1 beta, 2-3 den and alpha, 4 omega.
-__device__ __forceinline__ int scalar_warp(int k) { return (int)((blockIdx.x + (unsigned)k) % (kTPB / 32)); }
+// The scalar steps of an iteration. Each runs on one warp of a block (the last
+// block to arrive, on large grids), with all lanes alike, inside an exchange:
+// an FP64 instruction occupies its sub-partition's FP64 pipe for 64 cycles and
+// takes about 140 to complete, so tests and divisions repeated by every warp
+// of every resident block queued on the pipes between two sweeps.
 
-// a / b on one warp, returned to every thread (the slot is rewritten only
-// after later barriers).
-__device__ __forceinline__ double div_shared(double a, double b, int warp, double *slot) {
-    if ((int)(threadIdx.x >> 5) == warp) {
-        const double q = __ddiv_rn(a, b);
-        if ((threadIdx.x & 31) == 0) *slot = q;
+// r_0: rho = (r0, r_0), the stopping tolerance
+__device__ __forceinline__ void start_scalars(Scalars &S, double rr, double rtol) {
+    S.rho = rr;
+    S.nr = rr;
+    S.nr0 = sqrt(rr);
+    S.tol = __dmul_rn(rtol, S.nr0);
+    S.bound = norm_bound(S.tol);
+    S.alpha = S.beta = S.omega = 0.0;
+    S.status = PBCG_OK;
+    S.action = is_zero(S.nr0) ? kStop : kGo;
+}
+__device__ __forceinline__ void stop_scalars(Scalars &S, int status) {
+    S.action = kStop;
+    S.status = status;
+}
+// alpha = rho / d
+__device__ __forceinline__ void alpha_scalars(Scalars &S, double d) {
+    S.action = kGo;
+    if (!is_finite(d)) return stop_scalars(S, PBCG_NONFINITE);
+    if (is_zero(d)) return stop_scalars(S, PBCG_BREAKDOWN);
+    S.alpha = __ddiv_rn(S.rho, d);
+}
+// omega = (q,y) / (y,y), or the half step x + alpha p when ||q|| meets the tolerance
+__device__ __forceinline__ void omega_scalars(Scalars &S, double qy, double yy, double qq, bool fixed) {
+    S.action = kGo;
+    const bool small_q = !fixed && norm_below(qq, S.tol, S.bound);
+    if (small_q || is_zero(yy)) {
+        if (!small_q && !is_zero(qq)) return stop_scalars(S, PBCG_BREAKDOWN);
+        S.nr = qq;
+        S.action = kHalf;
+        return;
     }
-    __syncthreads();
-    return *slot;
+    S.omega = __ddiv_rn(qy, yy);
+    if (is_zero(S.omega)) stop_scalars(S, PBCG_BREAKDOWN);
 }
-
-// Denominator of eq. (3), r0w + beta r0s - beta omega r0z, and alpha_{i+1} =
-// rho_n / den (only when den != 0) on one warp; both returned to every thread.
-__device__ __forceinline__ void alpha_shared(double rho_n, double r0w, double r0s, double r0z, double beta,
-                                             double omega, double *sq, double &den, double &alpha) {
-    if ((int)(threadIdx.x >> 5) == scalar_warp(2)) {
-        const double d = __dsub_rn(__dadd_rn(r0w, __dmul_rn(beta, r0s)), __dmul_rn(__dmul_rn(beta, omega), r0z));
-        const double al = d == 0.0 ? 0.0 : __ddiv_rn(rho_n, d);
-        if ((threadIdx.x & 31) == 0) {
-            sq[2] = d;
-            sq[3] = al;
-        }
-    }
-    __syncthreads();
-    den = sq[2];
-    alpha = sq[3];
+// Test of r_{i+1}; beta = (alpha / omega) (rho' / rho): the two divisions are
+// one, by even and odd lanes.
+__device__ __forceinline__ void beta_scalars(Scalars &S, double rho_n, double rr, bool finite, bool fixed) {
+    S.action = kGo;
+    S.nr = rr;
+    if (!finite) return stop_scalars(S, PBCG_NONFINITE);
+    if (!fixed && norm_below(rr, S.tol, S.bound)) return stop_scalars(S, PBCG_OK);
+    if (is_zero(rho_n)) return stop_scalars(S, PBCG_BREAKDOWN);
+    const bool odd = threadIdx.x & 1;
+    const double f = __ddiv_rn(odd ? rho_n : S.alpha, odd ? S.rho : S.omega);
+    S.beta = __dmul_rn(__shfl_sync(kFull, f, 0), __shfl_sync(kFull, f, 1));
 }
-
-// beta = (alpha / omega) (rho_n / rho): the two divisions are independent, so
-// two warps evaluate one each (every warp has its own FP64 pipe) and share
-// them through shared memory.
-__device__ __forceinline__ double beta_of(double alpha, double omega, double rho_n, double rho, double *sq) {
-    const int wid = threadIdx.x >> 5;
-    if (wid == scalar_warp(0)) sq[0] = __ddiv_rn(alpha, omega);
-    if (wid == scalar_warp(1)) sq[1] = __ddiv_rn(rho_n, rho);
-    __syncthreads();
-    const double b = __dmul_rn(sq[0], sq[1]);
-    __syncthreads();
-    return b;
+// Algorithm 9: the test and beta, then the denominator of eq. (3),
+// r0w + beta r0s - beta omega r0z, and alpha_{i+1} = rho' / denominator
+__device__ __forceinline__ void beta_alpha_scalars(Scalars &S, double rho_n, double r0w, double rr, bool fixed) {
+    beta_scalars(S, rho_n, rr, is_finite(rho_n) && is_finite(r0w) && is_finite(rr), fixed);
+    if (S.action != kGo) return;
+    const double d = __dsub_rn(__dadd_rn(r0w, __dmul_rn(S.beta, S.r0s)),
+                               __dmul_rn(__dmul_rn(S.beta, S.omega), S.r0z));
+    if (is_zero(d)) return stop_scalars(S, PBCG_BREAKDOWN);
+    S.alpha = __ddiv_rn(rho_n, d);
+    S.rho = rho_n;
 }
 
 // Final true residual ||b - A x|| and the result record (block 0). The
 // history holds squared norms during the loop; they become norms here.
-template <class Op, class Sync>
-__device__ __forceinline__ void finish(const Op &A, const SolveArgs &a, Sync &g, double (*sm)[32], int *sflag,
-                                       int lo, int hi, const Outcome &o, int spmvs) {
+template <class Op, int B, class Sync>
+__device__ __forceinline__ void finish(const Op &A, const SolveArgs &a, Sync &g, Exchange<B> &X, int lo,
+                                       int hi, const Outcome &o, int spmvs) {
     double d[1] = {0.0};
     PBCG_ROWS(i) {
         const double res = a.b[i] - A.row(i, VecLoad{a.x});
         d[0] = fma(res, res, d[0]);
     }
-    if (!grid_sum<1>(g, d, sm, sflag)) return;
+    if (!exchange(g, d, X, [](Scalars &S, const double (&t)[1]) { S.aux = t[0]; })) return;
     if (blockIdx.x == 0) {
         if (a.hist)
-            for (int i = 1 + (int)threadIdx.x; i <= o.iters; i += kTPB) a.hist[i] = sqrt(a.hist[i]);
+            for (int i = 1 + (int)threadIdx.x; i <= o.iters; i += (int)blockDim.x) a.hist[i] = sqrt(a.hist[i]);
         if (threadIdx.x == 0) {
             Control *c = a.ctl;
-            const double nt = sqrt(d[0]);
+            const double nt = sqrt(X.s.aux);
             const double nr = o.iters > 0 ? sqrt(o.nr) : o.nr0;
             c->iters = o.iters;
             c->status = o.status;
@@ -212,16 +230,37 @@ struct DotAcc<float> {
     }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
-template <class Op, typename T>
-struct DotAccFor {
-    using type = DotAcc<T>;
-};
-
-template <class Acc, int K>
-__device__ __forceinline__ void dot_values(const Acc (&acc)[K], double (&d)[K]) {
+// The dot products P of a sweep accumulated one by one in T.
+template <class P, typename T>
+struct PlainDots {
+    DotAcc<T> acc[P::np];
+    __device__ __forceinline__ PlainDots(WideSlot *, bool) {}
+    __device__ __forceinline__ void add(const T (&v)[P::nv]) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) d[k] = acc[k].value();
-}
+        for (int k = 0; k < P::np; ++k) acc[k].add(v[P::a(k)], v[P::b(k)]);
+    }
+    __device__ __forceinline__ void values(double (&d)[P::np]) const {
+#pragma unroll
+        for (int k = 0; k < P::np; ++k) d[k] = acc[k].value();
+    }
+};
+// Accumulator of a sweep: FP64 sweeps of a Wide kernel sum on the integer pipes.
+template <bool Wide, class P, typename T, int B>
+struct DotsFor {
+    using type = PlainDots<P, T>;
+};
+template <class P, int B>
+struct SharedWideDots : WideDots<P> {
+    bool any;   // this thread has a row
+    __device__ __forceinline__ SharedWideDots(WideSlot *s, bool any_row)
+        : WideDots<P>(s + threadIdx.x, B, __ballot_sync(kFull, any_row)), any(any_row) {}
+    __device__ __forceinline__ void values(double (&d)[P::np]) const { WideDots<P>::values(any, d); }
+};
+template <class P, int B>
+struct DotsFor<true, P, double, B> {
+    using type = SharedWideDots<P, B>;
+};
+constexpr int kWideSlots = 5;   // dot products of the largest reduction
 
 // G adjacent elements p[i..i+cnt) of a vector (cnt <= G; the rest read as 0)
 // and their store. G = 2 uses one 64-bit access when both are present: i is
@@ -361,9 +400,9 @@ __device__ __forceinline__ void staged_pair(const float *tb, int k, int j, float
 // float for the inner solves of the mixed-precision refinement. Dot products
 // are summed per thread in T (DotAccFor) and across threads in double, and
 // alpha, beta, omega, rho are doubles; a sweep uses them rounded to T.
-template <class Op, typename T, class Sync = GridSync>
-__device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> &a, Sync &g, double (*sm)[32],
-                                               int *sflag, int lo, int hi, Outcome &o, int &spmvs,
+template <class Op, typename T, int B, class Sync = GridSync, bool Wide = false>
+__device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> &a, Sync &g, Exchange<B> &X,
+                                               int lo, int hi, Outcome &o, int &spmvs, WideSlot *wide,
                                                Stager *stg = nullptr) {
     const VectorsT<T> &V = a.V;
     T *x = a.x;
@@ -376,12 +415,11 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
     // halves their load and store instructions; their callers give every
     // block an even first row.
     constexpr int kGroup = sizeof(T) == 4 ? 2 : 1;
-    using Acc = typename DotAccFor<Op, T>::type;
 
     // r_0 := b - A x_0; shadow r0 := r_0; p, s, z, v := 0 (they are multiplied by beta_{-1} = 0)
     double d0[1];
     {
-        Acc acc[1];
+        DotAcc<T> acc;
         PBCG_ROWS(i) {
             const T ri = a.b[i] - A.row(i, VecLoadT<T>{x});
             V.r[i] = ri;
@@ -390,41 +428,37 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
             V.s[i] = T(0);
             V.z[i] = T(0);
             V.v[i] = T(0);
-            acc[0].add(ri, ri);
+            acc.add(ri, ri);
         }
-        dot_values(acc, d0);
+        d0[0] = acc.value();
     }
     ++spmvs;
-    if (!grid_sum<1>(g, d0, sm, sflag)) return false;
-    double rho = d0[0];                 // (r0, r_0)
-    o.nr0 = sqrt(rho);
+    if (!exchange(g, d0, X, [&](Scalars &S, const double (&t)[1]) { start_scalars(S, t[0], a.rtol); })) return false;
+    o.nr0 = X.s.nr0;
     o.nr = o.nr0;
     if (threadIdx.x == 0 && a.hist && is_leader(g)) a.hist[0] = o.nr0;
-    const double tol = __dmul_rn(a.rtol, o.nr0), tol2 = __dmul_rn(tol, tol);
-    if (o.nr0 == 0.0) { o.status = PBCG_OK; return true; }
+    if (X.s.action == kStop) { o.status = X.s.status; return true; }
 
     // w_0 := A r_0; alpha_0 := (r0, r0) / (r0, w0)
     {
-        Acc acc[1];
+        DotAcc<T> acc;
         PBCG_ROWS(i) {
             const T wi = A.row(i, VecLoadT<T>{V.r});
             V.w[i] = wi;
-            acc[0].add(V.r0[i], wi);
+            acc.add(V.r0[i], wi);
         }
-        dot_values(acc, d0);
+        d0[0] = acc.value();
     }
     ++spmvs;
-    if (!grid_sum<1>(g, d0, sm, sflag)) return false;
-    if (!isfinite(d0[0])) { o.status = PBCG_NONFINITE; return true; }
-    if (d0[0] == 0.0) { o.status = PBCG_BREAKDOWN; return true; }
-    double alpha = __ddiv_rn(rho, d0[0]), beta = 0.0, omega = 0.0;
+    if (!exchange(g, d0, X, [](Scalars &S, const double (&t)[1]) { alpha_scalars(S, t[0]); })) return false;
+    if (X.s.action == kStop) { o.status = X.s.status; return true; }
 
     bool replaced_rw = false;   // r_i, w_i were replaced at the end of iteration i-1
     int it = 0;
     while (it < a.limit) {
         // ---- phase A: t_i = A w_i; p_i, s_i, z_i, q_i, y_i; first reduction
-        Acc a1[5];   // (q,y) (y,y) (q,q) (r0,s) (r0,z)
-        const T al = (T)alpha, be = (T)beta, om = (T)omega;
+        typename DotsFor<Wide, PairsPipeA, T, B>::type a1(wide, lo + (int)threadIdx.x < hi);   // (q,y) (y,y) (q,q) (r0,s) (r0,z)
+        const T al = (T)X.s.alpha, be = (T)X.s.beta, om = (T)X.s.omega;
         bool swept = false;   // the staged sweep did phase A
         if constexpr (kGroup == 2 && HasRow2<Op>::value) {
             if (!replaced_rw && stg) {
@@ -458,13 +492,7 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
                         zn[u] = fmaT(be, fmaT(-om, vi[u], zi[u]), ti[u]);   // z_i, eq. (6)
                         qn[u] = fmaT(-al, sn[u], ri[u]);                    // q_i
                         yn[u] = fmaT(-al, zn[u], wi[u]);                    // y_i, eq. (4)
-                        if (u < cnt) {
-                            a1[0].add(qn[u], yn[u]);
-                            a1[1].add(yn[u], yn[u]);
-                            a1[2].add(qn[u], qn[u]);
-                            a1[3].add(r0i[u], sn[u]);
-                            a1[4].add(r0i[u], zn[u]);
-                        }
+                        if (u < cnt) a1.add({qn[u], yn[u], r0i[u], sn[u], zn[u]});
                     }
                     store_group(V.t, i0, cnt, ti);
                     store_group(V.p, i0, cnt, pn);
@@ -480,7 +508,7 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
         }
         if (swept) {
         } else if (!replaced_rw) {
-            for (int i0 = lo + kGroup * (int)threadIdx.x; i0 < hi; i0 += kGroup * kTPB) {
+            for (int i0 = lo + kGroup * (int)threadIdx.x; i0 < hi; i0 += kGroup * row_step(g)) {
                 const int cnt = kGroup == 1 ? 1 : (hi - i0 < kGroup ? hi - i0 : kGroup);
                 T ti[kGroup] = {}, ri[kGroup], wi[kGroup], si[kGroup], zi[kGroup], pi[kGroup], vi[kGroup], r0i[kGroup];
                 if constexpr (kGroup == 2 && HasRow2<Op>::value) {
@@ -511,13 +539,7 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
                     zn[u] = fmaT(be, fmaT(-om, vi[u], zi[u]), ti[u]);   // z_i, eq. (6)
                     qn[u] = fmaT(-al, sn[u], ri[u]);                    // q_i
                     yn[u] = fmaT(-al, zn[u], wi[u]);                    // y_i, eq. (4)
-                    if (u < cnt) {
-                        a1[0].add(qn[u], yn[u]);
-                        a1[1].add(yn[u], yn[u]);
-                        a1[2].add(qn[u], qn[u]);
-                        a1[3].add(r0i[u], sn[u]);
-                        a1[4].add(r0i[u], zn[u]);
-                    }
+                    if (u < cnt) a1.add({qn[u], yn[u], r0i[u], sn[u], zn[u]});
                 }
                 store_group(V.t, i0, cnt, ti);
                 store_group(V.p, i0, cnt, pn);
@@ -533,9 +555,9 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
                 V.t[i] = A.row(i, VecLoadT<T>{V.w});
                 V.p[i] = fmaT(be, fmaT(-om, V.s[i], V.p[i]), V.r[i]);
             }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) { V.s[i] = A.row(i, VecLoadT<T>{V.p}); }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const T zn = A.row(i, VecLoadT<T>{V.s});
                 const T sn = V.s[i], ri = V.r[i], wi = V.w[i];
@@ -545,39 +567,36 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
                 V.q[i] = qi;
                 V.y[i] = yi;
                 const T r0i = V.r0[i];
-                a1[0].add(qi, yi);
-                a1[1].add(yi, yi);
-                a1[2].add(qi, qi);
-                a1[3].add(r0i, sn);
-                a1[4].add(r0i, zn);
+                a1.add({qi, yi, r0i, sn, zn});
             }
             spmvs += 3;
         }
         double d1[5];
-        dot_values(a1, d1);
-        if (!grid_sum<5>(g, d1, sm, sflag)) return false;
-        const double qy = d1[0], yy = d1[1], qq = d1[2], r0s = d1[3], r0z = d1[4];
-        if (!all_finite(d1)) { o.status = PBCG_NONFINITE; break; }
-        const bool small_q = !fixed && norm_below(qq, tol, tol2);
-        if (small_q || yy == 0.0) {
-            if (!small_q && qq != 0.0) { o.status = PBCG_BREAKDOWN; break; }
+        a1.values(d1);
+        if (!exchange(g, d1, X, [&](Scalars &S, const double (&t)[5]) {
+                S.r0s = t[3];
+                S.r0z = t[4];
+                if (!all_finite(t)) return stop_scalars(S, PBCG_NONFINITE);
+                omega_scalars(S, t[0], t[1], t[2], fixed);
+            }))
+            return false;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
+        if (X.s.action == kHalf) {
             PBCG_ROWS(i) { x[i] = fmaT(al, V.p[i], x[i]); }   // half step x_i + alpha_i p_i
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             ++it;
-            o.nr = qq;
+            o.nr = X.s.nr;
             o.half = 1;
             o.status = PBCG_OK;
-            if (threadIdx.x == 0 && a.hist && is_leader(g)) a.hist[it] = qq;
+            if (threadIdx.x == 0 && a.hist && is_leader(g)) a.hist[it] = X.s.nr;
             break;
         }
-        omega = div_shared(qy, yy, scalar_warp(3), &sm[kMaxDots - 1][4]);
-        if (omega == 0.0) { o.status = PBCG_BREAKDOWN; break; }
 
         // ---- phase B: v_i = A z_i; x_{i+1}, r_{i+1}, w_{i+1}; second reduction
         const bool replace_now = a.replace_period > 0 && (it + 1) % a.replace_period == 0 &&
                                  (a.max_repl < 0 || o.nrr < a.max_repl);
-        Acc a2[3];   // (r0,r) (r0,w) (r,r)
-        const T om2 = (T)omega;
+        typename DotsFor<Wide, PairsPipeB, T, B>::type a2(wide, lo + (int)threadIdx.x < hi);   // (r0,r) (r0,w) (r,r)
+        const T om2 = (T)X.s.omega;
         bool swept_b = false;   // the staged sweep did phase B
         if constexpr (kGroup == 2 && HasRow2<Op>::value) {
             if (!replace_now && stg) {
@@ -608,11 +627,7 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
                         xn[u] = fmaT(om2, qi[u], fmaT(al, pi[u], xi[u]));
                         rn[u] = fmaT(-om2, yi[u], qi[u]);                     // eq. (7)
                         wn[u] = fmaT(-om2, fmaT(-al, vi[u], ti[u]), yi[u]);   // eq. (8)
-                        if (u < cnt) {
-                            a2[0].add(r0i[u], rn[u]);
-                            a2[1].add(r0i[u], wn[u]);
-                            a2[2].add(rn[u], rn[u]);
-                        }
+                        if (u < cnt) a2.add({r0i[u], rn[u], wn[u]});
                     }
                     store_group(x, i0, cnt, xn);
                     store_group(V.v, i0, cnt, vi);
@@ -626,7 +641,7 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
         }
         if (swept_b) {
         } else if (!replace_now) {
-            for (int i0 = lo + kGroup * (int)threadIdx.x; i0 < hi; i0 += kGroup * kTPB) {
+            for (int i0 = lo + kGroup * (int)threadIdx.x; i0 < hi; i0 += kGroup * row_step(g)) {
                 const int cnt = kGroup == 1 ? 1 : (hi - i0 < kGroup ? hi - i0 : kGroup);
                 T vi[kGroup] = {}, qi[kGroup], yi[kGroup], xi[kGroup], pi[kGroup], ti[kGroup], r0i[kGroup];
                 if constexpr (kGroup == 2 && HasRow2<Op>::value) {
@@ -654,11 +669,7 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
                     xn[u] = fmaT(om2, qi[u], fmaT(al, pi[u], xi[u]));
                     rn[u] = fmaT(-om2, yi[u], qi[u]);                     // eq. (7)
                     wn[u] = fmaT(-om2, fmaT(-al, vi[u], ti[u]), yi[u]);   // eq. (8)
-                    if (u < cnt) {
-                        a2[0].add(r0i[u], rn[u]);
-                        a2[1].add(r0i[u], wn[u]);
-                        a2[2].add(rn[u], rn[u]);
-                    }
+                    if (u < cnt) a2.add({r0i[u], rn[u], wn[u]});
                 }
                 store_group(x, i0, cnt, xn);
                 store_group(V.v, i0, cnt, vi);
@@ -669,37 +680,27 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
         } else {
             // replacement, first part: x_{i+1}; r_{i+1} := b - A x_{i+1}; w_{i+1} := A r_{i+1}
             PBCG_ROWS(i) { x[i] = fmaT(om2, V.q[i], fmaT(al, V.p[i], x[i])); }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) { V.r[i] = a.b[i] - A.row(i, VecLoadT<T>{x}); }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const T wn = A.row(i, VecLoadT<T>{V.r});
                 const T ri = V.r[i], r0i = V.r0[i];
                 V.w[i] = wn;
-                a2[0].add(r0i, ri);
-                a2[1].add(r0i, wn);
-                a2[2].add(ri, ri);
+                a2.add({r0i, ri, wn});
             }
             spmvs += 2;
             o.nrr++;
         }
         double d2[3];
-        dot_values(a2, d2);
+        a2.values(d2);
         replaced_rw = replace_now;
-        if (!grid_sum<3>(g, d2, sm, sflag)) return false;
+        if (!exchange(g, d2, X, [&](Scalars &S, const double (&t)[3]) { beta_alpha_scalars(S, t[0], t[1], t[2], fixed); }))
+            return false;
         ++it;
-        const double rho_n = d2[0], r0w = d2[1];
-        o.nr = d2[2];
-        if (threadIdx.x == 0 && a.hist && is_leader(g)) a.hist[it] = d2[2];
-        if (!all_finite(d2)) { o.status = PBCG_NONFINITE; break; }
-        if (!fixed && norm_below(d2[2], tol, tol2)) { o.status = PBCG_OK; break; }
-        if (rho_n == 0.0) { o.status = PBCG_BREAKDOWN; break; }
-        // beta_i = (alpha_i / omega_i) (r0, r_{i+1}) / (r0, r_i); alpha_{i+1} by eq. (3)
-        beta = beta_of(alpha, omega, rho_n, rho, sm[kMaxDots - 1]);
-        double den;
-        alpha_shared(rho_n, r0w, r0s, r0z, beta, omega, sm[kMaxDots - 1], den, alpha);
-        if (den == 0.0) { o.status = PBCG_BREAKDOWN; break; }
-        rho = rho_n;
+        o.nr = X.s.nr;
+        if (threadIdx.x == 0 && a.hist && is_leader(g)) a.hist[it] = X.s.nr;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
     }
     o.iters = it;
     if (it == a.limit && o.status == PBCG_NOT_CONVERGED && fixed) o.status = PBCG_OK;
@@ -721,9 +722,9 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
 // w := A r^ before the second reduction of iteration i-1; s := A p^ and
 // z := A s^ after p^_i; r^ and s^ are then stored as SpMV inputs (rh, sh).
 // ===========================================================================
-template <class Op>
-__device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs &a, GridSync &g, double (*sm)[32],
-                                                    int *sflag, int lo, int hi, Outcome &o, int &spmvs) {
+template <class Op, int B, bool Wide>
+__device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs &a, GridSync &g, Exchange<B> &X,
+                                                    int lo, int hi, Outcome &o, int &spmvs, WideSlot *wide) {
     const Vectors &V = a.V;
     double *x = a.x;
     const double *mi = a.minv;
@@ -744,13 +745,11 @@ __device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs
         d0[0] = fma(ri, ri, d0[0]);
     }
     ++spmvs;
-    if (!grid_sum<1>(g, d0, sm, sflag)) return false;
-    double rho = d0[0];
-    o.nr0 = sqrt(rho);
+    if (!exchange(g, d0, X, [&](Scalars &S, const double (&t)[1]) { start_scalars(S, t[0], a.rtol); })) return false;
+    o.nr0 = X.s.nr0;
     o.nr = o.nr0;
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[0] = o.nr0;
-    const double tol = __dmul_rn(a.rtol, o.nr0), tol2 = __dmul_rn(tol, tol);
-    if (o.nr0 == 0.0) { o.status = PBCG_OK; return true; }
+    if (X.s.action == kStop) { o.status = X.s.status; return true; }
 
     // w_0 := A r^_0; w^_0 := M^{-1} w_0; alpha_0 := (r0, r0) / (r0, w0)
     d0[0] = 0.0;
@@ -761,23 +760,22 @@ __device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs
         d0[0] = fma(V.r0[i], wi, d0[0]);
     }
     ++spmvs;
-    if (!grid_sum<1>(g, d0, sm, sflag)) return false;
-    if (!isfinite(d0[0])) { o.status = PBCG_NONFINITE; return true; }
-    if (d0[0] == 0.0) { o.status = PBCG_BREAKDOWN; return true; }
-    double alpha = __ddiv_rn(rho, d0[0]), beta = 0.0, omega = 0.0;
+    if (!exchange(g, d0, X, [](Scalars &S, const double (&t)[1]) { alpha_scalars(S, t[0]); })) return false;
+    if (X.s.action == kStop) { o.status = X.s.status; return true; }
 
     bool replaced = false;
     int it = 0;
     while (it < a.limit) {
+        const double alpha = X.s.alpha, beta = X.s.beta, om1 = X.s.omega;
         // ---- phase A: t = A w^; p^, s, z, z^, q, y; first reduction
-        double d1[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // (q,y) (y,y) (q,q) (r0,s) (r0,z)
+        typename DotsFor<Wide, PairsPipeA, double, B>::type a1(wide, lo + (int)threadIdx.x < hi);   // (q,y) (y,y) (q,q) (r0,s) (r0,z)
         if (!replaced) {
             PBCG_ROWS(i) {
                 const double ti = A.row(i, VecLoad{wh});
                 const double m = mi[i], ri = V.r[i], si = V.s[i], zi = V.z[i], wi = V.w[i];
-                const double ph = fma(beta, fma(-omega, m * si, V.p[i]), m * ri);   // p^_i = r^_i + beta (p^ - omega s^)
-                const double sn = fma(beta, fma(-omega, zi, si), wi);               // s_i
-                const double zn = fma(beta, fma(-omega, V.v[i], zi), ti);           // z_i
+                const double ph = fma(beta, fma(-om1, m * si, V.p[i]), m * ri);   // p^_i = r^_i + beta (p^ - omega s^)
+                const double sn = fma(beta, fma(-om1, zi, si), wi);               // s_i
+                const double zn = fma(beta, fma(-om1, V.v[i], zi), ti);           // z_i
                 const double qi = fma(-alpha, sn, ri);                              // q_i
                 const double yi = fma(-alpha, zn, wi);                              // y_i
                 V.t[i] = ti;
@@ -788,11 +786,7 @@ __device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs
                 V.q[i] = qi;
                 V.y[i] = yi;
                 const double r0i = V.r0[i];
-                d1[0] = fma(qi, yi, d1[0]);
-                d1[1] = fma(yi, yi, d1[1]);
-                d1[2] = fma(qi, qi, d1[2]);
-                d1[3] = fma(r0i, sn, d1[3]);
-                d1[4] = fma(r0i, zn, d1[4]);
+                a1.add({qi, yi, r0i, sn, zn});
             }
             ++spmvs;
         } else {
@@ -800,15 +794,15 @@ __device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs
             PBCG_ROWS(i) {
                 const double m = mi[i];
                 V.t[i] = A.row(i, VecLoad{wh});
-                V.p[i] = fma(beta, fma(-omega, m * V.s[i], V.p[i]), m * V.r[i]);   // r^ = M^{-1} r replaced
+                V.p[i] = fma(beta, fma(-om1, m * V.s[i], V.p[i]), m * V.r[i]);   // r^ = M^{-1} r replaced
             }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const double sn = A.row(i, VecLoad{V.p});
                 V.s[i] = sn;
                 sh[i] = mi[i] * sn;
             }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const double zn = A.row(i, VecLoad{sh});
                 const double sn = V.s[i];
@@ -819,36 +813,36 @@ __device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs
                 V.q[i] = qi;
                 V.y[i] = yi;
                 const double r0i = V.r0[i];
-                d1[0] = fma(qi, yi, d1[0]);
-                d1[1] = fma(yi, yi, d1[1]);
-                d1[2] = fma(qi, qi, d1[2]);
-                d1[3] = fma(r0i, sn, d1[3]);
-                d1[4] = fma(r0i, zn, d1[4]);
+                a1.add({qi, yi, r0i, sn, zn});
             }
             spmvs += 3;
         }
-        if (!grid_sum<5>(g, d1, sm, sflag)) return false;
-        const double qy = d1[0], yy = d1[1], qq = d1[2], r0s = d1[3], r0z = d1[4];
-        if (!all_finite(d1)) { o.status = PBCG_NONFINITE; break; }
-        const bool small_q = !fixed && norm_below(qq, tol, tol2);
-        if (small_q || yy == 0.0) {
-            if (!small_q && qq != 0.0) { o.status = PBCG_BREAKDOWN; break; }
+        double d1[5];
+        a1.values(d1);
+        if (!exchange(g, d1, X, [&](Scalars &S, const double (&t)[5]) {
+                S.r0s = t[3];
+                S.r0z = t[4];
+                if (!all_finite(t)) return stop_scalars(S, PBCG_NONFINITE);
+                omega_scalars(S, t[0], t[1], t[2], fixed);
+            }))
+            return false;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
+        if (X.s.action == kHalf) {
             PBCG_ROWS(i) { x[i] = fma(alpha, V.p[i], x[i]); }   // half step x_i + alpha_i p^_i
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             ++it;
-            o.nr = qq;
+            o.nr = X.s.nr;
             o.half = 1;
             o.status = PBCG_OK;
-            if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = qq;
+            if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = X.s.nr;
             break;
         }
-        omega = div_shared(qy, yy, scalar_warp(3), &sm[kMaxDots - 1][4]);
-        if (omega == 0.0) { o.status = PBCG_BREAKDOWN; break; }
 
         // ---- phase B: v = A z^; x, r, w, w^; second reduction
+        const double omega = X.s.omega;
         const bool replace_now = a.replace_period > 0 && (it + 1) % a.replace_period == 0 &&
                                  (a.max_repl < 0 || o.nrr < a.max_repl);
-        double d2[3] = {0.0, 0.0, 0.0};   // (r0,r) (r0,w) (r,r)
+        typename DotsFor<Wide, PairsPipeB, double, B>::type a2(wide, lo + (int)threadIdx.x < hi);   // (r0,r) (r0,w) (r,r)
         if (!replace_now) {
             PBCG_ROWS(i) {
                 const double vi = A.row(i, VecLoad{zh});
@@ -861,69 +855,61 @@ __device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs
                 V.w[i] = wn;
                 wh[i] = m * wn;                                         // w^_{i+1}
                 const double r0i = V.r0[i];
-                d2[0] = fma(r0i, rn, d2[0]);
-                d2[1] = fma(r0i, wn, d2[1]);
-                d2[2] = fma(rn, rn, d2[2]);
+                a2.add({r0i, rn, wn});
             }
             ++spmvs;
         } else {
             PBCG_ROWS(i) { x[i] = fma(omega, mi[i] * V.q[i], fma(alpha, V.p[i], x[i])); }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const double rn = a.b[i] - A.row(i, VecLoad{x});
                 V.r[i] = rn;
                 rh[i] = mi[i] * rn;
             }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const double wn = A.row(i, VecLoad{rh});
                 const double rn = V.r[i], r0i = V.r0[i];
                 V.w[i] = wn;
                 wh[i] = mi[i] * wn;
-                d2[0] = fma(r0i, rn, d2[0]);
-                d2[1] = fma(r0i, wn, d2[1]);
-                d2[2] = fma(rn, rn, d2[2]);
+                a2.add({r0i, rn, wn});
             }
             spmvs += 2;
             o.nrr++;
         }
         replaced = replace_now;
-        if (!grid_sum<3>(g, d2, sm, sflag)) return false;
+        double d2[3];
+        a2.values(d2);
+        if (!exchange(g, d2, X, [&](Scalars &S, const double (&t)[3]) { beta_alpha_scalars(S, t[0], t[1], t[2], fixed); }))
+            return false;
         ++it;
-        const double rho_n = d2[0], r0w = d2[1];
-        o.nr = d2[2];
-        if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = d2[2];
-        if (!all_finite(d2)) { o.status = PBCG_NONFINITE; break; }
-        if (!fixed && norm_below(d2[2], tol, tol2)) { o.status = PBCG_OK; break; }
-        if (rho_n == 0.0) { o.status = PBCG_BREAKDOWN; break; }
-        beta = beta_of(alpha, omega, rho_n, rho, sm[kMaxDots - 1]);
-        double den;
-        alpha_shared(rho_n, r0w, r0s, r0z, beta, omega, sm[kMaxDots - 1], den, alpha);
-        if (den == 0.0) { o.status = PBCG_BREAKDOWN; break; }
-        rho = rho_n;
+        o.nr = X.s.nr;
+        if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = X.s.nr;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
     }
     o.iters = it;
     if (it == a.limit && o.status == PBCG_NOT_CONVERGED && fixed) o.status = PBCG_OK;
     return true;
 }
 
-template <class Op, bool Prec>
-__global__ void __launch_bounds__(kTPB, Tune<Op>::kMinBlocks) pbicgstab_kernel(const Op A, const SolveArgs a) {
-    __shared__ double sm[kMaxDots][32];
-    __shared__ int sflag;
-    if (threadIdx.x == 0) sflag = 1;   // read only after the first exchange's barrier
-    GridSync g{a.ctl, a.partials, 0u, 0};   // partials: the exchange slots
-    const int lo = (int)((long long)blockIdx.x * a.n / gridDim.x);
-    const int hi = (int)((long long)(blockIdx.x + 1) * a.n / gridDim.x);
+template <class Op, bool Prec, bool Wide>
+__global__ void __launch_bounds__(SolverBlock<Wide>::kThreads, 1024 / SolverBlock<Wide>::kThreads)
+    pbicgstab_kernel(const Op A, const SolveArgs a) {
+    constexpr int B = SolverBlock<Wide>::kThreads;
+    __shared__ Exchange<B> X;
+    __shared__ WideSlot wide[Wide ? kWideSlots * B : 1];
+    if (threadIdx.x == 0) X.ok = 1;   // read only after the first exchange's barrier
+    GridSync g{a.ctl, a.partials, 0u, 0, (int)(gridDim.x * blockDim.x)};   // partials: the exchange slots
+    const int lo = (int)(blockIdx.x * blockDim.x), hi = a.n;
     Outcome o{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
     int spmvs = 0;
     bool ok;
     if constexpr (Prec)
-        ok = pipelined_prec_loop(A, a, g, sm, &sflag, lo, hi, o, spmvs);
+        ok = pipelined_prec_loop<Op, B, Wide>(A, a, g, X, lo, hi, o, spmvs, wide);
     else
-        ok = pipelined_loop<Op, double>(A, a, g, sm, &sflag, lo, hi, o, spmvs);
+        ok = pipelined_loop<Op, double, B, GridSync, Wide>(A, a, g, X, lo, hi, o, spmvs, wide);
     if (!ok) return;
-    finish(A, a, g, sm, &sflag, lo, hi, o, spmvs);
+    finish(A, a, g, X, lo, hi, o, spmvs);
 }
 
 // ===========================================================================
@@ -931,13 +917,13 @@ __global__ void __launch_bounds__(kTPB, Tune<Op>::kMinBlocks) pbicgstab_kernel(c
 // the phase that forms p_i for its SpMV reads p_{i-1}, s_{i-1} of neighbours
 // while writing p_i, s_i, so the old and new values must not share storage.
 // ===========================================================================
-template <class Op, class Sync = GridSync>
-__device__ __forceinline__ bool standard_loop(const Op &A, const SolveArgs &a, Sync &g, double (*sm)[32],
-                                              int *sflag, int lo, int hi, Outcome &o, int &spmvs) {
+template <class Op, int B, class Sync = GridSync, bool Wide = false>
+__device__ __forceinline__ bool standard_loop(const Op &A, const SolveArgs &a, Sync &g, Exchange<B> &X,
+                                              int lo, int hi, Outcome &o, int &spmvs, WideSlot *wide) {
     const Vectors &V = a.V;
     double *x = a.x;
     const bool fixed = a.fixed != 0;
-    const bool v3 = a.variant == 3;
+    const bool v3 = !Wide && a.variant == 3;   // the wide kernel holds variant 5 alone
     // buffers: variant 3 ping-pongs p between V.p / V.z and s between V.s / V.w
     double *pA = V.p, *pB = V.z, *sA = V.s, *sB = V.w;
 
@@ -952,45 +938,44 @@ __device__ __forceinline__ bool standard_loop(const Op &A, const SolveArgs &a, S
         d0[0] = fma(ri, ri, d0[0]);
     }
     ++spmvs;
-    if (!grid_sum<1>(g, d0, sm, sflag)) return false;
-    double rho = d0[0];
-    o.nr0 = sqrt(rho);
+    if (!exchange(g, d0, X, [&](Scalars &S, const double (&t)[1]) { start_scalars(S, t[0], a.rtol); })) return false;
+    o.nr0 = X.s.nr0;
     o.nr = o.nr0;
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[0] = o.nr0;
-    const double tol = __dmul_rn(a.rtol, o.nr0), tol2 = __dmul_rn(tol, tol);
-    if (o.nr0 == 0.0) { o.status = PBCG_OK; return true; }
-    double beta = 0.0, omega = 0.0;
+    if (X.s.action == kStop) { o.status = X.s.status; return true; }
 
     int it = 0;
     while (it < a.limit) {
+        const double beta = X.s.beta, om1 = X.s.omega;
         // ---- s_i = A p_i, alpha_i = (r0, r_i) / (r0, s_i)
-        double d1[1] = {0.0};
+        typename DotsFor<Wide, PairsOne, double, B>::type a1(wide, lo + (int)threadIdx.x < hi);   // (r0,s)
         if (v3) {
-            const PLoad pl{V.r, pA, sA, beta, omega};
+            const PLoad pl{V.r, pA, sA, beta, om1};
             PBCG_ROWS(i) {
                 const double si = A.row(i, pl);
                 pB[i] = pl(i);
                 sB[i] = si;
-                d1[0] = fma(V.r0[i], si, d1[0]);
+                a1.add({V.r0[i], si});
             }
         } else {
-            PBCG_ROWS(i) { pA[i] = fma(beta, fma(-omega, sA[i], pA[i]), V.r[i]); }
-            if (!grid_sync(g, sm, sflag)) return false;
+            PBCG_ROWS(i) { pA[i] = fma(beta, fma(-om1, sA[i], pA[i]), V.r[i]); }
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const double si = A.row(i, VecLoad{pA});
                 sA[i] = si;
-                d1[0] = fma(V.r0[i], si, d1[0]);
+                a1.add({V.r0[i], si});
             }
         }
         ++spmvs;
         double *pc = v3 ? pB : pA, *sc = v3 ? sB : sA;   // p_i, s_i
-        if (!grid_sum<1>(g, d1, sm, sflag)) return false;
-        if (!isfinite(d1[0])) { o.status = PBCG_NONFINITE; break; }
-        if (d1[0] == 0.0) { o.status = PBCG_BREAKDOWN; break; }
-        const double alpha = div_shared(rho, d1[0], scalar_warp(2), &sm[kMaxDots - 1][3]);
+        double d1[1];
+        a1.values(d1);
+        if (!exchange(g, d1, X, [](Scalars &S, const double (&t)[1]) { alpha_scalars(S, t[0]); })) return false;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
+        const double alpha = X.s.alpha;
 
         // ---- q_i = r_i - alpha s_i; y_i = A q_i; omega_i
-        double d2[3] = {0.0, 0.0, 0.0};   // (q,y) (y,y) (q,q)
+        typename DotsFor<Wide, PairsOmega, double, B>::type a2(wide, lo + (int)threadIdx.x < hi);   // (q,y) (y,y) (q,q)
         if (v3) {
             const QLoad ql{V.r, sc, alpha};
             PBCG_ROWS(i) {
@@ -998,61 +983,59 @@ __device__ __forceinline__ bool standard_loop(const Op &A, const SolveArgs &a, S
                 const double qi = ql(i);
                 V.q[i] = qi;
                 V.y[i] = yi;
-                d2[0] = fma(qi, yi, d2[0]);
-                d2[1] = fma(yi, yi, d2[1]);
-                d2[2] = fma(qi, qi, d2[2]);
+                a2.add({qi, yi});
             }
         } else {
             PBCG_ROWS(i) { V.q[i] = fma(-alpha, sc[i], V.r[i]); }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const double yi = A.row(i, VecLoad{V.q});
                 const double qi = V.q[i];
                 V.y[i] = yi;
-                d2[0] = fma(qi, yi, d2[0]);
-                d2[1] = fma(yi, yi, d2[1]);
-                d2[2] = fma(qi, qi, d2[2]);
+                a2.add({qi, yi});
             }
         }
         ++spmvs;
-        if (!grid_sum<3>(g, d2, sm, sflag)) return false;
-        const double qy = d2[0], yy = d2[1], qq = d2[2];
-        if (!all_finite(d2)) { o.status = PBCG_NONFINITE; break; }
-        const bool small_q = !fixed && norm_below(qq, tol, tol2);
-        if (small_q || yy == 0.0) {
-            if (!small_q && qq != 0.0) { o.status = PBCG_BREAKDOWN; break; }
+        double d2[3];
+        a2.values(d2);
+        if (!exchange(g, d2, X, [&](Scalars &S, const double (&t)[3]) {
+                if (!all_finite(t)) return stop_scalars(S, PBCG_NONFINITE);
+                omega_scalars(S, t[0], t[1], t[2], fixed);
+            }))
+            return false;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
+        if (X.s.action == kHalf) {
             PBCG_ROWS(i) { x[i] = fma(alpha, pc[i], x[i]); }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             ++it;
-            o.nr = qq;
+            o.nr = X.s.nr;
             o.half = 1;
             o.status = PBCG_OK;
-            if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = qq;
+            if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = X.s.nr;
             break;
         }
-        omega = div_shared(qy, yy, scalar_warp(3), &sm[kMaxDots - 1][4]);
-        if (omega == 0.0) { o.status = PBCG_BREAKDOWN; break; }
+        const double omega = X.s.omega;
 
         // ---- x_{i+1}, r_{i+1}; beta_i
-        double d3[2] = {0.0, 0.0};   // (r0,r) (r,r)
+        typename DotsFor<Wide, PairsRho, double, B>::type a3(wide, lo + (int)threadIdx.x < hi);   // (r0,r) (r,r)
         PBCG_ROWS(i) {
             const double qi = V.q[i];
             x[i] = fma(omega, qi, fma(alpha, pc[i], x[i]));
             const double rn = fma(-omega, V.y[i], qi);
             V.r[i] = rn;
-            d3[0] = fma(V.r0[i], rn, d3[0]);
-            d3[1] = fma(rn, rn, d3[1]);
+            a3.add({V.r0[i], rn});
         }
-        if (!grid_sum<2>(g, d3, sm, sflag)) return false;
+        double d3[2];
+        a3.values(d3);
+        if (!exchange(g, d3, X, [&](Scalars &S, const double (&t)[2]) {
+                beta_scalars(S, t[0], t[1], all_finite(t), fixed);
+                S.rho = t[0];
+            }))
+            return false;
         ++it;
-        const double rho_n = d3[0];
-        o.nr = d3[1];
-        if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = d3[1];
-        if (!all_finite(d3)) { o.status = PBCG_NONFINITE; break; }
-        if (!fixed && norm_below(d3[1], tol, tol2)) { o.status = PBCG_OK; break; }
-        if (rho_n == 0.0) { o.status = PBCG_BREAKDOWN; break; }
-        beta = beta_of(alpha, omega, rho_n, rho, sm[kMaxDots - 1]);
-        rho = rho_n;
+        o.nr = X.s.nr;
+        if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = X.s.nr;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
         if (v3) {
             double *tp = pA; pA = pB; pB = tp;
             double *ts = sA; sA = sB; sB = ts;
@@ -1068,9 +1051,9 @@ __device__ __forceinline__ bool standard_loop(const Op &A, const SolveArgs &a, S
 // five-exchange form of the standard loop with p^ = M^{-1} p and
 // q^ = M^{-1} q written next to p and q. Buffers: V.z holds p^, a.qh holds q^.
 // ===========================================================================
-template <class Op>
-__device__ __forceinline__ bool standard_prec_loop(const Op &A, const SolveArgs &a, GridSync &g, double (*sm)[32],
-                                                   int *sflag, int lo, int hi, Outcome &o, int &spmvs) {
+template <class Op, int B, bool Wide>
+__device__ __forceinline__ bool standard_prec_loop(const Op &A, const SolveArgs &a, GridSync &g, Exchange<B> &X,
+                                                   int lo, int hi, Outcome &o, int &spmvs, WideSlot *wide) {
     const Vectors &V = a.V;
     double *x = a.x;
     const double *mi = a.minv;
@@ -1087,111 +1070,111 @@ __device__ __forceinline__ bool standard_prec_loop(const Op &A, const SolveArgs 
         d0[0] = fma(ri, ri, d0[0]);
     }
     ++spmvs;
-    if (!grid_sum<1>(g, d0, sm, sflag)) return false;
-    double rho = d0[0];
-    o.nr0 = sqrt(rho);
+    if (!exchange(g, d0, X, [&](Scalars &S, const double (&t)[1]) { start_scalars(S, t[0], a.rtol); })) return false;
+    o.nr0 = X.s.nr0;
     o.nr = o.nr0;
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[0] = o.nr0;
-    const double tol = __dmul_rn(a.rtol, o.nr0), tol2 = __dmul_rn(tol, tol);
-    if (o.nr0 == 0.0) { o.status = PBCG_OK; return true; }
-    double beta = 0.0, omega = 0.0;
+    if (X.s.action == kStop) { o.status = X.s.status; return true; }
 
     int it = 0;
     while (it < a.limit) {
+        const double beta = X.s.beta, om1 = X.s.omega;
         // p_i := r_i + beta (p_{i-1} - omega s_{i-1}); p^_i := M^{-1} p_i; s_i := A p^_i
         PBCG_ROWS(i) {
-            const double pn = fma(beta, fma(-omega, V.s[i], V.p[i]), V.r[i]);
+            const double pn = fma(beta, fma(-om1, V.s[i], V.p[i]), V.r[i]);
             V.p[i] = pn;
             ph[i] = mi[i] * pn;
         }
-        if (!grid_sync(g, sm, sflag)) return false;
-        double d1[1] = {0.0};
+        if (!grid_sync(g, X)) return false;
+        typename DotsFor<Wide, PairsOne, double, B>::type a1(wide, lo + (int)threadIdx.x < hi);   // (r0,s)
         PBCG_ROWS(i) {
             const double si = A.row(i, VecLoad{ph});
             V.s[i] = si;
-            d1[0] = fma(V.r0[i], si, d1[0]);
+            a1.add({V.r0[i], si});
         }
         ++spmvs;
-        if (!grid_sum<1>(g, d1, sm, sflag)) return false;
-        if (!isfinite(d1[0])) { o.status = PBCG_NONFINITE; break; }
-        if (d1[0] == 0.0) { o.status = PBCG_BREAKDOWN; break; }
-        const double alpha = __ddiv_rn(rho, d1[0]);
+        double d1[1];
+        a1.values(d1);
+        if (!exchange(g, d1, X, [](Scalars &S, const double (&t)[1]) { alpha_scalars(S, t[0]); })) return false;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
+        const double alpha = X.s.alpha;
         // q_i := r_i - alpha s_i; q^_i := M^{-1} q_i; y_i := A q^_i
         PBCG_ROWS(i) {
             const double qi = fma(-alpha, V.s[i], V.r[i]);
             V.q[i] = qi;
             qh[i] = mi[i] * qi;
         }
-        if (!grid_sync(g, sm, sflag)) return false;
-        double d2[3] = {0.0, 0.0, 0.0};
+        if (!grid_sync(g, X)) return false;
+        typename DotsFor<Wide, PairsOmega, double, B>::type a2(wide, lo + (int)threadIdx.x < hi);   // (q,y) (y,y) (q,q)
         PBCG_ROWS(i) {
             const double yi = A.row(i, VecLoad{qh});
             const double qi = V.q[i];
             V.y[i] = yi;
-            d2[0] = fma(qi, yi, d2[0]);
-            d2[1] = fma(yi, yi, d2[1]);
-            d2[2] = fma(qi, qi, d2[2]);
+            a2.add({qi, yi});
         }
         ++spmvs;
-        if (!grid_sum<3>(g, d2, sm, sflag)) return false;
-        const double qy = d2[0], yy = d2[1], qq = d2[2];
-        if (!all_finite(d2)) { o.status = PBCG_NONFINITE; break; }
-        const bool small_q = !fixed && norm_below(qq, tol, tol2);
-        if (small_q || yy == 0.0) {
-            if (!small_q && qq != 0.0) { o.status = PBCG_BREAKDOWN; break; }
+        double d2[3];
+        a2.values(d2);
+        if (!exchange(g, d2, X, [&](Scalars &S, const double (&t)[3]) {
+                if (!all_finite(t)) return stop_scalars(S, PBCG_NONFINITE);
+                omega_scalars(S, t[0], t[1], t[2], fixed);
+            }))
+            return false;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
+        if (X.s.action == kHalf) {
             PBCG_ROWS(i) { x[i] = fma(alpha, ph[i], x[i]); }
-            if (!grid_sync(g, sm, sflag)) return false;
+            if (!grid_sync(g, X)) return false;
             ++it;
-            o.nr = qq;
+            o.nr = X.s.nr;
             o.half = 1;
             o.status = PBCG_OK;
-            if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = qq;
+            if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = X.s.nr;
             break;
         }
-        omega = __ddiv_rn(qy, yy);
-        if (omega == 0.0) { o.status = PBCG_BREAKDOWN; break; }
+        const double omega = X.s.omega;
         // x_{i+1} := x_i + alpha p^_i + omega q^_i; r_{i+1} := q_i - omega y_i
-        double d3[2] = {0.0, 0.0};
+        typename DotsFor<Wide, PairsRho, double, B>::type a3(wide, lo + (int)threadIdx.x < hi);   // (r0,r) (r,r)
         PBCG_ROWS(i) {
             x[i] = fma(omega, qh[i], fma(alpha, ph[i], x[i]));
             const double rn = fma(-omega, V.y[i], V.q[i]);
             V.r[i] = rn;
-            d3[0] = fma(V.r0[i], rn, d3[0]);
-            d3[1] = fma(rn, rn, d3[1]);
+            a3.add({V.r0[i], rn});
         }
-        if (!grid_sum<2>(g, d3, sm, sflag)) return false;
+        double d3[2];
+        a3.values(d3);
+        if (!exchange(g, d3, X, [&](Scalars &S, const double (&t)[2]) {
+                beta_scalars(S, t[0], t[1], all_finite(t), fixed);
+                S.rho = t[0];
+            }))
+            return false;
         ++it;
-        const double rho_n = d3[0];
-        o.nr = d3[1];
-        if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = d3[1];
-        if (!all_finite(d3)) { o.status = PBCG_NONFINITE; break; }
-        if (!fixed && norm_below(d3[1], tol, tol2)) { o.status = PBCG_OK; break; }
-        if (rho_n == 0.0) { o.status = PBCG_BREAKDOWN; break; }
-        beta = beta_of(alpha, omega, rho_n, rho, sm[kMaxDots - 1]);
-        rho = rho_n;
+        o.nr = X.s.nr;
+        if (blockIdx.x == 0 && threadIdx.x == 0 && a.hist) a.hist[it] = X.s.nr;
+        if (X.s.action == kStop) { o.status = X.s.status; break; }
     }
     o.iters = it;
     if (it == a.limit && o.status == PBCG_NOT_CONVERGED && fixed) o.status = PBCG_OK;
     return true;
 }
 
-template <class Op, bool Prec>
-__global__ void __launch_bounds__(kTPB, TunePlain<Op>::kMinBlocks) bicgstab_kernel(const Op A, const SolveArgs a) {
-    __shared__ double sm[kMaxDots][32];
-    __shared__ int sflag;
-    if (threadIdx.x == 0) sflag = 1;   // read only after the first exchange's barrier
-    GridSync g{a.ctl, a.partials, 0u, 0};   // partials: the exchange slots
-    const int lo = (int)((long long)blockIdx.x * a.n / gridDim.x);
-    const int hi = (int)((long long)(blockIdx.x + 1) * a.n / gridDim.x);
+template <class Op, bool Prec, bool Wide>
+__global__ void __launch_bounds__(SolverBlock<Wide>::kThreads, 1024 / SolverBlock<Wide>::kThreads)
+    bicgstab_kernel(const Op A, const SolveArgs a) {
+    constexpr int B = SolverBlock<Wide>::kThreads;
+    __shared__ Exchange<B> X;
+    __shared__ WideSlot wide[Wide ? kWideSlots * B : 1];
+    if (threadIdx.x == 0) X.ok = 1;   // read only after the first exchange's barrier
+    GridSync g{a.ctl, a.partials, 0u, 0, (int)(gridDim.x * blockDim.x)};   // partials: the exchange slots
+    const int lo = (int)(blockIdx.x * blockDim.x), hi = a.n;
     Outcome o{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
     int spmvs = 0;
     bool ok;
     if constexpr (Prec)
-        ok = standard_prec_loop(A, a, g, sm, &sflag, lo, hi, o, spmvs);
+        ok = standard_prec_loop<Op, B, Wide>(A, a, g, X, lo, hi, o, spmvs, wide);
     else
-        ok = standard_loop(A, a, g, sm, &sflag, lo, hi, o, spmvs);
+        ok = standard_loop<Op, B, GridSync, Wide>(A, a, g, X, lo, hi, o, spmvs, wide);
     if (!ok) return;
-    finish(A, a, g, sm, &sflag, lo, hi, o, spmvs);
+    finish(A, a, g, X, lo, hi, o, spmvs);
 }
 
 // ===========================================================================
@@ -1245,13 +1228,12 @@ struct MixedArgs {
 // blocks and 315 / 339 at 10, where the pairs spill more).
 template <class Op64, class Op32>
 __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32 A32, const MixedArgs m) {
-    __shared__ double sm[kMaxDots][32];
-    __shared__ int sflag;
+    __shared__ Exchange<kTPB> X;
     __shared__ uint64_t stage_full[kStages], stage_empty[kStages];
     extern __shared__ __align__(128) char stage_buf[];   // kStageSmemBytes when the sweeps are staged
     constexpr bool kStaged = HasRow2<Op32>::value;
     if (threadIdx.x == 0) {
-        sflag = 1;   // read only after the first exchange's barrier
+        X.ok = 1;   // read only after the first exchange's barrier
         if (kStaged) {
             for (int k = 0; k < kStages; ++k) {
                 mbar_init(&stage_full[k], 1);
@@ -1262,7 +1244,7 @@ __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32
     }
     __syncthreads();
     Stager stager{stage_buf, stage_full, stage_empty, 0u, m.ctl};
-    GridSync g{m.ctl, m.partials, 0u, 0};
+    GridSync g{m.ctl, m.partials, 0u, 0, kTPB};
     // row ranges start on multiples of 4 rows: the FP32 sweeps access rows in
     // aligned pairs, and the staged ones copy 16-byte aligned tiles
     const long long quads = (m.n + 3) / 4;
@@ -1270,7 +1252,7 @@ __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32
     const int hi_quad = (int)(4 * ((long long)(blockIdx.x + 1) * quads / gridDim.x));
     const int hi = hi_quad < m.n ? hi_quad : m.n;
     int outer = 0, inner_total = 0, status = PBCG_NOT_CONVERGED, spmvs = 0, stalls = 0;
-    double nr0 = 0.0, tol = 0.0, tol2 = 0.0, last = 0.0;
+    double nr0 = 0.0, tol = 0.0, bound = 0.0, last = 0.0;
     double best = 0.0;        // smallest squared FP64 residual so far (valid when have_best)
     bool have_best = false;
     bool at_best = false;     // x is the best iterate so far
@@ -1282,7 +1264,7 @@ __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32
                 if (save) m.xbest[i] = xi;
                 m.x[i] = xi + (double)m.d[i];
             }
-            if (!grid_sync(g, sm, &sflag)) return;
+            if (!grid_sync(g, X)) return;
         }
         double d[1] = {0.0};
         PBCG_ROWS(i) {
@@ -1292,16 +1274,17 @@ __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32
             d[0] = fma(r, r, d[0]);
         }
         ++spmvs;
-        if (!grid_sum<1>(g, d, sm, &sflag)) return;
+        if (!exchange(g, d, X, [](Scalars &S, const double (&t)[1]) { S.aux = t[0]; })) return;
+        d[0] = X.s.aux;
         last = d[0];
         if (outer == 0) {
             nr0 = sqrt(d[0]);
             tol = __dmul_rn(m.rtol, nr0);
-            tol2 = __dmul_rn(tol, tol);
+            bound = norm_bound(tol);
         }
         if (blockIdx.x == 0 && threadIdx.x == 0 && m.hist) m.hist[outer] = d[0];
         if (!isfinite(d[0])) { at_best = false; status = PBCG_NONFINITE; break; }
-        if (nr0 == 0.0 || norm_below(d[0], tol, tol2)) { at_best = true; status = PBCG_OK; break; }
+        if (nr0 == 0.0 || norm_below(d[0], tol, bound)) { at_best = true; status = PBCG_OK; break; }
         if (!have_best || d[0] < best) {
             best = d[0];
             have_best = true;
@@ -1327,7 +1310,7 @@ __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32
         ia.max_repl = -1;
         ia.variant = 0;
         Outcome io{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
-        if (!pipelined_loop<Op32, float>(A32, ia, g, sm, &sflag, lo, hi, io, spmvs, kStaged ? &stager : nullptr))
+        if (!pipelined_loop<Op32, float, kTPB>(A32, ia, g, X, lo, hi, io, spmvs, nullptr, kStaged ? &stager : nullptr))
             return;
         // the inner history holds squared norms after entry 0 (thread 0 of block 0 wrote them)
         if (blockIdx.x == 0 && threadIdx.x == 0 && ia.hist)
@@ -1372,11 +1355,10 @@ __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32
 // ===========================================================================
 template <class Op, bool Pipelined>
 __global__ void __launch_bounds__(kTPB, 1) cluster_solve_kernel(const Op A, const SolveArgs a) {
-    __shared__ double sm[kMaxDots][32];
-    __shared__ double slots[2][kMaxCluster][kSlotDoubles];
-    __shared__ int sflag;
+    __shared__ Exchange<kTPB> X;
+    __shared__ double slots[2][kMaxCluster][kSlotDoubles];   // cluster reductions: every CTA's block sums
     const unsigned size = cluster_ctas(), rank = cluster_rank();
-    if (threadIdx.x == 0) sflag = 1;
+    if (threadIdx.x == 0) X.ok = 1;
     cluster_barrier();   // every CTA started before its shared memory is written by the others
     ClusterSync g{slots, rank, size, 0u, 0};
     const int lo = (int)((long long)rank * a.n / size);
@@ -1384,10 +1366,10 @@ __global__ void __launch_bounds__(kTPB, 1) cluster_solve_kernel(const Op A, cons
     Outcome o{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
     int spmvs = 0;
     if constexpr (Pipelined)
-        pipelined_loop<Op, double, ClusterSync>(A, a, g, sm, &sflag, lo, hi, o, spmvs);
+        pipelined_loop<Op, double, kTPB, ClusterSync>(A, a, g, X, lo, hi, o, spmvs, nullptr);
     else
-        standard_loop<Op, ClusterSync>(A, a, g, sm, &sflag, lo, hi, o, spmvs);
-    finish(A, a, g, sm, &sflag, lo, hi, o, spmvs);
+        standard_loop<Op, kTPB, ClusterSync>(A, a, g, X, lo, hi, o, spmvs, nullptr);
+    finish(A, a, g, X, lo, hi, o, spmvs);
     cluster_barrier();   // no CTA leaves while another may still address its shared memory
 }
 
@@ -1457,7 +1439,7 @@ struct BatchArgs {
 // this CTA's share for ClusterSync); the first CTA writes the result.
 template <class Sync>
 __device__ __forceinline__ void batched_system(const BatchArgs &B, int sys, Sync &g, unsigned part, unsigned parts,
-                                               double (*sm)[32], int *sflag) {
+                                               Exchange<kTPB> &X) {
     const long long r0 = B.row_offset[sys], r1 = B.row_offset[sys + 1];
     // structure check of this system: its rows inside the batch, entries inside
     // the shared arrays, columns local to the system (each CTA checks its rows)
@@ -1472,9 +1454,9 @@ __device__ __forceinline__ void batched_system(const BatchArgs &B, int sys, Sync
             if (B.col[k] < 0 || B.col[k] >= n) bad = 1;
     }
     double fb[1] = {(double)bad};
-    grid_sum<1>(g, fb, sm, sflag);
+    exchange(g, fb, X, [](Scalars &S, const double (&t)[1]) { S.aux = t[0]; });
     pbcg_batch_result res{0, PBCG_ERR_ARG, 0, 0, 0.0, 0.0};
-    if (fb[0] == 0.0) {
+    if (X.s.aux == 0.0) {
         SolveArgs a;
         a.n = n;
         a.b = B.b + r0;
@@ -1494,7 +1476,7 @@ __device__ __forceinline__ void batched_system(const BatchArgs &B, int sys, Sync
         a.rh = a.sh = a.zh = a.qh = a.wh = nullptr;
         Outcome o{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
         int spmvs = 0;
-        pipelined_loop<CsrOpGatherL2, double, Sync>(A, a, g, sm, sflag, lo, hi, o, spmvs);
+        pipelined_loop<CsrOpGatherL2, double, kTPB, Sync>(A, a, g, X, lo, hi, o, spmvs, nullptr);
         // the history holds squared norms after entry 0 (written by this thread)
         if (a.hist && part == 0 && threadIdx.x == 0)
             for (int i = 1; i <= o.iters; ++i) a.hist[i] = sqrt(a.hist[i]);
@@ -1504,23 +1486,22 @@ __device__ __forceinline__ void batched_system(const BatchArgs &B, int sys, Sync
             const double rr = a.b[i] - A.row(i, VecLoad{a.x});
             d[0] = fma(rr, rr, d[0]);
         }
-        grid_sum<1>(g, d, sm, sflag);
+        exchange(g, d, X, [](Scalars &S, const double (&t)[1]) { S.aux = t[0]; });
         res.iters = o.iters;
         res.status = o.status;
         res.half_step = o.half;
         res.n_replacements = o.nrr;
         const double nr = o.iters > 0 ? sqrt(o.nr) : o.nr0;
         res.rel_res_recursive = o.nr0 > 0.0 ? nr / o.nr0 : 0.0;
-        res.rel_res_true = o.nr0 > 0.0 ? sqrt(d[0]) / o.nr0 : sqrt(d[0]);
+        res.rel_res_true = o.nr0 > 0.0 ? sqrt(X.s.aux) / o.nr0 : sqrt(X.s.aux);
     }
     if (part == 0 && threadIdx.x == 0) B.out[sys] = res;
 }
 
 __global__ void __launch_bounds__(kTPB, 6) batched_kernel(const BatchArgs B) {
-    __shared__ double sm[kMaxDots][32];
+    __shared__ Exchange<kTPB> X;
     __shared__ double slots[2][kMaxCluster][kSlotDoubles];   // cluster reductions: every CTA's block sums
     __shared__ int item[2];   // system of this CTA (-1: none), whole-cluster flag (-1: no work left)
-    __shared__ int sflag;
     const unsigned size = cluster_ctas(), rank = cluster_rank();
     if (size > 1) cluster_barrier();   // every CTA started before its shared memory is addressed
     for (;;) {
@@ -1554,10 +1535,10 @@ __global__ void __launch_bounds__(kTPB, 6) batched_kernel(const BatchArgs B) {
         if (whole < 0) return;   // the same for every CTA of the cluster
         if (whole == 1) {
             ClusterSync g{slots, rank, size, 0u, 0};
-            batched_system(B, sys, g, rank, size, sm, &sflag);
+            batched_system(B, sys, g, rank, size, X);
         } else if (sys >= 0) {
             BlockSync g{0};
-            batched_system(B, sys, g, 0u, 1u, sm, &sflag);
+            batched_system(B, sys, g, 0u, 1u, X);
         }
         // every CTA is done with this item (and with the slots) before the next claim
         if (size > 1) cluster_barrier();
@@ -1571,12 +1552,11 @@ __global__ void __launch_bounds__(kTPB, 6) batched_kernel(const BatchArgs B) {
 // PBCG_ERR_TIMEOUT in the abort flag; the others see the flag (or their own
 // limit) and return. Block 0 then reports the flag.
 __global__ void sync_timeout_probe_kernel(Control *ctl, double *slots, uint64_t limit_ns) {
-    __shared__ double sm[kMaxDots][32];
-    __shared__ int sflag;
+    __shared__ Exchange<kTPB> X;
     if (blockIdx.x == gridDim.x - 1) return;
-    if (threadIdx.x == 0) sflag = 1;
-    GridSync g{ctl, slots, 0u, 0, limit_ns};
-    const bool ok = grid_sync(g, sm, &sflag);
+    if (threadIdx.x == 0) X.ok = 1;
+    GridSync g{ctl, slots, 0u, 0, kTPB, limit_ns};
+    const bool ok = grid_sync(g, X);
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->status = ok ? (int)PBCG_OK : ld_relaxed_s32(&ctl->abort);
 }
 
