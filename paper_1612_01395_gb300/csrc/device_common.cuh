@@ -150,7 +150,7 @@ struct Exchange {
 };
 
 // Fixed-order block sums, returned to every lane of warp 0: the warps reduce
-// independently, then lane k of warp 0 adds value k of the warps in warp order.
+// independently, then warp 0 adds their sums.
 template <int K, int T>
 __device__ __forceinline__ void block_sum(double (&v)[K], Exchange<T> &X) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -161,16 +161,22 @@ __device__ __forceinline__ void block_sum(double (&v)[K], Exchange<T> &X) {
     }
     __syncthreads();
     if (wid == 0) {
-        double t = 0.0;
-        if (lane < K) {
-            t = X.part[0][lane];
-            const int warps = (int)(blockDim.x >> 5);
+        const int warps = (int)(blockDim.x >> 5);
+        if constexpr (T / 32 <= 8) {   // lane k adds value k of the warps in warp order
+            double t = 0.0;
+            if (lane < K) {
+                t = X.part[0][lane];
 #pragma unroll
-            for (int w = 1; w < T / 32; ++w)
-                if (w < warps) t += X.part[w][lane];
+                for (int w = 1; w < T / 32; ++w)
+                    if (w < warps) t += X.part[w][lane];
+            }
+#pragma unroll
+            for (int k = 0; k < K; ++k) v[k] = __shfl_sync(kFull, t, k);
+        } else {                       // lane w takes warp w: a tree is shorter than 15 additions in a row
+#pragma unroll
+            for (int k = 0; k < K; ++k) v[k] = lane < warps ? X.part[lane < warps ? lane : 0][k] : 0.0;
+            warp_allsum<K>(v);
         }
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = __shfl_sync(kFull, t, k);
     }
 }
 
@@ -344,62 +350,6 @@ __device__ __forceinline__ bool exchange(BlockSync &g, double (&v)[K], Exchange<
     if (threadIdx.x < 32) f(X.s, v);
     g.count++;
     __syncthreads();
-    return true;
-}
-
-// ---------------------------------------------------------------------------
-// 1-D bulk copies from global into shared memory (the TMA unit's untiled
-// copy, cp.async.bulk), completed on a shared-memory mbarrier. One thread
-// posts the expected byte count and issues the copies; every thread waits on
-// the barrier's phase. Addresses and sizes must be multiples of 16 bytes.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-// Make barrier initialisations visible to the asynchronous (copy) proxy.
-__device__ __forceinline__ void mbar_init_fence() {
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-// Order this thread's earlier generic-proxy global accesses before later
-// bulk copies (async proxy) of the same memory.
-__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
-
-// Wait until the barrier's phase of the given parity has completed. Bounded:
-// after kSyncTimeoutNs the launch is flagged PBCG_ERR_TIMEOUT and false is
-// returned (a copy can only stay incomplete if its byte count disagreed with
-// the posted one).
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, Control *ctl) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = globaltimer_ns();
-    while (!mbar_try_wait(bar, parity)) {
-        if (globaltimer_ns() - t0 > kSyncTimeoutNs) {
-            atomicCAS(&ctl->abort, 0, (int)PBCG_ERR_TIMEOUT);
-            return false;
-        }
-    }
     return true;
 }
 

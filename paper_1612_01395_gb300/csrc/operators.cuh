@@ -228,108 +228,97 @@ struct StencilOpT {
         return acc;
     }
 
-    // Coefficient d at the nodes (i, j, k) and (i+1, j, k): one load when the
-    // table does not vary along x (stride 0), else one per node; each sum of
-    // two tables formed per node as in coef().
-    __device__ __forceinline__ void coef2(int d, int i, int j, int k, C &v0, C &v1) const {
-        const StCoefT<C> &q = c[d];
-        if (q.t1) {
-            const int at = i * q.a1 + j * q.b1 + k * q.c1;
-            v0 = __ldg(q.t1 + PBCG_SAFE(at, q.len1));
-            v1 = q.a1 == 0 ? v0 : __ldg(q.t1 + PBCG_SAFE(at + q.a1, q.len1));
+    // ---- FP32 sweeps: groups of up to 4 adjacent rows of one x-line, so that
+    // a group shares the decomposition of its row number, the boundary tests
+    // and the coefficient loads that do not vary along x, and takes its vectors
+    // in 128-bit accesses where nx % 4 == 0 (then every group starts on a
+    // multiple of 4 rows, and so do its neighbours at nx and nx*ny).
+    int gx;        // groups per x-line, ceil(nx / 4)
+    FastDiv dg;    // by gx
+    int aligned;   // nx % 4 == 0
+
+    struct Group {
+        int r, cnt;     // first row, rows (4; fewer at the end of an x-line)
+        int i, j, k;    // node of the first row
+    };
+    __device__ __forceinline__ int groups() const { return gx * ny * nz; }
+    __device__ __forceinline__ Group group(int gi) const {
+        Group q;
+        const int t = (int)dg.div((uint32_t)gi);
+        q.i = 4 * (gi - t * gx);
+        q.k = (int)dy.div((uint32_t)t);
+        q.j = t - q.k * ny;
+        q.r = t * nx + q.i;
+        q.cnt = nx - q.i < 4 ? nx - q.i : 4;
+        return q;
+    }
+    // u at rows at .. at + cnt - 1, zero beyond
+    __device__ __forceinline__ void load4(const float *u, int at, int cnt, float (&v)[4]) const {
+        if (aligned) {
+            const float4 f = *reinterpret_cast<const float4 *>(u + PBCG_SAFE(at, n - 3));
+            v[0] = f.x;
+            v[1] = f.y;
+            v[2] = f.z;
+            v[3] = f.w;
         } else {
-            v0 = v1 = q.value;
-        }
-#pragma unroll 1
-        for (int m = 0; m < q.n2; ++m) {
-            const int at = i * q.a2 + j * q.b2 + k * q.c2;
-            const C w0 = __ldg(q.t2 + PBCG_SAFE(at, q.len2));
-            const C w1 = q.a2 == 0 ? w0 : __ldg(q.t2 + PBCG_SAFE(at + q.a2, q.len2));
-            v0 = add_rn(v0, w0);
-            v1 = add_rn(v1, w1);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v[m] = m < cnt ? u[PBCG_SAFE(at + m, n)] : 0.0f;
         }
     }
-
-    // Rows r and r+1 (r even) lie on one x-line for every even r when nx is
-    // even. The sweeps use row2 only then: with odd nx some pairs span two
-    // lines, and a warp holding one runs both of row2's paths.
-    __device__ __forceinline__ bool pairs_on_lines() const { return (nx & 1) == 0; }
-
-    // Rows r and r+1 (r even) of the FP32 inner sweeps, y[0] and y[1], each
-    // summed exactly as row() sums it: the same products in the same order,
-    // so the results are bitwise those of two row() calls. When both rows lie
-    // on one x-line they share the decomposition of r, the coefficient loads
-    // that do not vary along x, and their neighbour loads, taken as 64-bit
-    // pairs where both values are 8-byte aligned (r even; the offsets nx and
-    // nx*ny even). A pair that spans two x-lines (odd nx) takes two row()s.
-    template <class T>
-    __device__ __forceinline__ void row2(int r, const T *u, T (&y)[2]) const {
-        static_assert(sizeof(T) == 4 && sizeof(C) == 4, "pairs of FP32 rows");
-        const int t = (int)dx.div((uint32_t)r);
-        const int i = r - t * nx;
-        if (i + 1 >= nx) {
-            const VecLoadT<T> L{u};
-            y[0] = row(r, L);
-            y[1] = row(r + 1, L);
-            return;
-        }
-        const int k = (int)dy.div((uint32_t)t);
-        const int j = t - k * ny;
-        // u at offset o and o + 1 from r (o even when `even`)
-        auto pair_at = [&](int o, bool even, T &a, T &b) {
-            const int at = PBCG_SAFE(r + o, n - 1);   // both at and at + 1 in range
-            if (even) {
-                const float2 v = *reinterpret_cast<const float2 *>(u + at);
-                a = v.x;
-                b = v.y;
+    // acc[m] += coefficient d at node (i + m, j, k) * v[m]; each sum of two
+    // tables formed per node as in coef()
+    __device__ __forceinline__ void add4(int d, const Group &q, const float (&v)[4], float (&acc)[4]) const {
+        const StCoefT<C> &f = c[d];
+        float w[4];
+        if (f.t1) {
+            const int at = q.i * f.a1 + q.j * f.b1 + q.k * f.c1;
+            w[0] = __ldg(f.t1 + PBCG_SAFE(at, f.len1));
+            if (f.a1 == 0) {
+                w[1] = w[2] = w[3] = w[0];
             } else {
-                a = u[at];
-                b = u[at + 1];
+#pragma unroll
+                for (int m = 1; m < 4; ++m) w[m] = m < q.cnt ? __ldg(f.t1 + PBCG_SAFE(at + m * f.a1, f.len1)) : 0.0f;
             }
-        };
-        T a0 = T(0), a1 = T(0);
-        C c0, c1;
-        if (k > 0) {
-            T v0, v1;
-            pair_at(-nxy, (nxy & 1) == 0, v0, v1);
-            coef2(PBCG_B, i, j, k, c0, c1);
-            a0 = fmaT((T)c0, v0, a0);
-            a1 = fmaT((T)c1, v1, a1);
+        } else {
+            w[0] = w[1] = w[2] = w[3] = f.value;
         }
-        if (j > 0) {
-            T v0, v1;
-            pair_at(-nx, (nx & 1) == 0, v0, v1);
-            coef2(PBCG_S, i, j, k, c0, c1);
-            a0 = fmaT((T)c0, v0, a0);
-            a1 = fmaT((T)c1, v1, a1);
+        if (f.n2) {
+            const int at = q.i * f.a2 + q.j * f.b2 + q.k * f.c2;
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (m < q.cnt) w[m] = add_rn(w[m], __ldg(f.t2 + PBCG_SAFE(at + m * f.a2, f.len2)));
         }
-        T u0, u1;
-        pair_at(0, true, u0, u1);
-        coef2(PBCG_W, i, j, k, c0, c1);
-        if (i > 0) a0 = fmaT((T)c0, u[PBCG_SAFE(r - 1, n)], a0);
-        a1 = fmaT((T)c1, u0, a1);
-        coef2(PBCG_C, i, j, k, c0, c1);
-        a0 = fmaT((T)c0, u0, a0);
-        a1 = fmaT((T)c1, u1, a1);
-        coef2(PBCG_E, i, j, k, c0, c1);
-        a0 = fmaT((T)c0, u1, a0);
-        if (i + 2 < nx) a1 = fmaT((T)c1, u[PBCG_SAFE(r + 2, n)], a1);
-        if (j < ny - 1) {
-            T v0, v1;
-            pair_at(nx, (nx & 1) == 0, v0, v1);
-            coef2(PBCG_N, i, j, k, c0, c1);
-            a0 = fmaT((T)c0, v0, a0);
-            a1 = fmaT((T)c1, v1, a1);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc[m] = fmaT(w[m], v[m], acc[m]);
+    }
+    // y = A u on the rows of a group, mid = u there; each row summed as row()
+    // sums it, except that a neighbour outside the grid adds 0 instead of
+    // nothing (no change to a finite sum). Rows past cnt read 0.
+    __device__ __forceinline__ void product4(const Group &q, const float *u, float (&mid)[4], float (&y)[4]) const {
+        float vb[4] = {}, vs[4] = {}, vn[4] = {}, vt[4] = {}, ve[4], vw[4];
+        if (q.k > 0) load4(u, q.r - nxy, q.cnt, vb);
+        if (q.j > 0) load4(u, q.r - nx, q.cnt, vs);
+        load4(u, q.r, q.cnt, mid);
+        if (q.j < ny - 1) load4(u, q.r + nx, q.cnt, vn);
+        if (q.k < nz - 1) load4(u, q.r + nxy, q.cnt, vt);
+        const float left = q.i > 0 ? u[PBCG_SAFE(q.r - 1, n)] : 0.0f;
+        const float right = q.i + 4 < nx ? u[PBCG_SAFE(q.r + 4, n)] : 0.0f;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            vw[m] = m > 0 ? mid[m - 1] : left;
+            ve[m] = m < 3 ? mid[m + 1] : right;
+            y[m] = 0.0f;
         }
-        if (k < nz - 1) {
-            T v0, v1;
-            pair_at(nxy, (nxy & 1) == 0, v0, v1);
-            coef2(PBCG_T, i, j, k, c0, c1);
-            a0 = fmaT((T)c0, v0, a0);
-            a1 = fmaT((T)c1, v1, a1);
-        }
-        y[0] = a0;
-        y[1] = a1;
+        if (q.k > 0) add4(PBCG_B, q, vb, y);
+        if (q.j > 0) add4(PBCG_S, q, vs, y);
+        add4(PBCG_W, q, vw, y);
+        add4(PBCG_C, q, mid, y);
+        add4(PBCG_E, q, ve, y);
+        if (q.j < ny - 1) add4(PBCG_N, q, vn, y);
+        if (q.k < nz - 1) add4(PBCG_T, q, vt, y);
+#pragma unroll
+        for (int m = 1; m < 4; ++m)
+            if (m >= q.cnt) y[m] = 0.0f;
     }
 };
 using StencilOp = StencilOpT<double>;
@@ -345,13 +334,13 @@ struct SweepLoadsL2<CsrOpGatherL2> {
     static constexpr bool value = true;
 };
 
-// Operators with row2 (pairs of FP32 rows).
+// Operators with groups of FP32 rows.
 template <class Op>
-struct HasRow2 {
+struct HasGroups {
     static constexpr bool value = false;
 };
 template <>
-struct HasRow2<StencilOpT<float, false>> {
+struct HasGroups<StencilOpT<float, false>> {
     static constexpr bool value = true;
 };
 

@@ -177,37 +177,6 @@ long long max_index(const int64_t st[3], int nx, int ny, int nz) {
     return st[0] * (long long)(nx - 1) + st[1] * (long long)(ny - 1) + st[2] * (long long)(nz - 1);
 }
 
-// Work of a sweep: rows x max(1, entries per row / 7).
-double sweep_work(const pbicgstab_s *h) {
-    const double per_row = h->n > 0 ? (double)h->nnz / (double)h->n : 0.0;
-    return (double)h->n * (per_row > 7.0 ? per_row / 7.0 : 1.0);
-}
-
-// Blocks of the mixed-precision kernel (128 threads), occ co-resident per SM.
-int pick_grid(const pbicgstab_s *h, int occ, int req) {
-    int max_grid = occ * h->num_sms;
-    if (max_grid > pbcg::kMaxGrid) max_grid = pbcg::kMaxGrid;
-    if (req > 0) return req < max_grid ? req : max_grid;
-    // The time of an iteration is the sweep (rows per thread, one after the
-    // other) plus the grid-wide exchanges, whose cost grows with the number of
-    // blocks. Block counts by work, measured on GB300: 128 blocks up to
-    // w = 80k, then 2, 3, 4, 5 blocks per SM up to 180k, 400k, 1.2M, 3M and all
-    // co-resident blocks beyond; never fewer than one row per thread up to that
-    // count.
-    const double w = sweep_work(h);
-    long long want;
-    if (w <= 80000.0) {
-        want = 128;
-    } else {
-        const int per_sm = w <= 180000.0 ? 2 : w <= 400000.0 ? 3 : w <= 1200000.0 ? 4 : w <= 3000000.0 ? 5 : occ;
-        want = (long long)per_sm * h->num_sms;
-    }
-    const long long one_row = ((long long)h->n + pbcg::kTPB - 1) / pbcg::kTPB;
-    if (want > one_row) want = one_row;
-    if (want < 1) want = 1;
-    return (int)(want < max_grid ? want : max_grid);
-}
-
 // Kernel and launch shape of a grid solve. The blocks fill the SMs only where
 // the sweep is long enough to pay for what each block adds to an exchange, and
 // never hold less than one row per thread. Measured per iteration, p-BiCGStab /
@@ -635,18 +604,32 @@ namespace {
 template <class Op64, class Op32>
 pbcg_status launch_mixed(pbicgstab_s *h, const Op64 &a64, const Op32 &a32, const pbcg::MixedArgs &m, int req_grid,
                          int *grid_out) {
-    // stencil inner sweeps stage their streamed vectors in dynamic shared memory
-    const size_t smem = pbcg::HasRow2<Op32>::value ? pbcg::kStageSmemBytes : 0;
-    int occ = 0;
-    PBCG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pbcg::mixed_kernel<Op64, Op32>, pbcg::kTPB, smem));
-    if (occ < 1) return fail(PBCG_ERR_CUDA, "mixed-precision kernel cannot be resident on an SM");
-    const int grid = pick_grid(h, occ, req_grid);
+    // Blocks per SM by rows, as for the grid solvers (an exchange costs more
+    // blocks more; us per FP32 iteration, stencil / CSR, at 1 and 2 blocks of
+    // 256 per SM: 110k rows 19.8 / 20.5 and 24.4 / 23.9; 262k 25.1 / 27.5 and
+    // 26.6 / 28.4; 512k 36.8 / 43.1 and 32.2 / 36.6). A forced grid takes
+    // smaller blocks where the larger ones are not all resident.
+    int block = pbcg::kMixedTPB, occ = 0, grid = req_grid;
+    for (;; block /= 2) {
+        PBCG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pbcg::mixed_kernel<Op64, Op32>, block, 0));
+        if (occ < 1) return fail(PBCG_ERR_CUDA, "mixed-precision kernel cannot be resident on an SM");
+        if (req_grid <= occ * h->num_sms || block == 64) break;
+    }
+    const int all = occ * h->num_sms;
+    if (req_grid == 0) {
+        const int per_sm = h->n <= 300000 ? 1 : h->n <= 1000000 ? 2 : occ;
+        const long long one_row = ((long long)h->n + block - 1) / block;
+        grid = (per_sm < occ ? per_sm : occ) * h->num_sms;
+        if (grid > one_row) grid = (int)one_row;
+    }
+    if (grid > all) grid = all;
+    if (grid > pbcg::kMaxGrid) grid = pbcg::kMaxGrid;
     *grid_out = grid;
     PBCG_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(pbcg::Control), h->stream));
     if (h->ev0) PBCG_CUDA(cudaEventRecord(h->ev0, h->stream));
     void *params[3] = {(void *)&a64, (void *)&a32, (void *)&m};
-    PBCG_CUDA(cudaLaunchCooperativeKernel((const void *)pbcg::mixed_kernel<Op64, Op32>, dim3(grid),
-                                          dim3(pbcg::kTPB), params, smem, h->stream));
+    PBCG_CUDA(cudaLaunchCooperativeKernel((const void *)pbcg::mixed_kernel<Op64, Op32>, dim3(grid), dim3(block),
+                                          params, 0, h->stream));
     if (h->ev1) PBCG_CUDA(cudaEventRecord(h->ev1, h->stream));
     return PBCG_OK;
 }
@@ -724,6 +707,9 @@ extern "C" pbcg_status pbicgstab_solve_mixed(pbicgstab_t h, const void *d_val_lo
         a32.nxy = a64.nxy;
         a32.dx = a64.dx;
         a32.dy = a64.dy;
+        a32.gx = (a64.nx + 3) / 4;
+        a32.dg.init((uint32_t)a32.gx);
+        a32.aligned = a64.nx % 4 == 0;
         float *tab = f0 + 14 * s;
         const size_t cap = 10 * s;
         size_t used = 0;

@@ -262,16 +262,26 @@ struct DotsFor<true, P, double, B> {
 };
 constexpr int kWideSlots = 5;   // dot products of the largest reduction
 
-// G adjacent elements p[i..i+cnt) of a vector (cnt <= G; the rest read as 0)
-// and their store. G = 2 uses one 64-bit access when both are present: i is
-// even and the vectors are 8-byte aligned (the FP32 inner sweeps).
+// Adjacent elements p[i..i+cnt) of a vector (cnt <= G; the rest read as 0) and
+// their store. wide: the FP32 sweeps' one 64-bit (G = 2) or 128-bit (G = 4)
+// access, where all G elements are present and i is a multiple of G.
 template <int G, typename T>
-__device__ __forceinline__ void load_group(const T *p, int i, int cnt, T (&out)[G]) {
-    if constexpr (G == 2 && sizeof(T) == 4) {
-        if (cnt == 2) {
+__device__ __forceinline__ void load_group(const T *p, int i, int cnt, bool wide, T (&out)[G]) {
+    if constexpr (G == 2) {
+        if (wide) {
             const float2 q = *reinterpret_cast<const float2 *>(p + i);
             out[0] = q.x;
             out[1] = q.y;
+            return;
+        }
+    }
+    if constexpr (G == 4) {
+        if (wide) {
+            const float4 q = *reinterpret_cast<const float4 *>(p + i);
+            out[0] = q.x;
+            out[1] = q.y;
+            out[2] = q.z;
+            out[3] = q.w;
             return;
         }
     }
@@ -281,19 +291,25 @@ __device__ __forceinline__ void load_group(const T *p, int i, int cnt, T (&out)[
 // load_group for a fused sweep: through L2 only (ld.global.cg) for operators
 // whose sweeps leave L1 to their SpMV's row streams.
 template <class Op, int G, typename T>
-__device__ __forceinline__ void load_sweep(const T *p, int i, int cnt, T (&out)[G]) {
+__device__ __forceinline__ void load_sweep(const T *p, int i, int cnt, bool wide, T (&out)[G]) {
     if constexpr (SweepLoadsL2<Op>::value) {
 #pragma unroll
         for (int u = 0; u < G; ++u) out[u] = u < cnt ? __ldcg(p + i + u) : T(0);
     } else {
-        load_group(p, i, cnt, out);
+        load_group(p, i, cnt, wide, out);
     }
 }
 template <int G, typename T>
-__device__ __forceinline__ void store_group(T *p, int i, int cnt, const T (&in)[G]) {
-    if constexpr (G == 2 && sizeof(T) == 4) {
-        if (cnt == 2) {
+__device__ __forceinline__ void store_group(T *p, int i, int cnt, bool wide, const T (&in)[G]) {
+    if constexpr (G == 2) {
+        if (wide) {
             *reinterpret_cast<float2 *>(p + i) = make_float2(in[0], in[1]);
+            return;
+        }
+    }
+    if constexpr (G == 4) {
+        if (wide) {
+            *reinterpret_cast<float4 *>(p + i) = make_float4(in[0], in[1], in[2], in[3]);
             return;
         }
     }
@@ -302,93 +318,40 @@ __device__ __forceinline__ void store_group(T *p, int i, int cnt, const T (&in)[
         if (u < cnt) p[i + u] = in[u];
 }
 
-// ===========================================================================
-// Staged FP32 stencil sweeps (the inner solves of the mixed-precision
-// refinement). These sweeps move 96 bytes per unknown and iteration and were
-// bound by load latency with every thread issuing its own vector loads. Here
-// the vectors a phase streams (read once, by the rows' own block) arrive in
-// shared memory by 1-D bulk copies: a block walks its rows in tiles of
-// kStageRows, thread 0 keeps kStages - 1 tiles in flight ahead of the one it
-// computes, and the threads read their rows from shared memory. Each buffer
-// has a "full" mbarrier (the copies' bytes arrived) and an "empty" one (all
-// threads have read it): thread 0 refills a buffer only after every thread
-// released it, so warps are not held together tile by tile and may run up to
-// kStages - 1 tiles apart. The SpMV input (neighbours in other tiles and
-// blocks) and the stores stay ordinary global accesses. Block row ranges
-// start on multiples of 4 rows, so every copy starts on a 16-byte boundary;
-// the last tile's copy is rounded up to 16 bytes, inside the vectors' padding.
-// ===========================================================================
-// (The same staging of the FP64 stencil sweeps of Algorithm 9 gave bitwise
-// identical results but was 2.7 % slower at 256^3, 1178 against 1148 us per
-// iteration: those sweeps are bound by the FP64 pipe, and staging only adds
-// instructions. They keep their direct loads.)
-constexpr int kStageTileBytes = 1024;   // per vector and tile: 256 FP32 rows (a pair per thread) or 128 FP64 rows
-constexpr int kStages = 3;              // buffers: 2 tiles in flight ahead
-constexpr int kStageVecs = 6;           // streamed vectors per phase
-constexpr int kStageRows = kStageTileBytes / (int)sizeof(float);   // FP32 rows per tile
-constexpr size_t kStageSmemBytes = (size_t)kStages * kStageVecs * kStageTileBytes;
-
-struct Stager {
-    char *buf;         // shared [kStages][kStageVecs][kStageTileBytes]
-    uint64_t *full;    // shared [kStages]: copies of the buffer's tile arrived (count 1 + bytes)
-    uint64_t *empty;   // shared [kStages]: every thread finished reading the buffer (count kTPB)
-    unsigned seq;      // tiles begun by this block so far (every thread holds the same value)
-    Control *ctl;
+// Adjacent rows that a thread takes at a step of the two main sweeps, all
+// loaded before any is stored (the stores of one row may alias the loads of
+// the next as far as the compiler knows). FP64 sweeps are bound by the FP64
+// pipe and take one row; FP32 sweeps take two (CSR) or four of an x-line
+// (stencil, StencilOpT::Group) with 64- and 128-bit accesses. Groups are only
+// used on a grid, whose rows start at 0.
+template <class Op, typename T>
+struct RowGroup {
+    static constexpr int kRows = sizeof(T) == 8 ? 1 : HasGroups<Op>::value ? 4 : 2;
 };
-
-// thread 0: post and issue the copies of tile `seq` (rows [row0, row0 + rows)),
-// the byte count rounded up to 16.
-template <typename T, int NV>
-__device__ __forceinline__ void stage_issue(const Stager &S, unsigned seq, const T *const *src, int row0, int rows) {
-    const unsigned b = seq % kStages;
-    const unsigned bytes = ((unsigned)rows * (unsigned)sizeof(T) + 15u) & ~15u;
-    mbar_arrive_expect_tx(&S.full[b], bytes * NV);
+// Groups of the sweep: a group's number takes the place of a row's in PBCG_ROWS.
+template <class Op, int G>
+__device__ __forceinline__ int group_end(const Op &A, int hi) {
+    if constexpr (HasGroups<Op>::value && G == 4) return A.groups();
+    else return (hi + G - 1) / G;
+}
+// Rows i0 .. i0 + cnt - 1 of group gi, y = A u there and mid = u there (where asked for).
+template <bool kMid, class Op, int G, typename T>
+__device__ __forceinline__ void group_product(const Op &A, int gi, int hi, const T *u, int &i0, int &cnt, bool &wide,
+                                              T (&mid)[G], T (&y)[G]) {
+    if constexpr (HasGroups<Op>::value && G == 4) {
+        const auto q = A.group(gi);
+        i0 = q.r;
+        cnt = q.cnt;
+        wide = A.aligned != 0;
+        A.product4(q, u, mid, y);
+    } else {
+        i0 = G * gi;
+        cnt = G == 1 ? 1 : (hi - i0 < G ? hi - i0 : G);
+        wide = G > 1 && cnt == G;
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-        bulk_g2s(S.buf + ((size_t)b * kStageVecs + k) * kStageTileBytes, src[k] + row0, bytes, &S.full[b]);
-}
-
-// Run body(tile buffer, first row of the tile) over the block's rows [lo, hi)
-// with the NV (<= kStageVecs) vectors `src` staged, in tiles of
-// kStageTileBytes / sizeof(T) rows. Every staged vector must be a workspace
-// vector (16-byte aligned, padded past n). Returns false if a wait timed out.
-template <typename T, int NV, class Body>
-__device__ __forceinline__ bool staged_sweep(Stager &S, const T *const *src, int lo, int hi, Body body) {
-    static_assert(NV <= kStageVecs, "at most kStageVecs staged vectors");
-    constexpr int R = kStageTileBytes / (int)sizeof(T);
-    const int ntiles = hi > lo ? (hi - lo + R - 1) / R : 0;
-    // every thread: earlier generic writes of these rows (this block's, made
-    // visible by the preceding barriers) before the copies read them; after
-    // this barrier every thread has also released every buffer
-    fence_proxy_async_global();
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int t = 0; t < kStages - 1 && t < ntiles; ++t) {
-            const int r0 = lo + t * R;
-            stage_issue<T, NV>(S, S.seq + t, src, r0, hi - r0 < R ? hi - r0 : R);
-        }
-    for (int t = 0; t < ntiles; ++t) {
-        const unsigned seq = S.seq + (unsigned)t;
-        const int ahead = t + kStages - 1;
-        if (threadIdx.x == 0 && ahead < ntiles) {
-            // the buffer of tile seq + kStages - 1 last held tile seq - 1: wait until all threads released it
-            if (seq >= 1 && !mbar_wait(&S.empty[(seq - 1) % kStages], ((seq - 1) / kStages) & 1u, S.ctl)) return false;
-            const int r0 = lo + ahead * R;
-            stage_issue<T, NV>(S, seq + kStages - 1, src, r0, hi - r0 < R ? hi - r0 : R);
-        }
-        if (!mbar_wait(&S.full[seq % kStages], (seq / kStages) & 1u, S.ctl)) return false;
-        body(reinterpret_cast<const T *>(S.buf + (size_t)(seq % kStages) * kStageVecs * kStageTileBytes), lo + t * R);
-        mbar_arrive(&S.empty[seq % kStages]);   // this thread is done with the buffer
+        for (int m = 0; m < G; ++m) y[m] = m < cnt ? A.row(i0 + m, VecLoadT<T>{u}) : T(0);
+        if constexpr (kMid) load_sweep<Op>(u, i0, cnt, wide, mid);
     }
-    S.seq += (unsigned)ntiles;
-    return true;
-}
-
-// Elements j, j+1 of a staged vector (j even: one 64-bit shared load).
-__device__ __forceinline__ void staged_pair(const float *tb, int k, int j, float (&out)[2]) {
-    const float2 v = *reinterpret_cast<const float2 *>(tb + k * kStageRows + j);
-    out[0] = v.x;
-    out[1] = v.y;
 }
 
 // ===========================================================================
@@ -402,19 +365,11 @@ __device__ __forceinline__ void staged_pair(const float *tb, int k, int j, float
 // alpha, beta, omega, rho are doubles; a sweep uses them rounded to T.
 template <class Op, typename T, int B, class Sync = GridSync, bool Wide = false>
 __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> &a, Sync &g, Exchange<B> &X,
-                                               int lo, int hi, Outcome &o, int &spmvs, WideSlot *wide,
-                                               Stager *stg = nullptr) {
+                                               int lo, int hi, Outcome &o, int &spmvs, WideSlot *wide) {
     const VectorsT<T> &V = a.V;
     T *x = a.x;
     const bool fixed = a.fixed != 0;
-    // Rows per thread and step of the two main sweeps: kGroup adjacent rows,
-    // loaded before any is stored (the stores of one row may alias the loads
-    // of the next as far as the compiler knows). FP64 sweeps are bound by the
-    // FP64 pipe and take one row. The FP32 inner sweeps are bound by load
-    // latency and take two adjacent rows with 64-bit vector accesses, which
-    // halves their load and store instructions; their callers give every
-    // block an even first row.
-    constexpr int kGroup = sizeof(T) == 4 ? 2 : 1;
+    constexpr int kGroup = RowGroup<Op, T>::kRows;
 
     // r_0 := b - A x_0; shadow r0 := r_0; p, s, z, v := 0 (they are multiplied by beta_{-1} = 0)
     double d0[1];
@@ -459,78 +414,19 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
         // ---- phase A: t_i = A w_i; p_i, s_i, z_i, q_i, y_i; first reduction
         typename DotsFor<Wide, PairsPipeA, T, B>::type a1(wide, lo + (int)threadIdx.x < hi);   // (q,y) (y,y) (q,q) (r0,s) (r0,z)
         const T al = (T)X.s.alpha, be = (T)X.s.beta, om = (T)X.s.omega;
-        bool swept = false;   // the staged sweep did phase A
-        if constexpr (kGroup == 2 && HasRow2<Op>::value) {
-            if (!replaced_rw && stg) {
-                // staged: r s z p v r0 through shared memory, w (SpMV) from global
-                const float *src[kStageVecs] = {V.r, V.s, V.z, V.p, V.v, V.r0};
-                const bool ok = staged_sweep<float, kStageVecs>(*stg, src, lo, hi, [&](const float *tb, int row0) {
-                    const int j = 2 * (int)threadIdx.x;
-                    const int i0 = row0 + j;
-                    if (i0 >= hi) return;
-                    const int cnt = hi - i0 < 2 ? hi - i0 : 2;
-                    T ti[2] = {}, ri[2], wi[2], si[2], zi[2], pi[2], vi[2], r0i[2];
-                    if (cnt == 2 && A.pairs_on_lines()) {
-                        A.row2(i0, V.w, ti);
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < 2; ++u)
-                            if (u < cnt) ti[u] = A.row(i0 + u, VecLoadT<T>{V.w});
-                    }
-                    load_group(V.w, i0, cnt, wi);
-                    staged_pair(tb, 0, j, ri);
-                    staged_pair(tb, 1, j, si);
-                    staged_pair(tb, 2, j, zi);
-                    staged_pair(tb, 3, j, pi);
-                    staged_pair(tb, 4, j, vi);
-                    staged_pair(tb, 5, j, r0i);
-                    T pn[2], sn[2], zn[2], qn[2], yn[2];
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        pn[u] = fmaT(be, fmaT(-om, si[u], pi[u]), ri[u]);   // p_i
-                        sn[u] = fmaT(be, fmaT(-om, zi[u], si[u]), wi[u]);   // s_i, eq. (1)
-                        zn[u] = fmaT(be, fmaT(-om, vi[u], zi[u]), ti[u]);   // z_i, eq. (6)
-                        qn[u] = fmaT(-al, sn[u], ri[u]);                    // q_i
-                        yn[u] = fmaT(-al, zn[u], wi[u]);                    // y_i, eq. (4)
-                        if (u < cnt) a1.add({qn[u], yn[u], r0i[u], sn[u], zn[u]});
-                    }
-                    store_group(V.t, i0, cnt, ti);
-                    store_group(V.p, i0, cnt, pn);
-                    store_group(V.s, i0, cnt, sn);
-                    store_group(V.z, i0, cnt, zn);
-                    store_group(V.q, i0, cnt, qn);
-                    store_group(V.y, i0, cnt, yn);
-                });
-                if (!ok) return false;
-                ++spmvs;
-                swept = true;
-            }
-        }
-        if (swept) {
-        } else if (!replaced_rw) {
-            for (int i0 = lo + kGroup * (int)threadIdx.x; i0 < hi; i0 += kGroup * row_step(g)) {
-                const int cnt = kGroup == 1 ? 1 : (hi - i0 < kGroup ? hi - i0 : kGroup);
-                T ti[kGroup] = {}, ri[kGroup], wi[kGroup], si[kGroup], zi[kGroup], pi[kGroup], vi[kGroup], r0i[kGroup];
-                if constexpr (kGroup == 2 && HasRow2<Op>::value) {
-                    if (cnt == 2 && A.pairs_on_lines()) {
-                        A.row2(i0, V.w, ti);
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < kGroup; ++u)
-                            if (u < cnt) ti[u] = A.row(i0 + u, VecLoadT<T>{V.w});
-                    }
-                } else {
-#pragma unroll
-                    for (int u = 0; u < kGroup; ++u)
-                        if (u < cnt) ti[u] = A.row(i0 + u, VecLoadT<T>{V.w});
-                }
-                load_sweep<Op>(V.r, i0, cnt, ri);
-                load_sweep<Op>(V.w, i0, cnt, wi);
-                load_sweep<Op>(V.s, i0, cnt, si);
-                load_sweep<Op>(V.z, i0, cnt, zi);
-                load_sweep<Op>(V.p, i0, cnt, pi);
-                load_sweep<Op>(V.v, i0, cnt, vi);
-                load_sweep<Op>(V.r0, i0, cnt, r0i);
+        if (!replaced_rw) {
+            const int end = group_end<Op, kGroup>(A, hi);
+            for (int gi = lo + (int)threadIdx.x; gi < end; gi += row_step(g)) {
+                int i0, cnt;
+                bool vec;
+                T ti[kGroup], ri[kGroup], wi[kGroup], si[kGroup], zi[kGroup], pi[kGroup], vi[kGroup], r0i[kGroup];
+                group_product<true>(A, gi, hi, V.w, i0, cnt, vec, wi, ti);
+                load_sweep<Op>(V.r, i0, cnt, vec, ri);
+                load_sweep<Op>(V.s, i0, cnt, vec, si);
+                load_sweep<Op>(V.z, i0, cnt, vec, zi);
+                load_sweep<Op>(V.p, i0, cnt, vec, pi);
+                load_sweep<Op>(V.v, i0, cnt, vec, vi);
+                load_sweep<Op>(V.r0, i0, cnt, vec, r0i);
                 T pn[kGroup], sn[kGroup], zn[kGroup], qn[kGroup], yn[kGroup];
 #pragma unroll
                 for (int u = 0; u < kGroup; ++u) {
@@ -539,14 +435,14 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
                     zn[u] = fmaT(be, fmaT(-om, vi[u], zi[u]), ti[u]);   // z_i, eq. (6)
                     qn[u] = fmaT(-al, sn[u], ri[u]);                    // q_i
                     yn[u] = fmaT(-al, zn[u], wi[u]);                    // y_i, eq. (4)
-                    if (u < cnt) a1.add({qn[u], yn[u], r0i[u], sn[u], zn[u]});
+                    if (kGroup != 2 || u < cnt) a1.add({qn[u], yn[u], r0i[u], sn[u], zn[u]});
                 }
-                store_group(V.t, i0, cnt, ti);
-                store_group(V.p, i0, cnt, pn);
-                store_group(V.s, i0, cnt, sn);
-                store_group(V.z, i0, cnt, zn);
-                store_group(V.q, i0, cnt, qn);
-                store_group(V.y, i0, cnt, yn);
+                store_group(V.t, i0, cnt, vec, ti);
+                store_group(V.p, i0, cnt, vec, pn);
+                store_group(V.s, i0, cnt, vec, sn);
+                store_group(V.z, i0, cnt, vec, zn);
+                store_group(V.q, i0, cnt, vec, qn);
+                store_group(V.y, i0, cnt, vec, yn);
             }
             ++spmvs;
         } else {
@@ -597,84 +493,31 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
                                  (a.max_repl < 0 || o.nrr < a.max_repl);
         typename DotsFor<Wide, PairsPipeB, T, B>::type a2(wide, lo + (int)threadIdx.x < hi);   // (r0,r) (r0,w) (r,r)
         const T om2 = (T)X.s.omega;
-        bool swept_b = false;   // the staged sweep did phase B
-        if constexpr (kGroup == 2 && HasRow2<Op>::value) {
-            if (!replace_now && stg) {
-                // staged: q y x p t r0 through shared memory, z (SpMV) from global
-                const float *src[kStageVecs] = {V.q, V.y, x, V.p, V.t, V.r0};
-                const bool ok = staged_sweep<float, kStageVecs>(*stg, src, lo, hi, [&](const float *tb, int row0) {
-                    const int j = 2 * (int)threadIdx.x;
-                    const int i0 = row0 + j;
-                    if (i0 >= hi) return;
-                    const int cnt = hi - i0 < 2 ? hi - i0 : 2;
-                    T vi[2] = {}, qi[2], yi[2], xi[2], pi[2], ti[2], r0i[2];
-                    if (cnt == 2 && A.pairs_on_lines()) {
-                        A.row2(i0, V.z, vi);
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < 2; ++u)
-                            if (u < cnt) vi[u] = A.row(i0 + u, VecLoadT<T>{V.z});
-                    }
-                    staged_pair(tb, 0, j, qi);
-                    staged_pair(tb, 1, j, yi);
-                    staged_pair(tb, 2, j, xi);
-                    staged_pair(tb, 3, j, pi);
-                    staged_pair(tb, 4, j, ti);
-                    staged_pair(tb, 5, j, r0i);
-                    T xn[2], rn[2], wn[2];
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        xn[u] = fmaT(om2, qi[u], fmaT(al, pi[u], xi[u]));
-                        rn[u] = fmaT(-om2, yi[u], qi[u]);                     // eq. (7)
-                        wn[u] = fmaT(-om2, fmaT(-al, vi[u], ti[u]), yi[u]);   // eq. (8)
-                        if (u < cnt) a2.add({r0i[u], rn[u], wn[u]});
-                    }
-                    store_group(x, i0, cnt, xn);
-                    store_group(V.v, i0, cnt, vi);
-                    store_group(V.r, i0, cnt, rn);
-                    store_group(V.w, i0, cnt, wn);
-                });
-                if (!ok) return false;
-                ++spmvs;
-                swept_b = true;
-            }
-        }
-        if (swept_b) {
-        } else if (!replace_now) {
-            for (int i0 = lo + kGroup * (int)threadIdx.x; i0 < hi; i0 += kGroup * row_step(g)) {
-                const int cnt = kGroup == 1 ? 1 : (hi - i0 < kGroup ? hi - i0 : kGroup);
-                T vi[kGroup] = {}, qi[kGroup], yi[kGroup], xi[kGroup], pi[kGroup], ti[kGroup], r0i[kGroup];
-                if constexpr (kGroup == 2 && HasRow2<Op>::value) {
-                    if (cnt == 2 && A.pairs_on_lines()) {
-                        A.row2(i0, V.z, vi);
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < kGroup; ++u)
-                            if (u < cnt) vi[u] = A.row(i0 + u, VecLoadT<T>{V.z});
-                    }
-                } else {
-#pragma unroll
-                    for (int u = 0; u < kGroup; ++u)
-                        if (u < cnt) vi[u] = A.row(i0 + u, VecLoadT<T>{V.z});
-                }
-                load_sweep<Op>(V.q, i0, cnt, qi);
-                load_sweep<Op>(V.y, i0, cnt, yi);
-                load_sweep<Op>(x, i0, cnt, xi);
-                load_sweep<Op>(V.p, i0, cnt, pi);
-                load_sweep<Op>(V.t, i0, cnt, ti);
-                load_sweep<Op>(V.r0, i0, cnt, r0i);
+        if (!replace_now) {
+            const int end = group_end<Op, kGroup>(A, hi);
+            for (int gi = lo + (int)threadIdx.x; gi < end; gi += row_step(g)) {
+                int i0, cnt;
+                bool vec;
+                T vi[kGroup], mid[kGroup], qi[kGroup], yi[kGroup], xi[kGroup], pi[kGroup], ti[kGroup], r0i[kGroup];
+                group_product<false>(A, gi, hi, V.z, i0, cnt, vec, mid, vi);
+                load_sweep<Op>(V.q, i0, cnt, vec, qi);
+                load_sweep<Op>(V.y, i0, cnt, vec, yi);
+                load_sweep<Op>(x, i0, cnt, vec, xi);
+                load_sweep<Op>(V.p, i0, cnt, vec, pi);
+                load_sweep<Op>(V.t, i0, cnt, vec, ti);
+                load_sweep<Op>(V.r0, i0, cnt, vec, r0i);
                 T xn[kGroup], rn[kGroup], wn[kGroup];
 #pragma unroll
                 for (int u = 0; u < kGroup; ++u) {
                     xn[u] = fmaT(om2, qi[u], fmaT(al, pi[u], xi[u]));
                     rn[u] = fmaT(-om2, yi[u], qi[u]);                     // eq. (7)
                     wn[u] = fmaT(-om2, fmaT(-al, vi[u], ti[u]), yi[u]);   // eq. (8)
-                    if (u < cnt) a2.add({r0i[u], rn[u], wn[u]});
+                    if (kGroup != 2 || u < cnt) a2.add({r0i[u], rn[u], wn[u]});
                 }
-                store_group(x, i0, cnt, xn);
-                store_group(V.v, i0, cnt, vi);
-                store_group(V.r, i0, cnt, rn);
-                store_group(V.w, i0, cnt, wn);
+                store_group(x, i0, cnt, vec, xn);
+                store_group(V.v, i0, cnt, vec, vi);
+                store_group(V.r, i0, cnt, vec, rn);
+                store_group(V.w, i0, cnt, vec, wn);
             }
             ++spmvs;
         } else {
@@ -1222,35 +1065,18 @@ struct MixedArgs {
     int stall_steps;     // steps in a row without a new best residual that stop the loop
 };
 
-// 9 resident blocks per SM (56 registers). The FP32 inner sweeps are bound by
-// load latency; with rows in aligned pairs, 9 blocks measured fastest (192^3:
-// 281 us per stencil inner iteration and 331 us CSR, against 288 / 335 at 8
-// blocks and 315 / 339 at 10, where the pairs spill more).
+// Most threads per block of the mixed kernel (64 registers at 1024 threads per
+// SM). The 4-row groups spill there, and are faster than with 80 or 127
+// registers at fewer threads: 192^3, 167 us an inner iteration against 185 and
+// 217 (174 in blocks of 512).
+constexpr int kMixedTPB = 256;
 template <class Op64, class Op32>
-__global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32 A32, const MixedArgs m) {
-    __shared__ Exchange<kTPB> X;
-    __shared__ uint64_t stage_full[kStages], stage_empty[kStages];
-    extern __shared__ __align__(128) char stage_buf[];   // kStageSmemBytes when the sweeps are staged
-    constexpr bool kStaged = HasRow2<Op32>::value;
-    if (threadIdx.x == 0) {
-        X.ok = 1;   // read only after the first exchange's barrier
-        if (kStaged) {
-            for (int k = 0; k < kStages; ++k) {
-                mbar_init(&stage_full[k], 1);
-                mbar_init(&stage_empty[k], kTPB);
-            }
-            mbar_init_fence();
-        }
-    }
-    __syncthreads();
-    Stager stager{stage_buf, stage_full, stage_empty, 0u, m.ctl};
-    GridSync g{m.ctl, m.partials, 0u, 0, kTPB};
-    // row ranges start on multiples of 4 rows: the FP32 sweeps access rows in
-    // aligned pairs, and the staged ones copy 16-byte aligned tiles
-    const long long quads = (m.n + 3) / 4;
-    const int lo = (int)(4 * ((long long)blockIdx.x * quads / gridDim.x));
-    const int hi_quad = (int)(4 * ((long long)(blockIdx.x + 1) * quads / gridDim.x));
-    const int hi = hi_quad < m.n ? hi_quad : m.n;
+__global__ void __launch_bounds__(kMixedTPB, 4)
+    mixed_kernel(const Op64 A, const Op32 A32, const MixedArgs m) {
+    __shared__ Exchange<kMixedTPB> X;
+    if (threadIdx.x == 0) X.ok = 1;   // read only after the first exchange's barrier
+    GridSync g{m.ctl, m.partials, 0u, 0, (int)(gridDim.x * blockDim.x)};
+    const int lo = (int)(blockIdx.x * blockDim.x), hi = m.n;
     int outer = 0, inner_total = 0, status = PBCG_NOT_CONVERGED, spmvs = 0, stalls = 0;
     double nr0 = 0.0, tol = 0.0, bound = 0.0, last = 0.0;
     double best = 0.0;        // smallest squared FP64 residual so far (valid when have_best)
@@ -1310,7 +1136,7 @@ __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32
         ia.max_repl = -1;
         ia.variant = 0;
         Outcome io{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
-        if (!pipelined_loop<Op32, float, kTPB>(A32, ia, g, X, lo, hi, io, spmvs, nullptr, kStaged ? &stager : nullptr))
+        if (!pipelined_loop<Op32, float, kMixedTPB>(A32, ia, g, X, lo, hi, io, spmvs, nullptr))
             return;
         // the inner history holds squared norms after entry 0 (thread 0 of block 0 wrote them)
         if (blockIdx.x == 0 && threadIdx.x == 0 && ia.hist)
@@ -1327,7 +1153,7 @@ __global__ void __launch_bounds__(kTPB, 9) mixed_kernel(const Op64 A, const Op32
     }
     if (blockIdx.x == 0) {
         if (m.hist)
-            for (int i = (int)threadIdx.x; i <= outer; i += kTPB) m.hist[i] = sqrt(m.hist[i]);
+            for (int i = (int)threadIdx.x; i <= outer; i += (int)blockDim.x) m.hist[i] = sqrt(m.hist[i]);
         if (threadIdx.x == 0) {
             Control *c = m.ctl;
             c->iters = outer;
