@@ -66,6 +66,18 @@ struct SolverBlock {
     static constexpr int kThreads = Wide ? 512 : 256;
 };
 
+// lo of a grid kernel's thread. Consecutive runs of 32 rows go to the same warp
+// of consecutive blocks, so that a sweep with fewer rows (or groups of rows)
+// than threads, or a last round that is not full, still uses every SM. Against
+// blockDim.x rows in a row per block, us per iteration of Algorithm 9: 48^3
+// 22.2 -> 21.4, 96^3 74.7 -> 72.4, 256^3 CSR 1088 -> 1047, 200k random rows
+// 91.1 -> 82.1; FP32 stencil iterations of 64^3 26.0 -> 25.0, 110^3 68.0 ->
+// 58.7. The FP32 CSR sweeps lost 2 to 3 % (193x160x131 184 -> 190) and keep
+// whole blocks of rows.
+__device__ __forceinline__ int grid_lo() {
+    return (int)(((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32u + (threadIdx.x & 31u)) - (int)threadIdx.x;
+}
+
 struct Outcome {
     int iters, status, half, nrr;
     double nr0, nr;   // nr: squared norm of the last recursive residual (or of q after a half step)
@@ -743,7 +755,7 @@ __global__ void __launch_bounds__(SolverBlock<Wide>::kThreads, 1024 / SolverBloc
     __shared__ WideSlot wide[Wide ? kWideSlots * B : 1];
     if (threadIdx.x == 0) X.ok = 1;   // read only after the first exchange's barrier
     GridSync g{a.ctl, a.partials, 0u, 0, (int)(gridDim.x * blockDim.x)};   // partials: the exchange slots
-    const int lo = (int)(blockIdx.x * blockDim.x), hi = a.n;
+    const int lo = grid_lo(), hi = a.n;
     Outcome o{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
     int spmvs = 0;
     bool ok;
@@ -1008,7 +1020,7 @@ __global__ void __launch_bounds__(SolverBlock<Wide>::kThreads, 1024 / SolverBloc
     __shared__ WideSlot wide[Wide ? kWideSlots * B : 1];
     if (threadIdx.x == 0) X.ok = 1;   // read only after the first exchange's barrier
     GridSync g{a.ctl, a.partials, 0u, 0, (int)(gridDim.x * blockDim.x)};   // partials: the exchange slots
-    const int lo = (int)(blockIdx.x * blockDim.x), hi = a.n;
+    const int lo = grid_lo(), hi = a.n;
     Outcome o{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
     int spmvs = 0;
     bool ok;
@@ -1076,7 +1088,7 @@ __global__ void __launch_bounds__(kMixedTPB, 4)
     __shared__ Exchange<kMixedTPB> X;
     if (threadIdx.x == 0) X.ok = 1;   // read only after the first exchange's barrier
     GridSync g{m.ctl, m.partials, 0u, 0, (int)(gridDim.x * blockDim.x)};
-    const int lo = (int)(blockIdx.x * blockDim.x), hi = m.n;
+    const int lo = HasGroups<Op32>::value ? grid_lo() : (int)(blockIdx.x * blockDim.x), hi = m.n;
     int outer = 0, inner_total = 0, status = PBCG_NOT_CONVERGED, spmvs = 0, stalls = 0;
     double nr0 = 0.0, tol = 0.0, bound = 0.0, last = 0.0;
     double best = 0.0;        // smallest squared FP64 residual so far (valid when have_best)
