@@ -1012,7 +1012,11 @@ extern "C" pbcg_status pbicgstab_csr_transpose(int32_t n, int32_t nnz, const int
     const int blocks = 4 * sms;
     PBCG_CUDA(cudaMemsetAsync(d_trowptr, 0, (size_t)(n + 1) * sizeof(int), st));
     if (nnz > 0) pbcg::transpose_count_kernel<<<blocks, 256, 0, st>>>(nnz, d_col, d_trowptr);
-    pbcg::scan_kernel<<<1, 1024, 0, st>>>(n + 1, d_trowptr);
+    // the tile sums live in the cursors' array, which is cleared after the scan
+    const int m = n + 1, tiles = (int)(((long long)m + pbcg::kScanTile - 1) / pbcg::kScanTile);
+    pbcg::scan_tiles_kernel<<<tiles, pbcg::kScanThreads, 0, st>>>(m, d_trowptr, cursor);
+    pbcg::scan_sums_kernel<<<1, pbcg::kScanThreads, 0, st>>>(tiles, cursor);
+    pbcg::scan_apply_kernel<<<tiles, pbcg::kScanThreads, 0, st>>>(m, d_trowptr, cursor);
     PBCG_CUDA(cudaMemsetAsync(cursor, 0, (size_t)(n + 1) * sizeof(int), st));
     if (n > 0) {
         pbcg::transpose_scatter_kernel<<<blocks, 256, 0, st>>>(n, d_rowptr, d_col, d_val, d_trowptr, cursor, d_tcol,
