@@ -131,7 +131,8 @@ __device__ __forceinline__ void warp_allsum(double (&v)[K]) {
 // What the threads of a block share in an exchange. Every field after `part`
 // is the same in all blocks of a solve once an exchange has completed.
 struct alignas(16) Scalars {
-    double alpha, beta, omega, rho, r0s, r0z;   // of the iteration
+    double alpha, beta, omega, rho;   // of the iteration
+    double gain, slope;   // alpha / (rho omega) and (r0,s) - omega (r0,z): the next beta and alpha from them
     double nr;          // squared norm tested last
     double nr0, tol, bound;   // ||r_0||, the tolerance, the squared norms it can accept
     double aux;         // total of an exchange outside the iteration
@@ -149,6 +150,41 @@ struct Exchange {
     int last;
 };
 
+// Sum of the first `rows` (at most 16) rows of K values, returned to every lane of the warp:
+// warp_allsum on half-warps, the upper one holding the upper half of the values,
+// which saves the first level of additions.
+template <int K>
+__device__ __forceinline__ void sum_rows(const double (*a)[kMaxDots], int rows, double (&v)[K]) {
+    constexpr int P = K <= 1 ? 1 : K <= 2 ? 2 : K <= 4 ? 4 : 8;
+    constexpr int H = P > 1 ? P / 2 : 1;                      // values of a lane
+    constexpr int M = H == 1 ? 0 : H == 2 ? 1 : 2;            // halvings left
+    const int lane = threadIdx.x & 31, row = lane & 15, first = P > 1 && lane >= 16 ? H : 0;
+    double w[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) w[k] = row < rows && first + k < K ? a[row][first + k] : 0.0;
+#pragma unroll
+    for (int lvl = 0; lvl < M; ++lvl) {
+        const int o = 8 >> lvl, half = H >> (lvl + 1);
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < half; ++k) {
+            const double send = upper ? w[k] : w[k + half];
+            const double keep = upper ? w[k + half] : w[k];
+            w[k] = keep + __shfl_xor_sync(kFull, send, o);
+        }
+    }
+#pragma unroll
+    for (int o = 8 >> M; o > 0; o >>= 1) w[0] += __shfl_xor_sync(kFull, w[0], o);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        int src = k / H * 16;
+#pragma unroll
+        for (int b = 0; b < M; ++b)
+            if (k % H & (1 << (M - 1 - b))) src |= 8 >> b;
+        v[k] = __shfl_sync(kFull, w[0], src);
+    }
+}
+
 // Fixed-order block sums, returned to every lane of warp 0: the warps reduce
 // independently, then warp 0 adds their sums.
 template <int K, int T>
@@ -162,7 +198,7 @@ __device__ __forceinline__ void block_sum(double (&v)[K], Exchange<T> &X) {
     __syncthreads();
     if (wid == 0) {
         const int warps = (int)(blockDim.x >> 5);
-        if constexpr (T / 32 <= 8) {   // lane k adds value k of the warps in warp order
+        if constexpr (T / 32 <= 4) {   // lane k adds value k of the warps in warp order
             double t = 0.0;
             if (lane < K) {
                 t = X.part[0][lane];
@@ -172,10 +208,8 @@ __device__ __forceinline__ void block_sum(double (&v)[K], Exchange<T> &X) {
             }
 #pragma unroll
             for (int k = 0; k < K; ++k) v[k] = __shfl_sync(kFull, t, k);
-        } else {                       // lane w takes warp w: a tree is shorter than 15 additions in a row
-#pragma unroll
-            for (int k = 0; k < K; ++k) v[k] = lane < warps ? X.part[lane < warps ? lane : 0][k] : 0.0;
-            warp_allsum<K>(v);
+        } else {                       // a tree is shorter than 7 or 15 additions in a row
+            sum_rows<K>(X.part, warps, v);
         }
     }
 }
@@ -201,7 +235,7 @@ __device__ __forceinline__ void block_sum(double (&v)[K], Exchange<T> &X) {
 // reading exchange e). Results are bitwise identical in every block and do
 // not depend on arrival order. Every wait is bounded (limit_ns,
 // kSyncTimeoutNs by default) and watches the abort flag.
-constexpr int kSlotDoubles = 8;
+constexpr int kSlotDoubles = kMaxDots;
 constexpr int kLastReduceGrid = 512;
 
 struct GridSync {
@@ -415,7 +449,7 @@ struct ClusterSync {
 };
 
 __device__ __forceinline__ bool is_leader(const ClusterSync &g) { return g.rank == 0; }
-__device__ __forceinline__ int row_step(const ClusterSync &) { return kTPB; }
+__device__ __forceinline__ int row_step(const ClusterSync &) { return (int)blockDim.x; }
 
 template <int T>
 __device__ __forceinline__ bool grid_sync(ClusterSync &g, Exchange<T> &) {
@@ -435,9 +469,7 @@ __device__ __forceinline__ bool exchange(ClusterSync &g, double (&v)[K], Exchang
     }
     cluster_barrier();
     if (wid == 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = lane < (int)g.size ? g.slots[buf][lane][k] : 0.0;
-        warp_allsum<K>(v);
+        sum_rows<K>(g.slots[buf], (int)g.size, v);
         f(X.s, v);
     }
     g.epoch++;

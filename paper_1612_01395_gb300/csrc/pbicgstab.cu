@@ -70,6 +70,7 @@ struct pbicgstab_s {
     long long st_len[7][2];  // stencil: table elements the grid reaches (0: no table)
     long long nnz;           // stored entries (stencil: 7 per row), for the launch shape
     int cluster_max;         // largest resident cluster of the cluster solver (16 or 8; 0: none)
+    int onchip_max;          // and of its on-chip form at its largest shared memory
 };
 
 extern "C" {
@@ -229,78 +230,101 @@ pbcg_status launch_solver(pbicgstab_s *h, const Op &op, bool pipelined, const pb
     return PBCG_OK;
 }
 
-// Systems with up to this many stored entries (stencil: points x unknowns)
-// are solved by one thread-block cluster by default (pbcg_opts.cluster = 0).
-// Measured per iteration (100 fixed iterations, 16-CTA cluster against the
-// cooperative grid): 2-D 64^2 (20k entries) 11.3 against 12.4 us (both
-// methods faster, BiCGStab 12.4 against 15.2 us), 32^2 8.1 against 11.0 us;
-// but 3-D 16^3 (27k entries) in stencil form 13.7 against 13.1 us, and every
-// larger system slower on the cluster (its 16 SMs of FP64 throughput: 19.6
-// against 12.7 us at 8100 unknowns). The cluster's floor is the FP64 latency
-// of the reductions and the scalar updates, not the barrier.
+// Systems with up to this many stored entries (stencil: points x unknowns) are
+// solved by one thread-block cluster by default (pbcg_opts.cluster = 0), on
+// chip. Measured per iteration, 16-CTA cluster against the cooperative grid,
+// p-BiCGStab / BiCGStab, us: 2-D 32^2 7.2 / 8.2 against 13.3 / 18.6, 64^2 (20k
+// entries) 8.6 / 9.3 against 13.2 / 19.1; 3-D 16^3 (27k) 8.6 / 9.4 against 12.5
+// / 18.7. The lines cross near 9000 rows (2-D 96^2 13.0 / 12.9 against 13.2 /
+// 19.2, 3-D 22^3 13.2 / 13.1 against 12.7 / 18.8), where the 16 SMs' FP64
+// throughput decides; the bound is kept where the interface states it.
 constexpr long long kClusterMaxEntries = 24576;
 
-// Largest cluster (16, else 8) of cluster_solve_kernel<Op> that the device can
-// make resident; 0 if none.
-template <class Op, bool P>
-int cluster_capacity(int want) {
-    const void *fn = (const void *)pbcg::cluster_solve_kernel<Op, P>;
-    if (want > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
+// The launch of a cluster kernel: `size` CTAs of one cluster.
+struct ClusterLaunch {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)want;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)want);
-    cfg.blockDim = dim3(pbcg::kTPB);
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    ClusterLaunch(int size, int block, size_t bytes, cudaStream_t stream) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)size);
+        cfg.blockDim = dim3((unsigned)block);
+        cfg.dynamicSmemBytes = bytes;
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+    ClusterLaunch(const ClusterLaunch &) = delete;
+    ClusterLaunch &operator=(const ClusterLaunch &) = delete;
+};
+
+// Whether a cluster of `size` CTAs of kernel fn can be resident; allows fn the
+// cluster size and the shared memory.
+bool cluster_fits(const void *fn, int size, int block, size_t bytes) {
+    ClusterLaunch l(size, block, bytes, nullptr);
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess) {
+    if ((size > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+        (bytes > 0 &&
+         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) ||
+        cudaOccupancyMaxActiveClusters(&clusters, fn, &l.cfg) != cudaSuccess) {
         cudaGetLastError();
-        return 0;
+        return false;
     }
-    return clusters >= 1 ? want : 0;
+    return clusters >= 1;
+}
+
+// Largest clusters (16, else 8, else none) of the two cluster solvers.
+template <class Op>
+void cluster_limits(pbicgstab_s *h) {
+    h->cluster_max = h->onchip_max = 0;
+    for (int size = 16; size >= 8; size /= 2) {
+        if (!h->cluster_max && cluster_fits((const void *)pbcg::cluster_solve_kernel<Op, true>, size, pbcg::kTPB, 0) &&
+            cluster_fits((const void *)pbcg::cluster_solve_kernel<Op, false>, size, pbcg::kTPB, 0))
+            h->cluster_max = size;
+        if (!h->onchip_max &&
+            cluster_fits((const void *)pbcg::onchip_solve_kernel<Op, true>, size, pbcg::kOnChipTPB, pbcg::kOnChipMaxBytes) &&
+            cluster_fits((const void *)pbcg::onchip_solve_kernel<Op, false>, size, pbcg::kOnChipTPB, pbcg::kOnChipMaxBytes))
+            h->onchip_max = size;
+    }
+}
+
+// Entries that the CTA of an on-chip solve has room for: all of a stencil's, and
+// of a CSR matrix up to twice the average (a CTA with more reads its own from
+// global memory).
+int onchip_cap(const pbicgstab_s *h, int size, int m) {
+    if (h->kind == 1) return (h->st.nz == 1 ? 5 : 7) * m;
+    const long long twice = 2 * ((h->nnz + size - 1) / size) + 64;
+    return (int)(twice < h->nnz ? twice : h->nnz);
 }
 
 template <class Op>
-int cluster_max_for() {
-    int c = cluster_capacity<Op, true>(16);
-    if (c && !cluster_capacity<Op, false>(16)) c = 0;
-    if (!c) c = cluster_capacity<Op, true>(8) && cluster_capacity<Op, false>(8) ? 8 : 0;
-    return c;
-}
-
-template <class Op>
-pbcg_status launch_cluster(pbicgstab_s *h, const Op &op, bool pipelined, const pbcg::SolveArgs &args, int size) {
-    if (size > 8) {
+pbcg_status launch_cluster(pbicgstab_s *h, const Op &op, bool pipelined, const pbcg::SolveArgs &args, int size,
+                           bool any_variant, int *block) {
+    const int m = (h->n + size - 1) / size, cap = onchip_cap(h, size, m);
+    const size_t bytes = pbcg::onchip_bytes(m, cap);
+    if (size <= h->onchip_max && bytes <= pbcg::kOnChipMaxBytes) {
+        *block = m >= pbcg::kOnChipTPB ? pbcg::kOnChipTPB : (m + 31) / 32 * 32;
+        pbcg::FastDiv dm;
+        dm.init((uint32_t)m);
+        // a barrier of the cluster costs less than variant 3's recomputed neighbours: 17x15x13, 9.1 us an
+        // iteration of BiCGStab against 9.9
+        pbcg::SolveArgs a = args;
+        if (any_variant) a.variant = 5;
+        ClusterLaunch l(size, *block, bytes, h->stream);
         if (pipelined)
-            PBCG_CUDA(cudaFuncSetAttribute((const void *)pbcg::cluster_solve_kernel<Op, true>,
-                                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::onchip_solve_kernel<Op, true>, op, a, m, dm, cap));
         else
-            PBCG_CUDA(cudaFuncSetAttribute((const void *)pbcg::cluster_solve_kernel<Op, false>,
-                                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::onchip_solve_kernel<Op, false>, op, a, m, dm, cap));
+        return PBCG_OK;
     }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)size;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)size);
-    cfg.blockDim = dim3(pbcg::kTPB);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = h->stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    *block = pbcg::kTPB;
+    ClusterLaunch l(size, *block, 0, h->stream);
     if (pipelined)
-        PBCG_CUDA(cudaLaunchKernelEx(&cfg, pbcg::cluster_solve_kernel<Op, true>, op, args));
+        PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::cluster_solve_kernel<Op, true>, op, args));
     else
-        PBCG_CUDA(cudaLaunchKernelEx(&cfg, pbcg::cluster_solve_kernel<Op, false>, op, args));
+        PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::cluster_solve_kernel<Op, false>, op, args));
     return PBCG_OK;
 }
 
@@ -360,16 +384,16 @@ pbcg_status run_solve(pbicgstab_s *h, bool pipelined, const double *d_b, double 
     } else if (o.cluster > 0 && o.grid == 0) {
         return fail(PBCG_ERR_ARG, "cluster solves need an unpreconditioned handle on a device with clusters");
     }
-    const Shape shape = csize ? Shape{false, csize, pbcg::kTPB}
+    Shape shape = csize ? Shape{false, csize, pbcg::kTPB}
                               : pick_shape(h, h->occ[pipelined], pipelined || h->prec || a.variant == 5, o.grid);
     PBCG_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(pbcg::Control), h->stream));
     if (h->ev0) PBCG_CUDA(cudaEventRecord(h->ev0, h->stream));
     if (h->n > 0) {
         pbcg_status st;
         if (csize)
-            st = h->kind == 1 ? launch_cluster(h, h->st, pipelined, a, csize)
-                 : h->csr_chunked ? launch_cluster(h, chunked(h->csr), pipelined, a, csize)
-                                  : launch_cluster(h, h->csr, pipelined, a, csize);
+            st = h->kind == 1 ? launch_cluster(h, h->st, pipelined, a, csize, o.plain_variant == 0, &shape.block)
+                 : h->csr_chunked ? launch_cluster(h, chunked(h->csr), pipelined, a, csize, o.plain_variant == 0, &shape.block)
+                                  : launch_cluster(h, h->csr, pipelined, a, csize, o.plain_variant == 0, &shape.block);
         else
             st = h->kind == 1 ? launch_solver(h, h->st, pipelined, a, shape)
                  : h->csr_chunked ? launch_solver(h, chunked(h->csr), pipelined, a, shape)
@@ -450,10 +474,10 @@ pbcg_status pbicgstab_create_csr(int32_t n, int32_t nnz, const int32_t *d_rowptr
         h->csr_chunked = (long long)nnz > pbcg::kChunkedMinAvgRow * (long long)n;
         if (h->csr_chunked) {
             st = occupancy<pbcg::CsrOpChunked>(h);
-            h->cluster_max = cluster_max_for<pbcg::CsrOpChunked>();
+            cluster_limits<pbcg::CsrOpChunked>(h);
         } else {
             st = occupancy<pbcg::CsrOpScalar>(h);
-            h->cluster_max = cluster_max_for<pbcg::CsrOpScalar>();
+            cluster_limits<pbcg::CsrOpScalar>(h);
         }
     }
     if (st == PBCG_OK) st = check_csr(h, n, nnz, d_rowptr, d_col);
@@ -524,7 +548,7 @@ pbcg_status pbicgstab_create_stencil(const pbcg_stencil *desc, pbcg_prec prec, v
             h->st_len[d][1] = c.data2 ? max_index(c.stride2, nx, ny, nz) + 1 : 0;
         }
         st = occupancy<pbcg::StencilOp>(h);
-        h->cluster_max = cluster_max_for<pbcg::StencilOp>();
+        cluster_limits<pbcg::StencilOp>(h);
     }
     if (st == PBCG_OK && prec == PBCG_PREC_JACOBI)
         st = setup_jacobi(h, [&](int blocks, int *flag) {
@@ -1107,7 +1131,8 @@ extern "C" pbcg_status pbicgstab_solve_csr_noalloc(int32_t n, int32_t nnz, const
         h.nnz = nnz;
         h.csr_chunked = (long long)nnz > pbcg::kChunkedMinAvgRow * (long long)n;
         st = h.csr_chunked ? occupancy<pbcg::CsrOpChunked>(&h) : occupancy<pbcg::CsrOpScalar>(&h);
-        h.cluster_max = h.csr_chunked ? cluster_max_for<pbcg::CsrOpChunked>() : cluster_max_for<pbcg::CsrOpScalar>();
+        if (h.csr_chunked) cluster_limits<pbcg::CsrOpChunked>(&h);
+        else cluster_limits<pbcg::CsrOpScalar>(&h);
     }
     if (st == PBCG_OK) st = check_csr(&h, n, nnz, d_rowptr, d_col);
     if (st != PBCG_OK) return st;

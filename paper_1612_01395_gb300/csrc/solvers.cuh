@@ -89,6 +89,10 @@ struct Outcome {
 // FP64 pipe, about 140 to its result): finite and zero from the bits, and the
 // order of non-negative numbers as the order of their bits.
 __device__ __forceinline__ bool is_finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool is_normal(double v) {
+    const int e = __double2hiint(v) & 0x7ff00000;
+    return e != 0 && e != 0x7ff00000;
+}
 __device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
 template <int K>
 __device__ __forceinline__ bool all_finite(const double (&v)[K]) {
@@ -138,7 +142,11 @@ __device__ __forceinline__ void alpha_scalars(Scalars &S, double d) {
     if (is_zero(d)) return stop_scalars(S, PBCG_BREAKDOWN);
     S.alpha = __ddiv_rn(S.rho, d);
 }
-// omega = (q,y) / (y,y), or the half step x + alpha p when ||q|| meets the tolerance
+// omega = (q,y) / (y,y), or the half step x + alpha p when ||q|| meets the
+// tolerance. Lanes 1 and 2 divide for the next beta in the same instructions:
+// gain = (alpha / rho) (1 / omega), so that beta = gain rho' waits for no
+// division when rho' arrives (64^2 on one cluster 9.1 -> 8.5 us an iteration,
+// with the shorter sum of the cluster's slots).
 __device__ __forceinline__ void omega_scalars(Scalars &S, double qy, double yy, double qq, bool fixed) {
     S.action = kGo;
     const bool small_q = !fixed && norm_below(qq, S.tol, S.bound);
@@ -148,28 +156,34 @@ __device__ __forceinline__ void omega_scalars(Scalars &S, double qy, double yy, 
         S.action = kHalf;
         return;
     }
-    S.omega = __ddiv_rn(qy, yy);
-    if (is_zero(S.omega)) stop_scalars(S, PBCG_BREAKDOWN);
+    const int lane = threadIdx.x & 31;
+    const double f = __ddiv_rn(lane == 0 ? qy : lane == 1 ? yy : S.alpha, lane == 0 ? yy : lane == 1 ? qy : S.rho);
+    S.omega = __shfl_sync(kFull, f, 0);
+    if (is_zero(S.omega)) return stop_scalars(S, PBCG_BREAKDOWN);
+    S.gain = __dmul_rn(__shfl_sync(kFull, f, 2), __shfl_sync(kFull, f, 1));
 }
-// Test of r_{i+1}; beta = (alpha / omega) (rho' / rho): the two divisions are
-// one, by even and odd lanes.
+// Test of r_{i+1}; beta = (alpha / omega) (rho' / rho), by the gain where that
+// stayed in range, else by its two quotients on even and odd lanes.
 __device__ __forceinline__ void beta_scalars(Scalars &S, double rho_n, double rr, bool finite, bool fixed) {
     S.action = kGo;
     S.nr = rr;
     if (!finite) return stop_scalars(S, PBCG_NONFINITE);
     if (!fixed && norm_below(rr, S.tol, S.bound)) return stop_scalars(S, PBCG_OK);
     if (is_zero(rho_n)) return stop_scalars(S, PBCG_BREAKDOWN);
-    const bool odd = threadIdx.x & 1;
-    const double f = __ddiv_rn(odd ? rho_n : S.alpha, odd ? S.rho : S.omega);
-    S.beta = __dmul_rn(__shfl_sync(kFull, f, 0), __shfl_sync(kFull, f, 1));
+    if (is_normal(S.gain)) {
+        S.beta = __dmul_rn(S.gain, rho_n);
+    } else {
+        const bool odd = threadIdx.x & 1;
+        const double f = __ddiv_rn(odd ? rho_n : S.alpha, odd ? S.rho : S.omega);
+        S.beta = __dmul_rn(__shfl_sync(kFull, f, 0), __shfl_sync(kFull, f, 1));
+    }
 }
 // Algorithm 9: the test and beta, then the denominator of eq. (3),
-// r0w + beta r0s - beta omega r0z, and alpha_{i+1} = rho' / denominator
+// r0w + beta (r0s - omega r0z), and alpha_{i+1} = rho' / denominator
 __device__ __forceinline__ void beta_alpha_scalars(Scalars &S, double rho_n, double r0w, double rr, bool fixed) {
     beta_scalars(S, rho_n, rr, is_finite(rho_n) && is_finite(r0w) && is_finite(rr), fixed);
     if (S.action != kGo) return;
-    const double d = __dsub_rn(__dadd_rn(r0w, __dmul_rn(S.beta, S.r0s)),
-                               __dmul_rn(__dmul_rn(S.beta, S.omega), S.r0z));
+    const double d = fma(S.beta, S.slope, r0w);
     if (is_zero(d)) return stop_scalars(S, PBCG_BREAKDOWN);
     S.alpha = __ddiv_rn(rho_n, d);
     S.rho = rho_n;
@@ -482,10 +496,9 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
         double d1[5];
         a1.values(d1);
         if (!exchange(g, d1, X, [&](Scalars &S, const double (&t)[5]) {
-                S.r0s = t[3];
-                S.r0z = t[4];
                 if (!all_finite(t)) return stop_scalars(S, PBCG_NONFINITE);
                 omega_scalars(S, t[0], t[1], t[2], fixed);
+                if (S.action == kGo) S.slope = fma(-S.omega, t[4], t[3]);
             }))
             return false;
         if (X.s.action == kStop) { o.status = X.s.status; break; }
@@ -675,10 +688,9 @@ __device__ __forceinline__ bool pipelined_prec_loop(const Op &A, const SolveArgs
         double d1[5];
         a1.values(d1);
         if (!exchange(g, d1, X, [&](Scalars &S, const double (&t)[5]) {
-                S.r0s = t[3];
-                S.r0z = t[4];
                 if (!all_finite(t)) return stop_scalars(S, PBCG_NONFINITE);
                 omega_scalars(S, t[0], t[1], t[2], fixed);
+                if (S.action == kGo) S.slope = fma(-S.omega, t[4], t[3]);
             }))
             return false;
         if (X.s.action == kStop) { o.status = X.s.status; break; }
@@ -1208,6 +1220,164 @@ __global__ void __launch_bounds__(kTPB, 1) cluster_solve_kernel(const Op A, cons
     else
         standard_loop<Op, kTPB, ClusterSync>(A, a, g, X, lo, hi, o, spmvs, nullptr);
     finish(A, a, g, X, lo, hi, o, spmvs);
+    cluster_barrier();   // no CTA leaves while another may still address its shared memory
+}
+
+// ===========================================================================
+// The same with everything on the chip: CTA `rank` owns rows [rank m, rank m +
+// m) and keeps their vectors and their matrix entries in its shared memory. An
+// entry holds its value and the shared-memory address, in the window of the
+// CTA that owns its column, of that column's slot in the first vector; the
+// slot in another vector is a constant away. So a product with A reads
+// neighbours' values through distributed shared memory, and an iteration
+// touches neither L1 nor L2, whose round trips (row pointers, then entries,
+// then vector elements) took a quarter of it: 64^2 11.6 -> 9.1 us an iteration
+// of Algorithm 9, 17x15x13 14.1 -> 9.5 of Algorithm 7; what is left is the
+// FP64 latency of the sums and scalars. The loops are the same code: their
+// vectors are addressed as before, by generic pointers offset to the CTA's
+// first row.
+// ===========================================================================
+constexpr int kOnChipTPB = 256;
+constexpr int kOnChipVecs = 11;            // r r0 p s z q y w t v x
+constexpr size_t kOnChipMaxBytes = 200 * 1024;
+__host__ __device__ inline size_t onchip_bytes(int m, int cap) {
+    return (size_t)m * (kOnChipVecs * sizeof(double) + sizeof(int2)) + (size_t)cap * (sizeof(double) + sizeof(uint32_t));
+}
+
+struct OnChipOp {
+    int n, lo, m;
+    FastDiv dm;                // by m: the owner of a column
+    uint32_t pool;             // shared address of the first vector
+    const int2 *range;         // entries of each own row
+    const double *val;
+    const uint32_t *addr;      // null: the entries did not fit, taken from col and val in global memory
+    const int *col;
+
+    __device__ __forceinline__ uint32_t address(int c) const {
+        const uint32_t owner = dm.div((uint32_t)c);
+        uint32_t a;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(pool), "r"(owner));
+        return a + (uint32_t)(c - (int)owner * m) * 8u;
+    }
+    // Distance of vector p (as the loops address it) from the first one.
+    __device__ __forceinline__ uint32_t apart(const double *p) const {
+        return (uint32_t)__cvta_generic_to_shared(p + lo) - pool;
+    }
+    __device__ __forceinline__ static double peek(uint32_t a) {
+        double v;
+        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+        return v;
+    }
+    __device__ __forceinline__ double value(const VecLoad &u, uint32_t a) const { return peek(a + apart(u.x)); }
+    __device__ __forceinline__ double value(const PLoad &u, uint32_t a) const {
+        return fma(u.beta, fma(-u.omega, peek(a + apart(u.s)), peek(a + apart(u.p))), peek(a + apart(u.r)));
+    }
+    __device__ __forceinline__ double value(const QLoad &u, uint32_t a) const {
+        return fma(-u.alpha, peek(a + apart(u.s)), peek(a + apart(u.r)));
+    }
+
+    template <class L>
+    __device__ __forceinline__ double row(int i, const L &u) const {
+        constexpr int kC = 8;
+        const int2 q = range[i - lo];
+        double acc = 0.0;
+        for (int k0 = q.x; k0 < q.y; k0 += kC) {
+            double v[kC], x[kC];
+#pragma unroll
+            for (int j = 0; j < kC; ++j) {
+                v[j] = x[j] = 0.0;
+                if (k0 + j < q.y) {
+                    v[j] = val[k0 + j];
+                    x[j] = value(u, addr ? addr[k0 + j] : address(PBCG_SAFE(col[k0 + j], n)));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kC; ++j) {
+                if (k0 + j >= q.y) break;
+                acc = fma(v[j], x[j], acc);
+            }
+        }
+        return acc;
+    }
+};
+
+// The CTA's entries into shared memory.
+template <int kChunk>
+__device__ __forceinline__ void onchip_entries(const CsrOpT<double, kChunk> &A, OnChipOp &op, int hi, int cap, int2 *range,
+                                               double *val, uint32_t *addr) {
+    const int base = hi > op.lo ? A.rowptr[op.lo] : 0, count = hi > op.lo ? A.rowptr[hi] - base : 0;
+    const bool fits = count <= cap;
+    for (int i = op.lo + (int)threadIdx.x; i < hi; i += (int)blockDim.x) {
+        const int b = A.rowptr[i], e = A.rowptr[i + 1];
+        range[i - op.lo] = fits ? make_int2(b - base, e - base) : make_int2(b, e);
+    }
+    if (fits)
+        for (int k = (int)threadIdx.x; k < count; k += (int)blockDim.x) {
+            val[k] = A.val[base + k];
+            addr[k] = op.address(PBCG_SAFE(A.col[base + k], op.n));
+        }
+    op.val = fits ? val : A.val;
+    op.addr = fits ? addr : nullptr;
+    op.col = A.col;
+}
+__device__ __forceinline__ void onchip_entries(const StencilOp &A, OnChipOp &op, int hi, int, int2 *range, double *val,
+                                               uint32_t *addr) {
+    const int per = A.nz == 1 ? 5 : 7;   // the host gives per * m entries
+    for (int r = op.lo + (int)threadIdx.x; r < hi; r += (int)blockDim.x) {
+        const int t = (int)A.dx.div((uint32_t)r), i = r - t * A.nx, k = (int)A.dy.div((uint32_t)t), j = t - k * A.ny;
+        int at = per * (r - op.lo);
+        const int first = at;
+        auto put = [&](bool in, int d, int off) {
+            if (!in) return;
+            val[at] = A.coef(d, i, j, k);
+            addr[at] = op.address(r + off);
+            ++at;
+        };
+        put(k > 0, PBCG_B, -A.nxy);
+        put(j > 0, PBCG_S, -A.nx);
+        put(i > 0, PBCG_W, -1);
+        put(true, PBCG_C, 0);
+        put(i < A.nx - 1, PBCG_E, 1);
+        put(j < A.ny - 1, PBCG_N, A.nx);
+        put(k < A.nz - 1, PBCG_T, A.nxy);
+        range[r - op.lo] = make_int2(first, at);
+    }
+    op.val = val;
+    op.addr = addr;
+    op.col = nullptr;
+}
+
+template <class Op, bool Pipelined>
+__global__ void __launch_bounds__(kOnChipTPB, 1) onchip_solve_kernel(const Op A, const SolveArgs a, int m, FastDiv dm,
+                                                                     int cap) {
+    extern __shared__ __align__(16) double onchip[];
+    __shared__ Exchange<kOnChipTPB> X;
+    __shared__ double slots[2][kMaxCluster][kSlotDoubles];   // cluster reductions: every CTA's block sums
+    const unsigned size = cluster_ctas(), rank = cluster_rank();
+    if (threadIdx.x == 0) X.ok = 1;
+    ClusterSync g{slots, rank, size, 0u, 0};
+    const int lo = (int)rank * m < a.n ? (int)rank * m : a.n;
+    const int hi = lo + m < a.n ? lo + m : a.n;
+    // vectors (by rows of the system), then the entries' values, the rows' ranges, the entries' addresses
+    double *val = onchip + (size_t)kOnChipVecs * m;
+    int2 *range = reinterpret_cast<int2 *>(val + cap);
+    uint32_t *addr = reinterpret_cast<uint32_t *>(range + m);
+    OnChipOp op{a.n, lo, m, dm, (uint32_t)__cvta_generic_to_shared(onchip), range, nullptr, nullptr, nullptr};
+    onchip_entries(A, op, hi, cap, range, val, addr);
+    SolveArgs s = a;
+    double **vecs[kOnChipVecs] = {&s.V.r, &s.V.r0, &s.V.p, &s.V.s, &s.V.z, &s.V.q, &s.V.y, &s.V.w, &s.V.t, &s.V.v, &s.x};
+#pragma unroll
+    for (int k = 0; k < kOnChipVecs; ++k) *vecs[k] = onchip + (size_t)k * m - lo;
+    PBCG_ROWS(i) { s.x[i] = a.x[i]; }
+    cluster_barrier();   // every CTA started, and its x is in place
+    Outcome o{0, PBCG_NOT_CONVERGED, 0, 0, 0.0, 0.0};
+    int spmvs = 0;
+    if constexpr (Pipelined)
+        pipelined_loop<OnChipOp, double, kOnChipTPB, ClusterSync>(op, s, g, X, lo, hi, o, spmvs, nullptr);
+    else
+        standard_loop<OnChipOp, kOnChipTPB, ClusterSync>(op, s, g, X, lo, hi, o, spmvs, nullptr);
+    finish(op, s, g, X, lo, hi, o, spmvs);
+    PBCG_ROWS(i) { a.x[i] = s.x[i]; }
     cluster_barrier();   // no CTA leaves while another may still address its shared memory
 }
 

@@ -1,0 +1,150 @@
+"""The dispatch lines of the solvers (needs a GB300): the on-chip cluster, the
+wide kernel above 700k rows, the FP32 groups of rows, and what their sums do
+with zeros and non-finite values. Bars as in the parity tests: residual norms
+within 1e-8 relative and x within 1e-9 of the FP64 oracle over the first
+iterations; the transposes are compared exactly."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1612_01395_gb300 import native
+from paper_1612_01395_gb300 import problems as P
+
+pytestmark = pytest.mark.gpu
+K = 10
+
+
+def dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def grid_stencil(nx, ny, nz):
+    """Upwind convection-diffusion on any nx x ny x nz grid."""
+    c = [P.Coef(value=0.0) for _ in range(7)]
+    c[P.C] = P.Coef(table=6.3 + 0.01 * np.arange(ny), stride=(0, 1, 0), table2=0.02 * np.arange(nx), stride2=(1, 0, 0))
+    c[P.W], c[P.E] = P.Coef(value=-1.1), P.Coef(value=-0.9)
+    c[P.S] = P.Coef(table=-1.0 - 0.001 * np.arange(nx), stride=(1, 0, 0))
+    c[P.N] = P.Coef(value=-1.0)
+    if nz > 1:
+        c[P.B], c[P.T] = P.Coef(value=-1.05), P.Coef(value=-0.95)
+    return P.Stencil(nx=nx, ny=ny, nz=nz, coefs=c)
+
+
+def check(solver, A, b, method):
+    ref = (oracle.pbicgstab if method == "pipelined" else oracle.bicgstab)(A, b, rtol=0.0, maxit=K, fixed_iters=K)
+    x, info, hist = solver.solve(dev(b), rtol=0.0, maxit=K, fixed_iters=K, method=method, history=True)
+    h = hist.cpu().numpy()
+    assert np.max(np.abs(h - ref.hist[:K + 1]) / ref.hist[:K + 1]) <= 1e-8
+    assert np.linalg.norm(x.cpu().numpy() - ref.x) <= 1e-9 * np.linalg.norm(ref.x)
+    x2, _ = solver.solve(dev(b), rtol=0.0, maxit=K, fixed_iters=K, method=method)
+    np.testing.assert_array_equal(x.cpu().numpy(), x2.cpu().numpy())
+    return info
+
+
+@pytest.mark.parametrize("method", ["pipelined", "standard"])
+@pytest.mark.parametrize("form", ["csr", "stencil"])
+@pytest.mark.parametrize("dims", [(7, 1, 1), (33, 1, 1), (5, 7, 3), (31, 33, 1), (64, 64, 1), (69, 71, 1), (15, 15, 15)])
+def test_small_systems_on_chip(dims, form, method):
+    """One row a CTA and less, ragged last CTAs, one and several rows a thread."""
+    st = grid_stencil(*dims)
+    A = P.stencil_to_csr(st)
+    s = native.Solver.from_csr(A) if form == "csr" else native.Solver.from_stencil(st)
+    b = oracle.spmv(A, P.splitmix64_uniform(7, A.n))
+    if A.n > 100:
+        assert check(s, A, b, method)["cluster"] > 0
+    x, info = s.solve(dev(b), rtol=1e-12, maxit=400, method=method)
+    assert info["status"] == native.PBCG_OK and info["cluster"] > 0
+    assert np.linalg.norm(b - oracle.spmv(A, x.cpu().numpy())) <= 1e-11 * np.linalg.norm(b)
+    s.close()
+
+
+def test_on_chip_entries_that_do_not_fit_their_cta():
+    """The first rows hold most of the entries: their CTA reads them from global memory."""
+    n = 640
+    a = np.eye(n) * 40.0
+    a[:20] += np.where(np.arange(n) % 2 == 0, 0.01, -0.013)
+    a[np.arange(1, n), np.arange(n - 1)] += -1.0
+    A = P.dense_to_csr(a)
+    assert A.nnz <= 24576
+    s = native.Solver.from_csr(A)
+    for method in ("pipelined", "standard"):
+        x, info = s.solve(dev(A.to_dense() @ np.linspace(-1, 1, n)), rtol=1e-12, maxit=200, method=method)
+        assert info["cluster"] > 0 and info["status"] == native.PBCG_OK
+        assert np.max(np.abs(x.cpu().numpy() - np.linspace(-1, 1, n))) <= 1e-10
+    s.close()
+
+
+@pytest.mark.parametrize("method", ["pipelined", "standard"])
+@pytest.mark.parametrize("form", ["csr", "stencil"])
+@pytest.mark.parametrize("dims", [(100, 100, 70), (83, 89, 95), (839, 837, 1)])
+def test_wide_sums_above_their_line(dims, form, method):
+    """700 000 rows (the last below the line), 701 765 and 702 243 ragged ones; the
+    solution is zero on half of the grid, so products vanish and sums cancel."""
+    st = grid_stencil(*dims)
+    A = P.stencil_to_csr(st)
+    x = P.splitmix64_uniform(3, A.n)
+    x[: A.n // 2] = 0.0
+    s = native.Solver.from_csr(A) if form == "csr" else native.Solver.from_stencil(st)
+    info = check(s, A, oracle.spmv(A, x), method)
+    assert info["block"] == (512 if A.n > 700000 else 256)
+    s.close()
+
+
+def test_wide_sums_report_non_finite_values():
+    st = grid_stencil(100, 100, 71)
+    s = native.Solver.from_stencil(st)
+    b = P.splitmix64_uniform(1, st.n)
+    for bad in (np.nan, np.inf):
+        b[12345] = bad
+        for method in ("pipelined", "standard"):
+            _, info = s.solve(dev(b), rtol=1e-8, maxit=20, method=method)
+            assert info["status"] == native.PBCG_NONFINITE
+    b[:] = 0.0
+    x, info = s.solve(dev(b), rtol=1e-8, maxit=20)
+    assert info["status"] == native.PBCG_OK and info["iters"] == 0 and not x.any()
+    s.close()
+
+
+@pytest.mark.parametrize("dims", [(8, 9, 1), (6, 5, 4), (7, 3, 5), (4, 4, 4), (1, 9, 3), (2, 2, 2), (64, 3, 2), (65, 5, 3),
+                                  (66, 4, 5), (67, 3, 4)])
+def test_fp32_groups_of_rows(dims):
+    """x-lines of every length modulo 4, lines shorter than a group among them:
+    the refinement reaches 1e-12 and repeats bit for bit."""
+    st = grid_stencil(*dims)
+    A = P.stencil_to_csr(st)
+    b = oracle.spmv(A, P.splitmix64_uniform(2, A.n))
+    s = native.Solver.from_stencil(st)
+    x, info = s.solve_mixed(dev(b), None, rtol=1e-12, inner_rtol=1e-3)
+    x2, _ = s.solve_mixed(dev(b), None, rtol=1e-12, inner_rtol=1e-3)
+    assert info["status"] == native.PBCG_OK
+    assert np.linalg.norm(b - oracle.spmv(A, x.cpu().numpy())) <= 1e-11 * np.linalg.norm(b)
+    np.testing.assert_array_equal(x.cpu().numpy(), x2.cpu().numpy())
+    s.close()
+
+
+@pytest.mark.parametrize("n", [0, 1, 4094, 4095, 4096, 12289])
+def test_transpose_row_pointers_at_the_tiles_of_the_scan(n):
+    import torch
+    rng = np.random.default_rng(n)
+    counts = rng.integers(0, 4, n) if n else np.zeros(0, dtype=int)
+    rp = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    nnz = int(rp[-1])
+    col = rng.integers(0, max(n, 1), nnz).astype(np.int32)
+    val = rng.standard_normal(nnz)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()   # noqa: E731
+    drp, dcol, dval = t(rp), t(col if nnz else np.zeros(1, np.int32)), t(val if nnz else np.zeros(1))
+    trp = torch.empty(n + 1, dtype=torch.int32, device="cuda")
+    tcol, tval = torch.empty_like(dcol), torch.empty_like(dval)
+    wb = native.pbicgstab_transpose_work_bytes(n)
+    work = torch.empty(wb // 4 + 64, dtype=torch.int32, device="cuda")
+    rc = native.pbicgstab_csr_transpose(n, nnz, drp.data_ptr(), dcol.data_ptr(), dval.data_ptr(), trp.data_ptr(),
+                                        tcol.data_ptr(), tval.data_ptr(), work.data_ptr(), wb,
+                                        torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert rc == native.PBCG_OK
+    expect = np.concatenate([[0], np.cumsum(np.bincount(col, minlength=n))]) if n else np.zeros(1)
+    np.testing.assert_array_equal(trp.cpu().numpy(), expect)
+    rows = np.repeat(np.arange(n), counts)
+    order = np.lexsort((rows, col))
+    np.testing.assert_array_equal(tcol.cpu().numpy()[:nnz], rows[order])
