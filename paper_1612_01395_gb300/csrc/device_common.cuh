@@ -77,6 +77,17 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+// Add 1: every store of the block ordered before this thread's by a barrier is
+// ordered before the addition (release); the second form also returns the old
+// value and orders later loads after it (acquire).
+__device__ __forceinline__ void red_release_inc(unsigned *p) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ unsigned atom_acq_rel_inc(unsigned *p) {
+    unsigned v;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ int ld_relaxed_s32(const int *p) {
     int v;
     asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -216,10 +227,10 @@ __device__ __forceinline__ void block_sum(double (&v)[K], Exchange<T> &X) {
 
 // Grid-wide exchange of a cooperative launch. Each block owns one 64-byte
 // slot (8 doubles) in each of 3 rotating buffers; exchange number e uses
-// buffer e % 3. Thread 0 of a block stores its K block sums in its slot,
-// fences (gpu scope: every store of the phase, made visible to thread 0 by
-// __syncthreads, is ordered before the arrival) and adds 1 to the arrival
-// counter. Then, by grid size:
+// buffer e % 3. Thread 0 of a block stores its K block sums in its slot and adds
+// 1 to the arrival counter with release at gpu scope (every store of the phase,
+// made visible to thread 0 by __syncthreads, is ordered before the arrival;
+// the waits are acquire loads). Then, by grid size:
 //  * small grids: thread 0 spins on the counter until all blocks of exchange
 //    e arrived, every block adds all slots in the same fixed order, and its
 //    warp 0 forms the scalars;
@@ -266,7 +277,8 @@ __device__ __forceinline__ bool is_leader(const GridSync &) { return blockIdx.x 
 // Thread 0: spin until *word >= target, bounded; false on abort or timeout.
 __device__ __forceinline__ bool wait_at_least(GridSync &g, const unsigned *word, unsigned target) {
     const uint64_t t0 = globaltimer_ns();
-    while (ld_acquire_u32(word) < target) {
+    for (unsigned spin = 1; ld_acquire_u32(word) < target; ++spin) {
+        if (spin % 8 != 0) continue;   // the flag and the clock now and then: each poll is a round trip to L2
         if (ld_relaxed_s32(&g.ctl->abort) != 0) return false;
         if (globaltimer_ns() - t0 > g.limit_ns) {
             atomicCAS(&g.ctl->abort, 0, (int)PBCG_ERR_TIMEOUT);
@@ -281,10 +293,8 @@ template <int T>
 __device__ __forceinline__ bool grid_sync(GridSync &g, Exchange<T> &X) {
     __syncthreads();   // every thread's stores of this phase precede thread 0's fence
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&g.ctl->arrivals, 1u);
+        red_release_inc(&g.ctl->arrivals);
         if (!wait_at_least(g, &g.ctl->arrivals, (g.epoch + 1u) * gridDim.x)) X.ok = 0;
-        __threadfence();
     }
     __syncthreads();
     g.epoch++;
@@ -292,17 +302,29 @@ __device__ __forceinline__ bool grid_sync(GridSync &g, Exchange<T> &X) {
     return X.ok != 0;
 }
 
-// Fixed-order sum over all slots of buffer buf, returned to every lane of warp 0.
+// Fixed-order sum over all slots of buffer buf, returned to every lane of warp
+// 0. Warps without a slot add nothing: their additions would queue on the FP64
+// pipes with the others'.
 template <int K, int T>
 __device__ __forceinline__ void sum_slots(const GridSync &g, unsigned buf, double (&v)[K], Exchange<T> &X) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int grid = (int)gridDim.x, warps = (int)(blockDim.x >> 5);
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += (int)blockDim.x) {
-        const double *src = slot_ptr(g, buf, b);
+    if (wid * 32 < grid) {
+        for (int b = threadIdx.x; b < grid; b += (int)blockDim.x) {
+            const double *src = slot_ptr(g, buf, b);
 #pragma unroll
-        for (int k = 0; k < K; ++k) v[k] += __ldcg(src + k);
+            for (int k = 0; k < K; ++k) v[k] += __ldcg(src + k);
+        }
+        warp_allsum<K>(v);
+        if (lane == 0) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) X.part[wid][k] = v[k];
+        }
     }
-    block_sum(v, X);
+    __syncthreads();
+    if (wid == 0) sum_rows<K>(X.part, (grid + 31) / 32 < warps ? (grid + 31) / 32 : warps, v);
 }
 
 // Barrier that adds the K values v of all threads of the grid in a fixed order
@@ -321,13 +343,12 @@ __device__ __forceinline__ bool exchange(GridSync &g, double (&v)[K], Exchange<T
         double *out = slot_ptr(g, buf, blockIdx.x);
 #pragma unroll
         for (int k = 0; k < K; ++k) out[k] = v[k];
-        __threadfence();
-        const unsigned before = atomicAdd(&g.ctl->arrivals, 1u);
-        X.last = before == target - 1u;
-        if (!by_last) {
+        if (by_last) {
+            X.last = atom_acq_rel_inc(&g.ctl->arrivals) == target - 1u;
+        } else {
+            red_release_inc(&g.ctl->arrivals);
             if (!wait_at_least(g, &g.ctl->arrivals, target)) X.ok = 0;
         }
-        __threadfence();
     }
     __syncthreads();
     if (!by_last) {
@@ -342,14 +363,12 @@ __device__ __forceinline__ bool exchange(GridSync &g, double (&v)[K], Exchange<T
             if (lane < kScalarWords) tot[lane] = reinterpret_cast<const double *>(&X.s)[lane];
             __syncwarp();
             if (lane == 0) {
-                __threadfence();
                 st_release_u32(&g.ctl->ready, g.epoch + 1u);
             }
         }
     } else if (wid == 0) {
         if (lane == 0) {
             if (!wait_at_least(g, &g.ctl->ready, g.epoch + 1u)) X.ok = 0;
-            __threadfence();
         }
         __syncwarp();
         const double *tot = totals_ptr(g, buf);
