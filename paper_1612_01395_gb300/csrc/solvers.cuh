@@ -83,7 +83,46 @@ struct Outcome {
     double nr0, nr;   // nr: squared norm of the last recursive residual (or of q after a half step)
 };
 
-#define PBCG_ROWS(i) for (int i = lo + (int)threadIdx.x; i < hi; i += row_step(g))
+// The steps are unsigned: the row after the last may lie above 2^31.
+#define PBCG_STEPS(i, end)                                            \
+    for (int i = lo + (int)threadIdx.x; (unsigned)i < (unsigned)(end); \
+         i = (int)((unsigned)i + (unsigned)row_step(g)))
+#define PBCG_ROWS(i) PBCG_STEPS(i, hi)
+
+// A sweep of Algorithms 7 and 10 without a product with A, two of the thread's
+// rows a step: load(i) returns a row's values, use(i, values) may store. Bound
+// by DRAM, and the compiler moves no load across a store, so one row a step
+// left too few loads in flight. An iteration of Algorithm 7 takes 825 us
+// against 931 at 256^3, 120 against 130 at 128^3, 241 against 247 on CSR at
+// 2048^2; of Algorithm 10 at 500,001 rows 191 against 201. Three and four rows
+// a step, guarded one by one, were slower (869 and 890 us at 256^3).
+template <class Sync, class Load, class Use>
+__device__ __forceinline__ void sweep_pairs(const Sync &g, int lo, int hi, Load load, Use use) {
+    const unsigned step = (unsigned)row_step(g), end = (unsigned)hi;
+    for (unsigned i = (unsigned)lo + threadIdx.x; i < end; i += 2 * step) {
+        const unsigned j = i + step;
+        const bool two = j < end;
+        decltype(load(0)) v = load((int)i), w = {};
+        if (two) w = load((int)j);
+        use((int)i, v);
+        if (two) use((int)j, w);
+    }
+}
+struct Row2 {
+    double a, b;
+};
+struct Row3 {
+    double a, b, c;
+};
+struct Row4 {
+    double a, b, c, d;
+};
+struct Row5 {
+    double a, b, c, d, e;
+};
+struct Row6 {
+    double a, b, c, d, e, f;
+};
 
 // Tests on scalars that need no FP64 instruction (64 cycles of a sub-partition's
 // FP64 pipe, about 140 to its result): finite and zero from the bits, and the
@@ -442,7 +481,7 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
         const T al = (T)X.s.alpha, be = (T)X.s.beta, om = (T)X.s.omega;
         if (!replaced_rw) {
             const int end = group_end<Op, kGroup>(A, hi);
-            for (int gi = lo + (int)threadIdx.x; gi < end; gi += row_step(g)) {
+            PBCG_STEPS(gi, end) {
                 int i0, cnt;
                 bool vec;
                 T ti[kGroup], ri[kGroup], wi[kGroup], si[kGroup], zi[kGroup], pi[kGroup], vi[kGroup], r0i[kGroup];
@@ -520,7 +559,7 @@ __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> 
         const T om2 = (T)X.s.omega;
         if (!replace_now) {
             const int end = group_end<Op, kGroup>(A, hi);
-            for (int gi = lo + (int)threadIdx.x; gi < end; gi += row_step(g)) {
+            PBCG_STEPS(gi, end) {
                 int i0, cnt;
                 bool vec;
                 T vi[kGroup], mid[kGroup], qi[kGroup], yi[kGroup], xi[kGroup], pi[kGroup], ti[kGroup], r0i[kGroup];
@@ -825,7 +864,8 @@ __device__ __forceinline__ bool standard_loop(const Op &A, const SolveArgs &a, S
                 a1.add({V.r0[i], si});
             }
         } else {
-            PBCG_ROWS(i) { pA[i] = fma(beta, fma(-om1, sA[i], pA[i]), V.r[i]); }
+            sweep_pairs(g, lo, hi, [&](int i) { return Row3{sA[i], pA[i], V.r[i]}; },
+                        [&](int i, const Row3 &v) { pA[i] = fma(beta, fma(-om1, v.a, v.b), v.c); });
             if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const double si = A.row(i, VecLoad{pA});
@@ -853,7 +893,8 @@ __device__ __forceinline__ bool standard_loop(const Op &A, const SolveArgs &a, S
                 a2.add({qi, yi});
             }
         } else {
-            PBCG_ROWS(i) { V.q[i] = fma(-alpha, sc[i], V.r[i]); }
+            sweep_pairs(g, lo, hi, [&](int i) { return Row2{sc[i], V.r[i]}; },
+                        [&](int i, const Row2 &v) { V.q[i] = fma(-alpha, v.a, v.b); });
             if (!grid_sync(g, X)) return false;
             PBCG_ROWS(i) {
                 const double yi = A.row(i, VecLoad{V.q});
@@ -885,13 +926,13 @@ __device__ __forceinline__ bool standard_loop(const Op &A, const SolveArgs &a, S
 
         // ---- x_{i+1}, r_{i+1}; beta_i
         typename DotsFor<Wide, PairsRho, double, B>::type a3(wide, lo + (int)threadIdx.x < hi);   // (r0,r) (r,r)
-        PBCG_ROWS(i) {
-            const double qi = V.q[i];
-            x[i] = fma(omega, qi, fma(alpha, pc[i], x[i]));
-            const double rn = fma(-omega, V.y[i], qi);
-            V.r[i] = rn;
-            a3.add({V.r0[i], rn});
-        }
+        sweep_pairs(g, lo, hi, [&](int i) { return Row5{V.q[i], pc[i], x[i], V.y[i], V.r0[i]}; },
+                    [&](int i, const Row5 &v) {
+                        x[i] = fma(omega, v.a, fma(alpha, v.b, v.c));
+                        const double rn = fma(-omega, v.d, v.a);
+                        V.r[i] = rn;
+                        a3.add({v.e, rn});
+                      });
         double d3[2];
         a3.values(d3);
         if (!exchange(g, d3, X, [&](Scalars &S, const double (&t)[2]) {
@@ -947,11 +988,12 @@ __device__ __forceinline__ bool standard_prec_loop(const Op &A, const SolveArgs 
     while (it < a.limit) {
         const double beta = X.s.beta, om1 = X.s.omega;
         // p_i := r_i + beta (p_{i-1} - omega s_{i-1}); p^_i := M^{-1} p_i; s_i := A p^_i
-        PBCG_ROWS(i) {
-            const double pn = fma(beta, fma(-om1, V.s[i], V.p[i]), V.r[i]);
-            V.p[i] = pn;
-            ph[i] = mi[i] * pn;
-        }
+        sweep_pairs(g, lo, hi, [&](int i) { return Row4{V.s[i], V.p[i], V.r[i], mi[i]}; },
+                    [&](int i, const Row4 &v) {
+                        const double pn = fma(beta, fma(-om1, v.a, v.b), v.c);
+                        V.p[i] = pn;
+                        ph[i] = v.d * pn;
+                    });
         if (!grid_sync(g, X)) return false;
         typename DotsFor<Wide, PairsOne, double, B>::type a1(wide, lo + (int)threadIdx.x < hi);   // (r0,s)
         PBCG_ROWS(i) {
@@ -966,11 +1008,12 @@ __device__ __forceinline__ bool standard_prec_loop(const Op &A, const SolveArgs 
         if (X.s.action == kStop) { o.status = X.s.status; break; }
         const double alpha = X.s.alpha;
         // q_i := r_i - alpha s_i; q^_i := M^{-1} q_i; y_i := A q^_i
-        PBCG_ROWS(i) {
-            const double qi = fma(-alpha, V.s[i], V.r[i]);
-            V.q[i] = qi;
-            qh[i] = mi[i] * qi;
-        }
+        sweep_pairs(g, lo, hi, [&](int i) { return Row3{V.s[i], V.r[i], mi[i]}; },
+                    [&](int i, const Row3 &v) {
+                        const double qi = fma(-alpha, v.a, v.b);
+                        V.q[i] = qi;
+                        qh[i] = v.c * qi;
+                    });
         if (!grid_sync(g, X)) return false;
         typename DotsFor<Wide, PairsOmega, double, B>::type a2(wide, lo + (int)threadIdx.x < hi);   // (q,y) (y,y) (q,q)
         PBCG_ROWS(i) {
@@ -1001,12 +1044,13 @@ __device__ __forceinline__ bool standard_prec_loop(const Op &A, const SolveArgs 
         const double omega = X.s.omega;
         // x_{i+1} := x_i + alpha p^_i + omega q^_i; r_{i+1} := q_i - omega y_i
         typename DotsFor<Wide, PairsRho, double, B>::type a3(wide, lo + (int)threadIdx.x < hi);   // (r0,r) (r,r)
-        PBCG_ROWS(i) {
-            x[i] = fma(omega, qh[i], fma(alpha, ph[i], x[i]));
-            const double rn = fma(-omega, V.y[i], V.q[i]);
-            V.r[i] = rn;
-            a3.add({V.r0[i], rn});
-        }
+        sweep_pairs(g, lo, hi, [&](int i) { return Row6{qh[i], ph[i], x[i], V.y[i], V.q[i], V.r0[i]}; },
+                    [&](int i, const Row6 &v) {
+                        x[i] = fma(omega, v.a, fma(alpha, v.b, v.c));
+                        const double rn = fma(-omega, v.d, v.e);
+                        V.r[i] = rn;
+                        a3.add({v.f, rn});
+                      });
         double d3[2];
         a3.values(d3);
         if (!exchange(g, d3, X, [&](Scalars &S, const double (&t)[2]) {
@@ -1598,5 +1642,6 @@ __global__ void csr_check_kernel(int n, int nnz, const int *rowptr, const int *c
 }
 
 #undef PBCG_ROWS
+#undef PBCG_STEPS
 
 }  // namespace pbcg
