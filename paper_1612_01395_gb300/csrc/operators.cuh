@@ -63,14 +63,16 @@ struct QLoad {
 //   half as much, 4 at a time lost. Taking only whole chunks and the rest one
 //   at a time lost 10 %: warps holding a boundary row ran both paths.
 // * Random rows of 9-33 entries (2^20 rows): 7 at a time 4-5 % faster.
-// * 5-point rows (1024^2): one at a time fastest; 5 at a time 4 % and 7 at a
-//   time 3-9 % slower. A predicated-off FP64 FMA occupies the FP64 pipe like
-//   a live one, and 2 of every 7 were dead.
-// The library therefore uses 7 at a time for matrices averaging more than 6
-// entries per row and the plain loop otherwise. FP32 and BF16 values (the
-// inner solves) take 8 at a time (4 and 6 measured slower); the batched
-// solver keeps the plain loop (its rows gained nothing from chunks), with
-// its gathers through L2 only (CsrOpGatherL2).
+// * 5-point rows: 5 at a time 3-6 % (Algorithm 9) and 1-5 % (Algorithm 7)
+//   faster than one at a time, from 160^2 (13.0 against 13.4 us an iteration)
+//   to 2048^2 (254.6 against 269.7 us); 3 at a time slower than one, and 7
+//   slower still: a predicated-off FP64 FMA occupies the FP64 pipe like a
+//   live one, and 2 of every 7 were dead.
+// The grid solves therefore use 7 at a time for matrices averaging more than
+// 6 entries per row and 5 otherwise. FP32 and BF16 values (the inner solves)
+// take 8 at a time (4 and 6 measured slower); the batched solver keeps the
+// plain loop (its rows gained nothing from chunks), with its gathers through
+// L2 only (CsrOpGatherL2).
 template <typename V, int kChunk = 8>
 struct CsrOpT {
     int n;
@@ -90,23 +92,25 @@ struct CsrOpT {
                 acc = fmaT(value_as<T>(__ldg(val + kk)), u(PBCG_SAFE(__ldg(col + kk), n)), acc);
             }
         } else {
-            for (int k0 = b; k0 < e; k0 += kChunk) {
+            // counted by what is left: k0 + kChunk may pass 2^31
+            int k0 = b;
+            for (int left = e - b; left > 0; left -= kChunk, k0 = (int)((unsigned)k0 + kChunk)) {
                 int c[kChunk] = {};
                 V v[kChunk] = {};
                 T xv[kChunk] = {};
 #pragma unroll
                 for (int j = 0; j < kChunk; ++j)
-                    if (k0 + j < e) {
+                    if (j < left) {
                         const int kk = PBCG_SAFE(k0 + j, nnz);
                         c[j] = __ldg(col + kk);
                         v[j] = __ldg(val + kk);
                     }
 #pragma unroll
                 for (int j = 0; j < kChunk; ++j)
-                    if (k0 + j < e) xv[j] = u(PBCG_SAFE(c[j], n));
+                    if (j < left) xv[j] = u(PBCG_SAFE(c[j], n));
 #pragma unroll
                 for (int j = 0; j < kChunk; ++j)
-                    if (k0 + j < e) acc = fmaT(value_as<T>(v[j]), xv[j], acc);
+                    if (j < left) acc = fmaT(value_as<T>(v[j]), xv[j], acc);
             }
         }
         return acc;
@@ -114,6 +118,7 @@ struct CsrOpT {
 };
 using CsrOpScalar = CsrOpT<double, 1>;    // one entry at a time
 using CsrOpChunked = CsrOpT<double, 7>;   // 7 entries at a time
+using CsrOpShort = CsrOpT<double, 5>;     // 5 entries at a time
 
 // A loader whose vector reads bypass L1 (ld.global.cg: cached in L2 only).
 template <class L>

@@ -46,6 +46,7 @@ constexpr int kPrecVectors = 6;   // preconditioned handles: M^{-1}, r^ s^ z^ q^
 
 size_t vec_stride(int32_t n) { return ((size_t)(n > 0 ? n : 1) + 31) / 32 * 32; }   // doubles
 
+pbcg::CsrOpShort shortrows(const pbcg::CsrOpScalar &a) { return pbcg::CsrOpShort{a.n, a.rowptr, a.col, a.val, a.nnz}; }
 pbcg::CsrOpChunked chunked(const pbcg::CsrOpScalar &a) { return pbcg::CsrOpChunked{a.n, a.rowptr, a.col, a.val, a.nnz}; }
 
 }  // namespace
@@ -397,7 +398,7 @@ pbcg_status run_solve(pbicgstab_s *h, bool pipelined, const double *d_b, double 
         else
             st = h->kind == 1 ? launch_solver(h, h->st, pipelined, a, shape)
                  : h->csr_chunked ? launch_solver(h, chunked(h->csr), pipelined, a, shape)
-                                  : launch_solver(h, h->csr, pipelined, a, shape);
+                                  : launch_solver(h, shortrows(h->csr), pipelined, a, shape);
         if (st != PBCG_OK) return st;
     }
     if (h->ev1) PBCG_CUDA(cudaEventRecord(h->ev1, h->stream));
@@ -476,7 +477,7 @@ pbcg_status pbicgstab_create_csr(int32_t n, int32_t nnz, const int32_t *d_rowptr
             st = occupancy<pbcg::CsrOpChunked>(h);
             cluster_limits<pbcg::CsrOpChunked>(h);
         } else {
-            st = occupancy<pbcg::CsrOpScalar>(h);
+            st = occupancy<pbcg::CsrOpShort>(h);
             cluster_limits<pbcg::CsrOpScalar>(h);
         }
     }
@@ -1130,7 +1131,7 @@ extern "C" pbcg_status pbicgstab_solve_csr_noalloc(int32_t n, int32_t nnz, const
         h.csr = pbcg::CsrOpScalar{n, d_rowptr, d_col, d_val, nnz};
         h.nnz = nnz;
         h.csr_chunked = (long long)nnz > pbcg::kChunkedMinAvgRow * (long long)n;
-        st = h.csr_chunked ? occupancy<pbcg::CsrOpChunked>(&h) : occupancy<pbcg::CsrOpScalar>(&h);
+        st = h.csr_chunked ? occupancy<pbcg::CsrOpChunked>(&h) : occupancy<pbcg::CsrOpShort>(&h);
         if (h.csr_chunked) cluster_limits<pbcg::CsrOpChunked>(&h);
         else cluster_limits<pbcg::CsrOpScalar>(&h);
     }

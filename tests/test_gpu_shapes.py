@@ -76,6 +76,30 @@ def test_on_chip_entries_that_do_not_fit_their_cta():
 
 
 @pytest.mark.parametrize("method", ["pipelined", "standard"])
+@pytest.mark.parametrize("prec", [native.PBCG_PREC_NONE, native.PBCG_PREC_JACOBI])
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 255, 256, 257, 1283])
+def test_short_rows_and_pairs_of_rows_on_a_grid(n, prec, method):
+    """Rows of 1 to 11 entries (averaging under 6) around the chunk of five, on
+    one and two blocks: no, one, an odd and an even number of rows a thread."""
+    a = np.zeros((n, n))
+    for i in range(n):
+        for k in range(1 + (7 * i) % 11 if i % 3 == 0 else 1 + i % 6):
+            a[i, (i + k * k * 5) % n] = -0.1 - 0.01 * k
+        a[i, i] = 3.0 + 0.001 * (i % 17)
+    A = P.dense_to_csr(a)
+    assert A.nnz <= 6 * n
+    s = native.Solver.from_csr(A, prec=prec)
+    b = oracle.spmv(A, P.splitmix64_uniform(3, n))
+    for grid in (1, 2):
+        x, info = s.solve(dev(b), rtol=1e-12, maxit=200, method=method, cluster=-1, grid=grid)
+        assert info["status"] == native.PBCG_OK and info["cluster"] == 0
+        # off-diagonal sums are at most 1.55, so |A^-1| <= 1 / 1.45 in the maximum norm;
+        # 4: the true residual against the recursive one that ended the solve
+        assert np.max(np.abs(x.cpu().numpy() - P.splitmix64_uniform(3, n))) <= 4 * 1e-12 * np.linalg.norm(b) / 1.45
+    s.close()
+
+
+@pytest.mark.parametrize("method", ["pipelined", "standard"])
 @pytest.mark.parametrize("form", ["csr", "stencil"])
 @pytest.mark.parametrize("dims", [(100, 100, 70), (83, 89, 95), (839, 837, 1)])
 def test_wide_sums_above_their_line(dims, form, method):
