@@ -11,7 +11,7 @@
 
 namespace pbcg {
 
-constexpr int kTPB = 128;          // threads per block of the cluster, batched and mixed-precision kernels
+constexpr int kTPB = 128;          // threads per block of the batched kernel, the cluster kernel and the SpMV
 constexpr int kMaxGrid = 2040;     // upper bound on thread blocks (kPartialBytes holds their slots)
 constexpr int kMaxDots = 8;        // dot products carried by one reduction
 constexpr uint64_t kSyncTimeoutNs = 4000000000ull;   // 4 s per grid-wide wait

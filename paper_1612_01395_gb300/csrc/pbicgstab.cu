@@ -184,11 +184,13 @@ long long max_index(const int64_t st[3], int nx, int ny, int nz) {
 // never hold less than one row per thread. Measured per iteration, p-BiCGStab /
 // BiCGStab, us:
 //                          1 x 256     2 x 256     2 x 512 wide  (blocks per SM)
-//    110k, 5-7 entries     22 / 26     26 / 31     -
-//    262k                  36 / 41     36 / 39     39 / 42
-//    490k                  55 / 62     52 / 52     56 / 55
-//    885k                  88 / 91     78 / 72     75 / 69
-//    1.05M, 5 entries      194 / 173   119 / 107   89 / 82
+//    110k, 7 points        20 / 24     23 / 26     -
+//    262k, 7 points        34 / 36     33 / 35     34 / 35
+//    262k, 5 entries       33 / 36     31 / 33     31 / 33
+//    491k, 7 points        53 / 52     49 / 48     49 / 47
+//    490k, 5 entries       54 / 53     45 / 44     43 / 42
+//    885k, 7 points        84 / 79     75 / 67     69 / 62
+//    1.05M, 5 entries      174 / 161   108 / 102   81 / 75
 // Long rows (21 random entries) are bound by their gathers, which the wide
 // sums do not shorten and their shared memory takes L1 from: 200k 91 / 90 at 2
 // x 256 against 126 / 128, 500k 212 / 208 against 264 / 251. Systems of less
@@ -360,10 +362,11 @@ pbcg_status run_solve(pbicgstab_s *h, bool pipelined, const double *d_b, double 
     a.replace_period = pipelined ? replace_period : 0;
     a.max_repl = o.max_replacements;
     // Variant 3 saves two grid synchronisations per iteration at the price of
-    // 18 more FP64 operations per row. Measured per iteration on 3-D
-    // convection-diffusion: variant 3 is faster up to 110k unknowns (33.0 vs
-    // 34.1 us), variant 5 from 176k (42.5 vs 43.1 us; 65 vs 74 us at 512k).
-    a.variant = o.plain_variant ? o.plain_variant : (h->n < 150000 ? 3 : 5);
+    // 18 more FP64 operations per row. Measured per iteration, variant 3 / 5,
+    // stencil and CSR, us: 64k rows 19.5 / 20.2 and 20.2 / 20.6; 90k (2-D) 22.9
+    // / 22.7 and 22.6 / 23.1; 110k 23.8 / 23.8 and 25.0 / 24.5; 141k 27.7 / 26.2
+    // and 29.3 / 27.6; 176k 31.4 / 29.6 and 33.4 / 31.2.
+    a.variant = o.plain_variant ? o.plain_variant : (h->n < 100000 ? 3 : 5);
     a.minv = h->prec == PBCG_PREC_JACOBI ? h->minv : nullptr;
     a.rh = h->rh;
     a.sh = h->sh;

@@ -60,7 +60,7 @@ using SolveArgs = SolveArgsT<double>;
 // and slot sums, so large blocks are cheaper: at 1216 blocks of 128 threads an
 // exchange cost about 15 us, at 304 of 512 about 5. Per iteration of Algorithm
 // 9 (stencil): 110k unknowns 28.7 us with 304 blocks of 128 threads, 22.1 with
-// 152 of 256; 2.1M 178 and 143 us; 16.8M 1177 and 960 us (with the wide sums).
+// 152 of 256; 2.1M 178 and 138 us; 16.8M 1177 and 940 us (with the wide sums).
 template <bool Wide>
 struct SolverBlock {
     static constexpr int kThreads = Wide ? 512 : 256;
