@@ -92,25 +92,29 @@ struct CsrOpT {
                 acc = fmaT(value_as<T>(__ldg(val + kk)), u(PBCG_SAFE(__ldg(col + kk), n)), acc);
             }
         } else {
-            // counted by what is left: k0 + kChunk may pass 2^31
-            int k0 = b;
-            for (int left = e - b; left > 0; left -= kChunk, k0 = (int)((unsigned)k0 + kChunk)) {
+            // Counted from the row's first entry, as b + kChunk may pass 2^31. 7 at
+            // a time compares with the length (SpMV at 256^3 311 against 332 us),
+            // the others with what is left (FP32 iterations at 64^3 26.4 against
+            // 27.6 us, 5-entry rows at 2048^2 254 against 261).
+            const int len = e - b;
+            for (int k0 = 0, left = len; left > 0; k0 += kChunk, left -= kChunk) {
+                const auto has = [&](int j) { return kChunk == 7 ? k0 + j < len : j < left; };
                 int c[kChunk] = {};
                 V v[kChunk] = {};
                 T xv[kChunk] = {};
 #pragma unroll
                 for (int j = 0; j < kChunk; ++j)
-                    if (j < left) {
-                        const int kk = PBCG_SAFE(k0 + j, nnz);
+                    if (has(j)) {
+                        const int kk = PBCG_SAFE(b + k0 + j, nnz);
                         c[j] = __ldg(col + kk);
                         v[j] = __ldg(val + kk);
                     }
 #pragma unroll
                 for (int j = 0; j < kChunk; ++j)
-                    if (j < left) xv[j] = u(PBCG_SAFE(c[j], n));
+                    if (has(j)) xv[j] = u(PBCG_SAFE(c[j], n));
 #pragma unroll
                 for (int j = 0; j < kChunk; ++j)
-                    if (j < left) acc = fmaT(value_as<T>(v[j]), xv[j], acc);
+                    if (has(j)) acc = fmaT(value_as<T>(v[j]), xv[j], acc);
             }
         }
         return acc;

@@ -46,6 +46,19 @@ constexpr int kPrecVectors = 6;   // preconditioned handles: M^{-1}, r^ s^ z^ q^
 
 size_t vec_stride(int32_t n) { return ((size_t)(n > 0 ? n : 1) + 31) / 32 * 32; }   // doubles
 
+// The same operator with a row's loads where they are used.
+pbcg::StencilOpLean lean(const pbcg::StencilOp &a) {
+    pbcg::StencilOpLean o;
+    o.n = a.n;
+    o.nx = a.nx;
+    o.ny = a.ny;
+    o.nz = a.nz;
+    o.nxy = a.nxy;
+    o.dx = a.dx;
+    o.dy = a.dy;
+    for (int d = 0; d < 7; ++d) o.c[d] = a.c[d];
+    return o;
+}
 pbcg::CsrOpShort shortrows(const pbcg::CsrOpScalar &a) { return pbcg::CsrOpShort{a.n, a.rowptr, a.col, a.val, a.nnz}; }
 pbcg::CsrOpChunked chunked(const pbcg::CsrOpScalar &a) { return pbcg::CsrOpChunked{a.n, a.rowptr, a.col, a.val, a.nnz}; }
 
@@ -608,6 +621,8 @@ pbcg_status pbicgstab_spmv(pbicgstab_t h, const double *d_x, double *d_y) {
         pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(chunked(h->csr), d_x, d_y);
     else if (h->kind == 0)
         pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(h->csr, d_x, d_y);
+    else if (h->st.nz == 1)   // loads ahead: 1024^2 16.8 against 15.4 us, 256^3 249 against 291
+        pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(lean(h->st), d_x, d_y);
     else
         pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(h->st, d_x, d_y);
     PBCG_CUDA(cudaGetLastError());
@@ -718,16 +733,7 @@ extern "C" pbcg_status pbicgstab_solve_mixed(pbicgstab_t h, const void *d_val_lo
         // vector area the 12 float vectors and the best iterate leave free
         // (10 * s floats).
         pbcg::StencilOpT<float, false> a32;
-        const pbcg::StencilOp &st64 = h->st;
-        pbcg::StencilOpLean a64;
-        a64.n = st64.n;
-        a64.nx = st64.nx;
-        a64.ny = st64.ny;
-        a64.nz = st64.nz;
-        a64.nxy = st64.nxy;
-        a64.dx = st64.dx;
-        a64.dy = st64.dy;
-        for (int d = 0; d < 7; ++d) a64.c[d] = st64.c[d];
+        const pbcg::StencilOpLean a64 = lean(h->st);
         a32.n = a64.n;
         a32.nx = a64.nx;
         a32.ny = a64.ny;
