@@ -274,9 +274,10 @@ struct StencilOpT {
             for (int m = 0; m < 4; ++m) v[m] = m < cnt ? u[PBCG_SAFE(at + m, n)] : 0.0f;
         }
     }
-    // acc[m] += coefficient d at node (i + m, j, k) * v[m]; each sum of two
-    // tables formed per node as in coef()
-    __device__ __forceinline__ void add4(int d, const Group &q, const float (&v)[4], float (&acc)[4]) const {
+    // acc[m] += coefficient d at node (i + m, j, k) * v[m] for m in [from, to);
+    // each sum of two tables formed per node as in coef()
+    __device__ __forceinline__ void add4(int d, const Group &q, const float (&v)[4], float (&acc)[4], int from = 0,
+                                         int to = 4) const {
         const StCoefT<C> &f = c[d];
         float w[4];
         if (f.t1) {
@@ -298,11 +299,15 @@ struct StencilOpT {
                 if (m < q.cnt) w[m] = add_rn(w[m], __ldg(f.t2 + PBCG_SAFE(at + m * f.a2, f.len2)));
         }
 #pragma unroll
-        for (int m = 0; m < 4; ++m) acc[m] = fmaT(w[m], v[m], acc[m]);
+        for (int m = 0; m < 4; ++m) {
+            const float t = fmaT(w[m], v[m], acc[m]);
+            acc[m] = m >= from && m < to ? t : acc[m];
+        }
     }
     // y = A u on the rows of a group, mid = u there; each row summed as row()
-    // sums it, except that a neighbour outside the grid adds 0 instead of
-    // nothing (no change to a finite sum). Rows past cnt read 0.
+    // sums it. The entries of neighbours outside the grid are left out, whatever
+    // the tables hold there (0 times a NaN or an infinity would be NaN). Rows
+    // past cnt read 0.
     __device__ __forceinline__ void product4(const Group &q, const float *u, float (&mid)[4], float (&y)[4]) const {
         float vb[4] = {}, vs[4] = {}, vn[4] = {}, vt[4] = {}, ve[4], vw[4];
         if (q.k > 0) load4(u, q.r - nxy, q.cnt, vb);
@@ -320,9 +325,9 @@ struct StencilOpT {
         }
         if (q.k > 0) add4(PBCG_B, q, vb, y);
         if (q.j > 0) add4(PBCG_S, q, vs, y);
-        add4(PBCG_W, q, vw, y);
+        add4(PBCG_W, q, vw, y, q.i > 0 ? 0 : 1);
         add4(PBCG_C, q, mid, y);
-        add4(PBCG_E, q, ve, y);
+        add4(PBCG_E, q, ve, y, 0, nx - 1 - q.i);
         if (q.j < ny - 1) add4(PBCG_N, q, vn, y);
         if (q.k < nz - 1) add4(PBCG_T, q, vt, y);
 #pragma unroll

@@ -147,6 +147,28 @@ def test_fp32_groups_of_rows(dims):
     s.close()
 
 
+@pytest.mark.parametrize("bad", [np.nan, -np.inf, 1e300])
+@pytest.mark.parametrize("dims", [(8, 9, 1), (5, 6, 4), (6, 5, 4), (7, 3, 5), (1, 9, 3), (64, 3, 2)])
+def test_fp32_groups_drop_the_entries_outside_the_grid(dims, bad):
+    """West and east entries at the ends of an x-line belong to no neighbour: what
+    the tables (or, on lines of one node, the constants) hold there changes nothing."""
+    nx = dims[0]
+    out = {}
+    for fill in (0.0, bad):
+        st = grid_stencil(*dims)
+        west, east = -1.1 - 0.01 * np.arange(nx), -0.9 + 0.01 * np.arange(nx)
+        west[0] = east[-1] = fill
+        st.coefs[P.W] = P.Coef(table=west, stride=(1, 0, 0))
+        st.coefs[P.E] = P.Coef(table=east, stride=(1, 0, 0)) if nx > 1 else P.Coef(value=fill)
+        s = native.Solver.from_stencil(st)
+        x, info = s.solve_mixed(dev(P.splitmix64_uniform(4, st.n)), None, rtol=1e-12, inner_rtol=1e-3)
+        assert info["status"] == native.PBCG_OK
+        out[fill == 0.0] = x.cpu().numpy(), info["inner_iters"]
+        s.close()
+    np.testing.assert_array_equal(out[True][0], out[False][0])
+    assert out[True][1] == out[False][1]
+
+
 @pytest.mark.parametrize("n", [0, 1, 4094, 4095, 4096, 12289])
 def test_transpose_row_pointers_at_the_tiles_of_the_scan(n):
     import torch
