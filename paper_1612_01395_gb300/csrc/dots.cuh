@@ -55,14 +55,24 @@ PBCG_HD uint32_t wide_mulhi(uint32_t a, uint32_t b) {
     return (uint32_t)(((uint64_t)a * b) >> 32);
 #endif
 }
-// v >> s for 0 <= s, 0 from 64 on
+// v >> s, 0 for s < 0 and from 64 on (the instruction takes s as unsigned and clamps it)
 PBCG_HD uint64_t wide_shr(uint64_t v, int s) {
 #ifdef __CUDA_ARCH__
     uint64_t r;
     asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
     return r;
 #else
-    return s > 63 ? 0 : v >> s;
+    return s < 0 || s > 63 ? 0 : v >> s;
+#endif
+}
+// v << s, 0 for s < 0 and from 32 on
+PBCG_HD uint32_t wide_shl(uint32_t v, int s) {
+#ifdef __CUDA_ARCH__
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
+    return r;
+#else
+    return s < 0 || s > 31 ? 0 : v << s;
 #endif
 }
 PBCG_HD uint64_t wide_bits(double v) {
@@ -100,25 +110,34 @@ PBCG_HD int wide_clz(uint32_t v) {   // 32 for 0
 // integer instructions of different warps overlap fully.
 //
 // A product of two 53-bit significands (each shifted to the top of 63 bits) is
-// formed to 62 bits by three 32-bit multiplies, with an error of at most 3
-// units in the last place, shifted right by the distance of its exponent to a
-// reference exponent, and added with its sign; the top word leaves room for
-// 2^33 products. The reference is kWideMargin binades above the largest product
-// of the warp's first rows; a product above it moves it to kWideMargin binades
+// formed to 62 bits by three 32-bit multiplies, 3 units too small at most,
+// shifted right by the distance of its exponent to a reference exponent, and
+// added with its sign; kWideRoom bits above it leave room for kWideThreadRows
+// products. The reference is kWideMargin binades above the largest product of
+// the WARP's first rows; a product above it moves it to kWideMargin binades
 // above itself and shifts the sum. (A reference from each thread's own first
 // row moved in some lane of the warp at every other row, and the sweep was
-// slower than with FP64 sums.) So each term is exact to 2^-(60 - kWideMargin)
-// = 2^-54 of the largest product met, where an FP64 FMA chain rounds the
-// running sum to 2^-53 of itself at every step: over 2 to 1000 products of
-// normal, uniform and log-normal values the largest error, relative to the sum
-// of the absolute products, was 1.4e-16 to 2.2e-16 against 2.0e-16 to 3.2e-15.
-// Subnormal values count as zero (their products are below 2^-510 of the
-// square of any value whose square is representable). A product with an
-// infinite or NaN factor is noted and decides the result as in an FP64 sum.
+// slower than with FP64 sums.) A term keeps all bits down to the unit of the
+// sum, which is at most 2^-73 of the largest product that the warp has met:
+// all units that the 32 x kWideThreadRows terms of a warp can lose (one at the
+// addition, one at a move) add up to less than 2^-53 of that product, so the
+// warp's common reference costs no accuracy next to the rounding of one
+// thread's sum to a double, whatever the ratio between its lanes. An FP64 FMA
+// chain rounds the running sum at every step. Largest error of a warp's sum,
+// relative to the sum of its absolute products, over 107, 1000 and 13000 rows a
+// thread of normal values with one of 1, 1e2, 1e4 or 1e6 times that among the
+// first: 1.1e-16, against 1.3e-14 with FP64 chains. (With the product aligned
+// to the upper two words, a unit of 2^-54 of the warp's largest product, the
+// outlier cost the other lanes their low bits: 4e-12 at 13000 rows and 1e4.)
+// A product with an infinite or NaN factor is noted and decides the result as
+// in an FP64 sum.
 constexpr int kWideMargin = 6;
+constexpr int kWideRoom = 13;               // products below 2^(95 - 14): 2^14 of them and a sign
+constexpr int kWideThreadRows = 1 << 14;    // most rows of a thread
+constexpr int kWideBias = 2106 + 32 - kWideRoom;
 constexpr int kWideAbsent = -8192;   // exponent of a value whose products vanish
 
-// A fixed-point number (w2 w1 w0) 2^(ref - 2106), two's complement: the sum of
+// A fixed-point number (w2 w1 w0) 2^(ref - kWideBias), two's complement: the sum of
 // one dot product over the rows of a thread.
 struct alignas(16) WideSlot {
     uint32_t w0, w1, w2;
@@ -157,7 +176,7 @@ PBCG_HD double wide_value(const WideSlot &c, unsigned f) {
     t = (uint64_t)(c.w1 ^ sign) + (t >> 32);
     uint32_t a1 = (uint32_t)t;
     uint32_t a2 = (c.w2 ^ sign) + (uint32_t)(t >> 32);
-    int ex = c.ref - 2106 + 64;   // |sum| = (a2 a1 a0) 2^(ex - 64); move its leading word to a2
+    int ex = c.ref - kWideBias + 64;   // |sum| = (a2 a1 a0) 2^(ex - 64); move its leading word to a2
     if (a2 == 0) {
         a2 = a1;
         a1 = a0;
@@ -207,27 +226,31 @@ PBCG_HD WideParts wide_parts(double v) {
     return p;
 }
 
-// Add the product of a and b (square: a times itself) to c; its exponent is at most the reference.
-PBCG_HD void wide_add(WideSlot &c, const WideParts &a, const WideParts &b, bool square, int shift) {
+// Add the product of a and b (square: a times itself) to c; its exponent is `distance` below the reference.
+PBCG_HD void wide_add(WideSlot &c, const WideParts &a, const WideParts &b, bool square, int distance) {
     const uint32_t mid = square ? 2u * wide_mulhi(a.mh, a.ml) : wide_mulhi(a.mh, b.ml) + wide_mulhi(a.ml, b.mh);
-    const uint64_t q = wide_shr((uint64_t)a.mh * b.mh + mid, shift);
+    const uint64_t q = (uint64_t)a.mh * b.mh + mid;
     const uint32_t sg = square ? 0u : (uint32_t)((int)(a.hi ^ b.hi) >> 31);
-    const uint32_t q0 = (uint32_t)q ^ sg, q1 = (uint32_t)(q >> 32) ^ sg;   // ~q for a negative product
+    // the words of q 2^32 >> shift; the lowest from the left shift below 32 and from the right one above
+    const int shift = distance + kWideRoom;
+    const uint64_t top = wide_shr(q, shift);
+    const uint32_t q0 = (wide_shl((uint32_t)q, 32 - shift) | (uint32_t)wide_shr(q, shift - 32)) ^ sg;
+    const uint32_t q1 = (uint32_t)top ^ sg, q2 = (uint32_t)(top >> 32) ^ sg;   // ~q for a negative product
 #ifdef __CUDA_ARCH__
     if (square)
-        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, 0;"
+        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
             : "+r"(c.w0), "+r"(c.w1), "+r"(c.w2)
-            : "r"(q0), "r"(q1));
+            : "r"(q0), "r"(q1), "r"(q2));
     else   // the first addition only makes the carry, 1 for a negative product: -q = ~q + 1
-        asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %5, %5;\n\taddc.cc.u32 %0, %0, %3;\n\t"
+        asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %6, %6;\n\taddc.cc.u32 %0, %0, %3;\n\t"
             "addc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;\n\t}"
             : "+r"(c.w0), "+r"(c.w1), "+r"(c.w2)
-            : "r"(q0), "r"(q1), "r"(sg));
+            : "r"(q0), "r"(q1), "r"(q2), "r"(sg));
 #else
     const uint64_t t0 = (uint64_t)c.w0 + q0 + (sg & 1u), t1 = (uint64_t)c.w1 + q1 + (t0 >> 32);
     c.w0 = (uint32_t)t0;
     c.w1 = (uint32_t)t1;
-    c.w2 += sg + (uint32_t)(t1 >> 32);
+    c.w2 += q2 + (uint32_t)(t1 >> 32);
 #endif
 }
 
@@ -283,19 +306,24 @@ struct WideDots {
             if (p[j].e == 0 || p[j].e == 2047) p[j].e = kWideAbsent;
     }
 
+    // Exponent of product k of a row.
+    PBCG_HD static int product_exponent(const WideParts (&p)[P::nv], int k) {
+        const int e = p[P::a(k)].e + p[P::b(k)].e;
+        return e < 0 ? 0 : e;
+    }
     // Empty sums with their references above the largest product of the warp's first rows.
     PBCG_HD void first(const WideParts (&p)[P::nv]) {
 #pragma unroll
         for (int k = 0; k < P::np; ++k) {
-            int top = p[P::a(k)].e + p[P::b(k)].e;
-            top = top < 0 ? 0 : top;
+            int top = product_exponent(p, k);
 #ifdef __CUDA_ARCH__
             top = __reduce_max_sync(lanes, top);
 #endif
-            slot[k * stride] = WideSlot{0u, 0u, 0u, top + kWideMargin};
+            begin(k, top);
         }
         lanes = 0u;
     }
+    PBCG_HD void begin(int k, int top) { slot[k * stride] = WideSlot{0u, 0u, 0u, top + kWideMargin}; }
 
     // The sums (a thread without a row has none to read).
     PBCG_HD void values(bool any, double (&d)[P::np]) const {

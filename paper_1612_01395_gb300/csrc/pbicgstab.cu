@@ -225,7 +225,8 @@ Shape pick_shape(const pbicgstab_s *h, const int occ[2], bool can_wide, int req)
         const bool long_rows = h->nnz > kLongRow * n;
         int per_sm = n <= kOneBlockRows && !long_rows ? 1 : 2;
         if (long_rows && n > kWideRows) per_sm = occ[0];
-        s.wide = can_wide && !long_rows && n > kWideRows;
+        const long long wide_threads = (per_sm < occ[1] ? per_sm : occ[1]) * h->num_sms * solver_threads(true);
+        s.wide = can_wide && !long_rows && n > kWideRows && n <= wide_threads * pbcg::kWideThreadRows;
         s.block = solver_threads(s.wide);
         if (n <= (long long)h->num_sms * (s.block / 2)) s.block /= 2;
         const long long one_row = (n + s.block - 1) / s.block;

@@ -5,7 +5,8 @@ A term is formed with an error of at most 3 units and truncated by less than
 one unit of 2^-(60 - 6) = 2^-54 of the largest product met; a move of the
 reference drops less than one unit, at most once a term; the result is rounded
 to 53 bits. So the error of a sum of n terms is at most
-5 n 2^-54 max|a b| + 2^-53 |sum|.
+5 n 2^-54 max|a b| + 2^-53 |sum|. The sums of a warp's lanes, which share their
+first reference, are held to what their code keeps (test of a warp).
 """
 import ctypes
 import math
@@ -18,6 +19,8 @@ import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1612_01395_gb300", "csrc")
 SOURCE = r"""
+#include <algorithm>
+#include <vector>
 #include "dots.cuh"
 using namespace pbcg;
 template <class P> static void run(int n, const double *v, double *out) {
@@ -31,6 +34,31 @@ template <class P> static void run(int n, const double *v, double *out) {
     double o[P::np];
     d.values(n > 0, o);
     for (int k = 0; k < P::np; ++k) out[k] = o[k];
+}
+// One warp: lane l has the rows l, l + 32, ...; the first references are common, as in a kernel.
+extern "C" void warp_one(int rows, const double *v, double *out) {
+    using D = WideDots<PairsOne>;
+    std::vector<WideSlot> slots(32);
+    std::vector<D> lanes;
+    int top = 0;
+    for (int l = 0; l < 32; ++l) {
+        lanes.emplace_back(&slots[l], 1, 1);
+        double r[2] = {v[2 * l], v[2 * l + 1]};
+        WideParts p[2] = {wide_parts(r[0]), wide_parts(r[1])};
+        D probe(nullptr, 1, 1);
+        probe.unusual(r, p, p[0].e > p[1].e ? p[0].e : p[1].e);
+        top = std::max(top, D::product_exponent(p, 0));
+    }
+    for (int l = 0; l < 32; ++l) {
+        lanes[l].begin(0, top);
+        lanes[l].lanes = 0u;
+    }
+    for (int i = 0; i < rows * 32; ++i) lanes[i % 32].add({v[2 * i], v[2 * i + 1]});
+    for (int l = 0; l < 32; ++l) {
+        double o[1];
+        lanes[l].values(true, o);
+        out[l] = o[0];
+    }
 }
 extern "C" void pipe_a(int n, const double *v, double *o) { run<PairsPipeA>(n, v, o); }
 extern "C" void pipe_b(int n, const double *v, double *o) { run<PairsPipeB>(n, v, o); }
@@ -111,3 +139,35 @@ def test_no_rows_zero_rows_and_non_finite_values(lib):
     assert one([1e200, 1e200], [1.0, 1.0]) == inf   # a sum above the range
     b = sums(lib, "pipe_b", np.array([[1.0, 2.0, 3.0], [1.0, 4.0, nan]]))   # r0, r, w: only (r0, w) meets the NaN
     assert b[0] == 6.0 and math.isnan(b[1]) and b[2] == 20.0
+
+
+def exact_products(v):
+    """The products of each pair as whole numbers and the exponent of 2 they share."""
+    m, e = np.frexp(v)
+    m = (m * 2.0 ** 53).astype(np.int64)
+    e = e.sum(axis=1) - 106
+    low = int(e.min())
+    return [int(a) * int(b) << int(x) - low for (a, b), x in zip(m, e)], low
+
+
+@pytest.mark.parametrize("square", [True, False])
+@pytest.mark.parametrize("outlier", [1.0, 1e2, 1e4, 1e6, 1e12])
+@pytest.mark.parametrize("rows", [1, 107, 3000])
+def test_lanes_of_a_warp_with_one_outlier(lib, rows, outlier, square):
+    """Lanes share the reference of the warp's first rows. A term loses one unit of the
+    sum at the addition and one at most at moves, each at most 2^-73 of the warp's largest
+    product, and 3 * 2^-60 of itself; a lane's sum is rounded to 53 bits."""
+    g = np.random.default_rng(rows)
+    v = g.standard_normal((32 * rows, 2))
+    v[5] *= outlier
+    if square:
+        v[:, 1] = v[:, 0]
+    v = np.ascontiguousarray(v)
+    out = np.empty(32)
+    lib.warp_one(rows, v.ctypes.data_as(ctypes.c_void_p), out.ctypes.data_as(ctypes.c_void_p))
+    p, low = exact_products(v)
+    scale = Fraction(2) ** low
+    lane = [sum(p[k::32]) * scale for k in range(32)]
+    bound = 2 * len(p) * max(map(abs, p)) * scale / 2 ** 73 + 3 * sum(map(abs, p)) * scale / 2 ** 60
+    bound += sum(map(abs, lane)) / 2 ** 53
+    assert abs(sum(Fraction(float(o)) for o in out) - sum(lane)) <= bound
