@@ -46,7 +46,8 @@ ORACLE_ITERS = {"pbicgstab_rr50": 415, "bicgstab": 352}
 # launch, valid only for the kernel sources it was taken on: SHA-256 over
 # KERNEL_SOURCES.
 KERNEL_SOURCES = ["paper_1612_01395_gb300/csrc/device_common.cuh", "paper_1612_01395_gb300/csrc/dots.cuh",
-                  "paper_1612_01395_gb300/csrc/operators.cuh", "paper_1612_01395_gb300/csrc/solvers.cuh"]
+                  "paper_1612_01395_gb300/csrc/operators.cuh", "paper_1612_01395_gb300/csrc/portable.cuh",
+                  "paper_1612_01395_gb300/csrc/solvers.cuh"]
 TRAFFIC_CAPTURE = {"bytes_per_launch": 706966556672 + 502009335296, "n": 16777216, "iters": 374, "grid": 304,
                    "sources_sha256": "15f2ef40324ea677bf49b8a4fca468e20bd4cff07542f3eb4a1b9df4634790c3"}
 

@@ -14,7 +14,7 @@ namespace pbcg {
 
 // counts[c + 1] += 1 for every stored column c (counts zeroed by the caller)
 __global__ void transpose_count_kernel(int nnz, const int *col, int *counts) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nnz; k += gridDim.x * blockDim.x)
+    PBCG_ELEMENTS(k, nnz)
         atomicAdd(&counts[col[k] + 1], 1);
 }
 
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(int m, int *a,
 // Scatter entry (i, c, v) of A to row c of A^T at the next free slot.
 __global__ void transpose_scatter_kernel(int n, const int *rowptr, const int *col, const double *val,
                                          const int *trow, int *cursor, int *tcol, double *tval) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    PBCG_ELEMENTS(i, n) {
         for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) {
             const int c = PBCG_SAFE(col[k], n);
             const int pos = trow[c] + atomicAdd(&cursor[c], 1);
@@ -104,7 +104,7 @@ __global__ void transpose_scatter_kernel(int n, const int *rowptr, const int *co
 
 // Sort every row of A^T by column (insertion sort; rows are short).
 __global__ void sort_rows_kernel(int n, const int *rowptr, int *col, double *val) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    PBCG_ELEMENTS(i, n) {
         const int b = rowptr[i], e = rowptr[i + 1];
         for (int k = b + 1; k < e; ++k) {
             const int c = col[k];
@@ -124,7 +124,7 @@ __global__ void sort_rows_kernel(int n, const int *rowptr, int *col, double *val
 // g[k] = -lambda[i] * x[col[k]] for every stored entry k of row i.
 __global__ void value_grad_kernel(int n, const int *rowptr, const int *col, const double *lambda, const double *x,
                                   double *g) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    PBCG_ELEMENTS(i, n) {
         const double li = lambda[i];
         for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) g[k] = -li * x[PBCG_SAFE(col[k], n)];
     }

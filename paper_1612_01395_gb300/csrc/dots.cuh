@@ -9,11 +9,7 @@
 #include <cstdint>
 #include <cstring>
 
-#ifdef __CUDACC__
-#define PBCG_HD __host__ __device__ __forceinline__
-#else
-#define PBCG_HD inline
-#endif
+#include "portable.cuh"
 
 namespace pbcg {
 

@@ -175,7 +175,7 @@ template <class Launch>
 pbcg_status setup_jacobi(pbicgstab_s *h, Launch launch) {
     int *flag = &h->ctl->abort;
     PBCG_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), h->stream));
-    int blocks = (h->n + 255) / 256;
+    int blocks = (int)(((long long)h->n + 255) / 256);
     if (blocks > 4 * h->num_sms) blocks = 4 * h->num_sms;
     if (blocks < 1) blocks = 1;
     launch(blocks, flag);
@@ -319,7 +319,7 @@ int onchip_cap(const pbicgstab_s *h, int size, int m) {
 template <class Op>
 pbcg_status launch_cluster(pbicgstab_s *h, const Op &op, bool pipelined, const pbcg::SolveArgs &args, int size,
                            bool any_variant, int *block) {
-    const int m = (h->n + size - 1) / size, cap = onchip_cap(h, size, m);
+    const int m = (int)(((long long)h->n + size - 1) / size), cap = onchip_cap(h, size, m);
     const size_t bytes = pbcg::onchip_bytes(m, cap);
     if (size <= h->onchip_max && bytes <= pbcg::kOnChipMaxBytes) {
         *block = m >= pbcg::kOnChipTPB ? pbcg::kOnChipTPB : (m + 31) / 32 * 32;
@@ -616,7 +616,7 @@ pbcg_status pbicgstab_spmv(pbicgstab_t h, const double *d_x, double *d_y) {
     if (h->n == 0) return PBCG_OK;
     if (!d_x || !d_y) return fail(PBCG_ERR_ARG, "x or y is NULL");
     if ((d_x < d_y + h->n) && (d_y < d_x + h->n)) return fail(PBCG_ERR_ARG, "x and y overlap");
-    int blocks = (h->n + pbcg::kTPB - 1) / pbcg::kTPB;
+    int blocks = (int)(((long long)h->n + pbcg::kTPB - 1) / pbcg::kTPB);
     if (blocks > 16 * h->num_sms) blocks = 16 * h->num_sms;
     if (h->kind == 0 && h->csr_chunked)
         pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(chunked(h->csr), d_x, d_y);

@@ -1427,7 +1427,7 @@ __global__ void __launch_bounds__(kOnChipTPB, 1) onchip_solve_kernel(const Op A,
 
 // M^{-1} = 1 / diag(A) (Jacobi). A zero or non-finite diagonal entry sets *bad.
 __global__ void jacobi_csr_kernel(int n, const int *rowptr, const int *col, const double *val, double *minv, int *bad) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    PBCG_ELEMENTS(i, n) {
         double d = 0.0;
         for (int k = rowptr[i]; k < rowptr[i + 1]; ++k)
             if (col[k] == i) d = val[k];
@@ -1437,7 +1437,7 @@ __global__ void jacobi_csr_kernel(int n, const int *rowptr, const int *col, cons
     }
 }
 __global__ void jacobi_stencil_kernel(const StencilOp A, double *minv, int *bad) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < A.n; r += gridDim.x * blockDim.x) {
+    PBCG_ELEMENTS(r, A.n) {
         const int t = (int)A.dx.div((uint32_t)r);
         const int i = r - t * A.nx;
         const int k = (int)A.dy.div((uint32_t)t);
@@ -1622,20 +1622,19 @@ __global__ void to_float_kernel(const double *in, float *out, long long len) {
 template <class Op>
 __global__ void __launch_bounds__(kTPB) spmv_kernel(const Op A, const double *x, double *y) {
     const VecLoad u{x};
-    for (int i = blockIdx.x * kTPB + threadIdx.x; i < A.n; i += gridDim.x * kTPB) y[i] = A.row(i, u);
+    PBCG_ELEMENTS(i, A.n) y[i] = A.row(i, u);
 }
 
 // CSR structure check: rowptr[0] == 0, non-decreasing, rowptr[n] == nnz, 0 <= col < n.
 __global__ void csr_check_kernel(int n, int nnz, const int *rowptr, const int *col, int *bad) {
-    const int stride = gridDim.x * blockDim.x;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += stride) {
+    PBCG_ELEMENTS(i, (unsigned)n + 1u) {
         const int a = rowptr[i];
         if (i == 0 && a != 0) atomicOr(bad, 1);
         if (i == n && a != nnz) atomicOr(bad, 2);
         if (i < n && rowptr[i + 1] < a) atomicOr(bad, 4);
         if (a < 0 || a > nnz) atomicOr(bad, 8);
     }
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nnz; k += stride) {
+    PBCG_ELEMENTS(k, nnz) {
         const int c = col[k];
         if (c < 0 || c >= n) atomicOr(bad, 16);
     }

@@ -1,0 +1,56 @@
+"""Index arithmetic of the kernels near 2^31 (csrc/portable.cuh), compiled for
+the host: sizes that the entry points accept, whose kernels are too large to
+run in a test."""
+import ctypes
+import glob
+import os
+import re
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1612_01395_gb300", "csrc")
+SOURCE = r"""
+#include "portable.cuh"
+struct Dim { unsigned x; };
+static Dim blockIdx, blockDim, threadIdx, gridDim;
+// The first four elements of a thread of a grid of grid x block threads.
+extern "C" int elements(unsigned grid, unsigned block, unsigned b, unsigned t, unsigned count, int *out) {
+    gridDim.x = grid; blockDim.x = block; blockIdx.x = b; threadIdx.x = t;
+    int c = 0;
+    PBCG_ELEMENTS(i, count) {
+        out[c++] = i;
+        if (c == 4) break;
+    }
+    return c;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("index")
+    src, so = d / "index.cpp", d / "index.so"
+    src.write_text(SOURCE)
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-o", str(so), str(src)])
+    return ctypes.CDLL(str(so))
+
+
+@pytest.mark.parametrize("count", [0, 1, 1000, 46340 * 46340, 2 ** 31 - 1, 2 ** 31])
+@pytest.mark.parametrize("grid,block", [(608, 256), (2432, 128), (1, 32)])
+def test_last_elements_of_a_thread(lib, grid, block, count):
+    """A block index beyond the grid stands for a later step of a block of it."""
+    out = (ctypes.c_int * 4)()
+    step = grid * block
+    for start in {0, 5, max(0, count - 1), max(0, count - step), max(0, count - step - 1), max(0, count - 2 * step)}:
+        c = lib.elements(grid, block, start // block, start % block, ctypes.c_uint(count), out)
+        expect = [i for i in range(start, start + 4 * step, step) if i < count]
+        assert list(out[:c]) == expect
+
+
+def test_kernels_step_through_elements_by_this_loop():
+    """No kernel adds the threads of the grid to a signed 32-bit index of its own."""
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        text = open(path).read()
+        if not path.endswith("portable.cuh"):
+            assert not re.search(r"\+=\s*(gridDim\.x|stride)\b", text), path
