@@ -242,7 +242,7 @@ struct StencilOpT {
     // and the coefficient loads that do not vary along x, and takes its vectors
     // in 128-bit accesses where nx % 4 == 0 (then every group starts on a
     // multiple of 4 rows, and so do its neighbours at nx and nx*ny).
-    int gx;        // groups per x-line, ceil(nx / 4)
+    int gx;        // groups per x-line, groups_of(nx, 4)
     FastDiv dg;    // by gx
     int aligned;   // nx % 4 == 0
 
@@ -316,7 +316,7 @@ struct StencilOpT {
         if (q.j < ny - 1) load4(u, q.r + nx, q.cnt, vn);
         if (q.k < nz - 1) load4(u, q.r + nxy, q.cnt, vt);
         const float left = q.i > 0 ? u[PBCG_SAFE(q.r - 1, n)] : 0.0f;
-        const float right = q.i + 4 < nx ? u[PBCG_SAFE(q.r + 4, n)] : 0.0f;
+        const float right = q.i < nx - 4 ? u[PBCG_SAFE(q.r + 4, n)] : 0.0f;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             vw[m] = m > 0 ? mid[m - 1] : left;

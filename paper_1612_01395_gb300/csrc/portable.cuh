@@ -7,6 +7,9 @@
 #define PBCG_HD inline
 #endif
 
+// Groups of g that n elements make, the last perhaps smaller (n + g - 1 may pass 2^31).
+PBCG_HD int groups_of(int n, int g) { return n / g + (n % g != 0); }
+
 // The elements below count (at most 2^31) that belong to a thread of a kernel:
 // every (threads of the grid)-th. The steps are unsigned: the index after the
 // last may lie above 2^31, and a signed one would wrap below the bound again.

@@ -397,7 +397,7 @@ struct RowGroup {
 template <class Op, int G>
 __device__ __forceinline__ int group_end(const Op &A, int hi) {
     if constexpr (HasGroups<Op>::value && G == 4) return A.groups();
-    else return (hi + G - 1) / G;
+    else return groups_of(hi, G);
 }
 // Rows i0 .. i0 + cnt - 1 of group gi, y = A u there and mid = u there (where asked for).
 template <bool kMid, class Op, int G, typename T>

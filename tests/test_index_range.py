@@ -12,6 +12,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1612_01395_gb300", "csrc")
 SOURCE = r"""
 #include "portable.cuh"
+extern "C" int groups(int n, int g) { return groups_of(n, g); }
 struct Dim { unsigned x; };
 static Dim blockIdx, blockDim, threadIdx, gridDim;
 // The first four elements of a thread of a grid of grid x block threads.
@@ -46,6 +47,14 @@ def test_last_elements_of_a_thread(lib, grid, block, count):
         c = lib.elements(grid, block, start // block, start % block, ctypes.c_uint(count), out)
         expect = [i for i in range(start, start + 4 * step, step) if i < count]
         assert list(out[:c]) == expect
+
+
+@pytest.mark.parametrize("g", [1, 2, 4])
+@pytest.mark.parametrize("n", [0, 1, 2, 3, 4, 5, 2 ** 31 - 4, 2 ** 31 - 3, 2 ** 31 - 2, 2 ** 31 - 1])
+def test_groups_of_rows(lib, n, g):
+    """Groups of a system or of an x-line; their first rows stay below 2^31."""
+    assert lib.groups(n, g) == -(-n // g)
+    assert (lib.groups(n, g) - 1) * g < 2 ** 31
 
 
 def test_kernels_step_through_elements_by_this_loop():
