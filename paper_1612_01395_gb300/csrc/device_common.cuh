@@ -274,10 +274,11 @@ __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v) {
 // solves alone; CTA rank 0 of a cluster (is_leader overloads below).
 __device__ __forceinline__ bool is_leader(const GridSync &) { return blockIdx.x == 0; }
 
-// Thread 0: spin until *word >= target, bounded; false on abort or timeout.
-__device__ __forceinline__ bool wait_at_least(GridSync &g, const unsigned *word, unsigned target) {
+// Thread 0: spin until *word has reached target, bounded; false on abort or timeout.
+// (A solve of more than 2^32 / blocks exchanges wraps the counter of arrivals.)
+__device__ __forceinline__ bool wait_until(GridSync &g, const unsigned *word, unsigned target) {
     const uint64_t t0 = globaltimer_ns();
-    for (unsigned spin = 1; ld_acquire_u32(word) < target; ++spin) {
+    for (unsigned spin = 1; !reached(ld_acquire_u32(word), target); ++spin) {
         if (spin % 8 != 0) continue;   // the flag and the clock now and then: each poll is a round trip to L2
         if (ld_relaxed_s32(&g.ctl->abort) != 0) return false;
         if (globaltimer_ns() - t0 > g.limit_ns) {
@@ -294,7 +295,7 @@ __device__ __forceinline__ bool grid_sync(GridSync &g, Exchange<T> &X) {
     __syncthreads();   // every thread's stores of this phase precede thread 0's fence
     if (threadIdx.x == 0) {
         red_release_inc(&g.ctl->arrivals);
-        if (!wait_at_least(g, &g.ctl->arrivals, (g.epoch + 1u) * gridDim.x)) X.ok = 0;
+        if (!wait_until(g, &g.ctl->arrivals, (g.epoch + 1u) * gridDim.x)) X.ok = 0;
     }
     __syncthreads();
     g.epoch++;
@@ -347,7 +348,7 @@ __device__ __forceinline__ bool exchange(GridSync &g, double (&v)[K], Exchange<T
             X.last = atom_acq_rel_inc(&g.ctl->arrivals) == target - 1u;
         } else {
             red_release_inc(&g.ctl->arrivals);
-            if (!wait_at_least(g, &g.ctl->arrivals, target)) X.ok = 0;
+            if (!wait_until(g, &g.ctl->arrivals, target)) X.ok = 0;
         }
     }
     __syncthreads();
@@ -368,7 +369,7 @@ __device__ __forceinline__ bool exchange(GridSync &g, double (&v)[K], Exchange<T
         }
     } else if (wid == 0) {
         if (lane == 0) {
-            if (!wait_at_least(g, &g.ctl->ready, g.epoch + 1u)) X.ok = 0;
+            if (!wait_until(g, &g.ctl->ready, g.epoch + 1u)) X.ok = 0;
         }
         __syncwarp();
         const double *tot = totals_ptr(g, buf);

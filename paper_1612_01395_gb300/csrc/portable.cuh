@@ -7,6 +7,10 @@
 #define PBCG_HD inline
 #endif
 
+// Whether a counter that starts at 0 and wraps at 2^32 has reached `target`,
+// which is never 2^31 or more away from it.
+PBCG_HD bool reached(unsigned counter, unsigned target) { return (int)(counter - target) >= 0; }
+
 // Groups of g that n elements make, the last perhaps smaller (n + g - 1 may pass 2^31).
 PBCG_HD int groups_of(int n, int g) { return n / g + (n % g != 0); }
 

@@ -12,6 +12,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1612_01395_gb300", "csrc")
 SOURCE = r"""
 #include "portable.cuh"
+extern "C" int has_reached(unsigned counter, unsigned target) { return reached(counter, target); }
 extern "C" int groups(int n, int g) { return groups_of(n, g); }
 struct Dim { unsigned x; };
 static Dim blockIdx, blockDim, threadIdx, gridDim;
@@ -55,6 +56,14 @@ def test_groups_of_rows(lib, n, g):
     """Groups of a system or of an x-line; their first rows stay below 2^31."""
     assert lib.groups(n, g) == -(-n // g)
     assert (lib.groups(n, g) - 1) * g < 2 ** 31
+
+
+@pytest.mark.parametrize("target", [1, 152, 2 ** 31, 2 ** 32 - 1, 2 ** 32, 2 ** 32 + 151, 5 * 2 ** 32 + 7])
+def test_counter_of_arrivals_past_2_32(lib, target):
+    """Within the blocks of an exchange of its target, on both sides, at any lap."""
+    for d in (-2040, -1, 0, 1, 2040):
+        if target + d >= 0:
+            assert lib.has_reached(ctypes.c_uint((target + d) % 2 ** 32), ctypes.c_uint(target % 2 ** 32)) == (d >= 0)
 
 
 def test_kernels_step_through_elements_by_this_loop():
