@@ -71,15 +71,6 @@ PBCG_HD uint32_t wide_shl(uint32_t v, int s) {
     return s < 0 || s > 31 ? 0 : v << s;
 #endif
 }
-PBCG_HD uint64_t wide_bits(double v) {
-#ifdef __CUDA_ARCH__
-    return (uint64_t)__double_as_longlong(v);
-#else
-    uint64_t u;
-    memcpy(&u, &v, 8);
-    return u;
-#endif
-}
 PBCG_HD double wide_from_bits(uint64_t u) {
 #ifdef __CUDA_ARCH__
     return __longlong_as_double((long long)u);
@@ -213,7 +204,7 @@ struct WideParts {
 };
 PBCG_HD WideParts wide_parts(double v) {
     WideParts p;
-    const uint64_t u = wide_bits(v);
+    const uint64_t u = bits_of(v);
     p.hi = (uint32_t)(u >> 32);
     p.e = (int)((p.hi >> 20) & 0x7ffu);
     const uint64_t m = ((uint64_t)((p.hi & 0xfffffu) | 0x100000u) << 32 | (uint32_t)u) << 10;

@@ -742,7 +742,7 @@ extern "C" pbcg_status pbicgstab_solve_mixed(pbicgstab_t h, const void *d_val_lo
         a32.nxy = a64.nxy;
         a32.dx = a64.dx;
         a32.dy = a64.dy;
-        a32.gx = groups_of(a64.nx, 4);
+        a32.gx = pbcg::groups_of(a64.nx, 4);
         a32.dg.init((uint32_t)a32.gx);
         a32.aligned = a64.nx % 4 == 0;
         float *tab = f0 + 14 * s;

@@ -128,10 +128,6 @@ struct Row6 {
 // FP64 pipe, about 140 to its result): finite and zero from the bits, and the
 // order of non-negative numbers as the order of their bits.
 __device__ __forceinline__ bool is_finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
-__device__ __forceinline__ bool is_normal(double v) {
-    const int e = __double2hiint(v) & 0x7ff00000;
-    return e != 0 && e != 0x7ff00000;
-}
 __device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
 template <int K>
 __device__ __forceinline__ bool all_finite(const double (&v)[K]) {
@@ -199,7 +195,7 @@ __device__ __forceinline__ void omega_scalars(Scalars &S, double qy, double yy, 
     const double f = __ddiv_rn(lane == 0 ? qy : lane == 1 ? yy : S.alpha, lane == 0 ? yy : lane == 1 ? qy : S.rho);
     S.omega = __shfl_sync(kFull, f, 0);
     if (is_zero(S.omega)) return stop_scalars(S, PBCG_BREAKDOWN);
-    S.gain = __dmul_rn(__shfl_sync(kFull, f, 2), __shfl_sync(kFull, f, 1));
+    S.gain = beta_gain(__shfl_sync(kFull, f, 2), __shfl_sync(kFull, f, 1));
 }
 // Test of r_{i+1}; beta = (alpha / omega) (rho' / rho), by the gain where that
 // stayed in range, else by its two quotients on even and odd lanes.
@@ -209,7 +205,7 @@ __device__ __forceinline__ void beta_scalars(Scalars &S, double rho_n, double rr
     if (!finite) return stop_scalars(S, PBCG_NONFINITE);
     if (!fixed && norm_below(rr, S.tol, S.bound)) return stop_scalars(S, PBCG_OK);
     if (is_zero(rho_n)) return stop_scalars(S, PBCG_BREAKDOWN);
-    if (is_normal(S.gain)) {
+    if (!is_zero(S.gain)) {
         S.beta = __dmul_rn(S.gain, rho_n);
     } else {
         const bool odd = threadIdx.x & 1;

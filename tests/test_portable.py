@@ -1,17 +1,21 @@
-"""Index arithmetic of the kernels near 2^31 (csrc/portable.cuh), compiled for
-the host: sizes that the entry points accept, whose kernels are too large to
-run in a test."""
+"""Arithmetic of the kernels at the ends of its range (csrc/portable.cuh), compiled
+for the host: indices near 2^31, of sizes that the entry points accept and that
+are too large to run in a test, and scalars near the ends of the FP64 range."""
 import ctypes
 import glob
+import math
 import os
 import re
 import subprocess
+from fractions import Fraction
 
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1612_01395_gb300", "csrc")
 SOURCE = r"""
 #include "portable.cuh"
+using namespace pbcg;
+extern "C" double gain(double alpha_rho, double inv_omega) { return beta_gain(alpha_rho, inv_omega); }
 extern "C" int has_reached(unsigned counter, unsigned target) { return reached(counter, target); }
 extern "C" int groups(int n, int g) { return groups_of(n, g); }
 struct Dim { unsigned x; };
@@ -31,11 +35,13 @@ extern "C" int elements(unsigned grid, unsigned block, unsigned b, unsigned t, u
 
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
-    d = tmp_path_factory.mktemp("index")
-    src, so = d / "index.cpp", d / "index.so"
+    d = tmp_path_factory.mktemp("portable")
+    src, so = d / "portable.cpp", d / "portable.so"
     src.write_text(SOURCE)
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-o", str(so), str(src)])
-    return ctypes.CDLL(str(so))
+    lib = ctypes.CDLL(str(so))
+    lib.gain.argtypes, lib.gain.restype = [ctypes.c_double] * 2, ctypes.c_double
+    return lib
 
 
 @pytest.mark.parametrize("count", [0, 1, 1000, 46340 * 46340, 2 ** 31 - 1, 2 ** 31])
@@ -64,6 +70,21 @@ def test_counter_of_arrivals_past_2_32(lib, target):
     for d in (-2040, -1, 0, 1, 2040):
         if target + d >= 0:
             assert lib.has_reached(ctypes.c_uint((target + d) % 2 ** 32), ctypes.c_uint(target % 2 ** 32)) == (d >= 0)
+
+
+@pytest.mark.parametrize("rho,alpha,omega", [(3.7, 0.21, 0.7), (1.7e300, 0.3, 0.9), (1.3 * 2.0 ** 1021, 0.3, 0.01),
+                                             (1.7e300, 1.3e-12, 1e-6), (1.1e-300, 7e9, 1.7e-290),
+                                             (1.3e-5, 1.7 * 2.0 ** 40, 1.3 * 2.0 ** 1023), (1.0, 1e-200, 1e200)])
+def test_beta_by_one_product_is_as_exact_as_its_factors(lib, rho, alpha, omega):
+    """alpha, rho and omega stand for values known exactly. Four roundings of 2^-53 (two
+    quotients, two products) where the short form is used; 0 asks for the long one."""
+    g = lib.gain(alpha / rho, 1.0 / omega)
+    rho_next = 0.77 * rho
+    exact = Fraction(alpha) / Fraction(rho) / Fraction(omega) * Fraction(rho_next)
+    if g != 0.0:
+        assert abs(Fraction(g * rho_next) - exact) <= 4.5 * exact / 2 ** 53
+    else:
+        assert any(not 2.0 ** -1022 <= v < math.inf for v in (alpha / rho, 1.0 / omega, alpha / rho * (1.0 / omega)))
 
 
 def test_kernels_step_through_elements_by_this_loop():
