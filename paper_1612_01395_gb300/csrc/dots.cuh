@@ -213,6 +213,21 @@ PBCG_HD WideParts wide_parts(double v) {
     return p;
 }
 
+// The parts of a zero (exponent kWideAbsent) or subnormal value.
+PBCG_HD void wide_subnormal(double v, WideParts &p) {
+    const uint64_t f = bits_of(v) & 0xfffffffffffffull;
+    if (f == 0) {
+        p.e = kWideAbsent;
+        return;
+    }
+    const uint32_t hi = (uint32_t)(f >> 32);
+    const int z = hi ? wide_clz(hi) : 32 + wide_clz((uint32_t)f);
+    const uint64_t m = f << (z - 1);   // the leading bit to bit 62; that of a normal number of exponent e is 2^(e - 1023)
+    p.e = 12 - z;
+    p.mh = (uint32_t)(m >> 32);
+    p.ml = (uint32_t)m;
+}
+
 // Add the product of a and b (square: a times itself) to c; its exponent is `distance` below the reference.
 PBCG_HD void wide_add(WideSlot &c, const WideParts &a, const WideParts &b, bool square, int distance) {
     const uint32_t mid = square ? 2u * wide_mulhi(a.mh, a.ml) : wide_mulhi(a.mh, b.ml) + wide_mulhi(a.ml, b.mh);
@@ -278,7 +293,8 @@ struct WideDots {
         }
     }
 
-    // Zero and subnormal values vanish; infinite and NaN ones are noted and vanish.
+    // Zeros vanish; infinite and NaN values are noted and vanish; subnormal ones get their
+    // leading bit in place and the exponent that goes with it.
     PBCG_HD void unusual(const double (&v)[P::nv], WideParts (&p)[P::nv], int emax) {
         if (emax == 2047) {
 #pragma unroll
@@ -289,8 +305,10 @@ struct WideDots {
                 }
         }
 #pragma unroll
-        for (int j = 0; j < P::nv; ++j)
-            if (p[j].e == 0 || p[j].e == 2047) p[j].e = kWideAbsent;
+        for (int j = 0; j < P::nv; ++j) {
+            if (p[j].e == 0) wide_subnormal(v[j], p[j]);
+            else if (p[j].e == 2047) p[j].e = kWideAbsent;
+        }
     }
 
     // Exponent of product k of a row.

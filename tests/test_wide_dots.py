@@ -171,3 +171,17 @@ def test_lanes_of_a_warp_with_one_outlier(lib, rows, outlier, square):
     bound = 2 * len(p) * max(map(abs, p)) * scale / 2 ** 73 + 3 * sum(map(abs, p)) * scale / 2 ** 60
     bound += sum(map(abs, lane)) / 2 ** 53
     assert abs(sum(Fraction(float(o)) for o in out) - sum(lane)) <= bound
+
+
+@pytest.mark.parametrize("small", [3e-309, 1e-315, 4e-323])
+@pytest.mark.parametrize("n", [1, 3, 200])
+def test_subnormal_values(lib, n, small):
+    """A subnormal value keeps its bits next to one that brings the product into range;
+    bound of the sums above."""
+    g = np.random.default_rng(n)
+    v = g.standard_normal((n, 2)) * [small, 1e300]
+    v[n // 2, 0] = np.sign(v[n // 2, 0]) * 5e-324
+    p = [Fraction(float(x)) * Fraction(float(y)) for x, y in v]
+    exact = sum(p)
+    bound = 5 * n * Fraction(1, 2 ** 54) * max(map(abs, p)) + Fraction(1, 2 ** 53) * abs(exact)
+    assert abs(Fraction(float(sums(lib, "one", v)[0])) - exact) <= bound
