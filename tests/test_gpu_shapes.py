@@ -169,6 +169,34 @@ def test_fp32_groups_drop_the_entries_outside_the_grid(dims, bad):
     assert out[True][1] == out[False][1]
 
 
+@pytest.mark.parametrize("dims", [(1, 9, 3), (1, 64, 50), (1, 1, 37), (1, 30, 1), (1, 203, 301)])
+def test_fp32_sweeps_of_x_lines_of_one_node(dims):
+    """The same system, bit for bit, as on the grid without that axis."""
+    out = []
+    for drop in range(2 if dims[1] > 1 else 3):
+        nx, ny, nz = (dims + (1, 1))[drop:drop + 3]
+        along = {1: (0, 1, 0), 2: (0, 0, 1)}   # the strides of the first grid's axes y and z
+        move = lambda st: (st + (0, 0))[drop:drop + 3]   # noqa: E731
+        coefs = [P.Coef(value=0.0) for _ in range(7)]
+        coefs[P.C] = P.Coef(table=6.3 + 0.01 * np.arange(dims[1]), stride=move(along[1]),
+                            table2=0.02 * np.arange(dims[2]), stride2=move(along[2]))
+        back = P.Coef(table=-1.0 - 0.001 * np.arange(dims[1]), stride=move(along[1]))
+        pairs = [(P.W, P.E), (P.S, P.N), (P.B, P.T)]
+        for axis, (lo, hi) in enumerate([(back, P.Coef(value=-0.9)), (P.Coef(value=-1.05), P.Coef(value=-0.95))]):
+            to = axis + 1 - drop
+            if to >= 0:
+                coefs[pairs[to][0]], coefs[pairs[to][1]] = lo, hi
+        st = P.Stencil(nx=nx, ny=ny, nz=nz, coefs=coefs)
+        s = native.Solver.from_stencil(st)
+        x, info = s.solve_mixed(dev(P.splitmix64_uniform(4, st.n)), None, rtol=1e-12, inner_rtol=1e-3)
+        assert info["status"] == native.PBCG_OK
+        out.append((x.cpu().numpy(), info["inner_iters"]))
+        s.close()
+    for x, iters in out[1:]:
+        np.testing.assert_array_equal(x, out[0][0])
+        assert iters == out[0][1]
+
+
 @pytest.mark.parametrize("n", [0, 1, 4094, 4095, 4096, 12289])
 def test_transpose_row_pointers_at_the_tiles_of_the_scan(n):
     import torch
