@@ -674,13 +674,15 @@ void drop_x_axis(pbcg::StencilOpT<float, false> &o) {
 }
 
 template <class Op64, class Op32>
-pbcg_status launch_mixed(pbicgstab_s *h, const Op64 &a64, const Op32 &a32, const pbcg::MixedArgs &m, int req_grid,
+pbcg_status launch_mixed(pbicgstab_s *h, const Op64 &a64, const Op32 &a32, pbcg::MixedArgs m, int req_grid,
                          int *grid_out) {
     // Blocks per SM by rows, as for the grid solvers (an exchange costs more
     // blocks more; us per FP32 iteration, stencil / CSR, at 1 and 2 blocks of
     // 256 per SM: 110k rows 19.8 / 20.5 and 24.4 / 23.9; 262k 25.1 / 27.5 and
-    // 26.6 / 28.4; 512k 36.8 / 43.1 and 32.2 / 36.6). A forced grid takes
-    // smaller blocks where the larger ones are not all resident.
+    // 26.6 / 28.4; 512k 36.8 / 43.1 and 32.2 / 36.6; rows of 21 random entries,
+    // FP32: 50k 27.8 and 30.6, 100k 44.7 and 42.2, 200k 67.9 and 67.4, 300k 92.8
+    // and 89.6, 500k 171.2 and 149.9, 1M at 2 and 4 per SM 284 and 298). A forced
+    // grid takes smaller blocks where the larger ones are not all resident.
     int block = pbcg::kMixedTPB, occ = 0, grid = req_grid;
     for (;; block /= 2) {
         PBCG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pbcg::mixed_kernel<Op64, Op32>, block, 0));
@@ -696,6 +698,11 @@ pbcg_status launch_mixed(pbicgstab_s *h, const Op64 &a64, const Op32 &a32, const
     }
     if (grid > all) grid = all;
     if (grid > pbcg::kMaxGrid) grid = pbcg::kMaxGrid;
+    // Long rows, and the rows of a forced grid, are dealt to all blocks alike: in
+    // whole blocks of rows, those of the last round kept the others waiting (and
+    // the polls of waiting blocks seem to slow the busy ones of their SM): 100k rows of 21 entries 49.8 -> 44.7 us an FP32 iteration,
+    // 500k 166 -> 150, 1M 294 -> 284; 20k on 608 blocks 73.0 -> 31.4.
+    m.dealt = req_grid > 0 || h->nnz > kLongRow * h->n;
     *grid_out = grid;
     PBCG_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(pbcg::Control), h->stream));
     if (h->ev0) PBCG_CUDA(cudaEventRecord(h->ev0, h->stream));

@@ -72,8 +72,8 @@ struct SolverBlock {
 // blockDim.x rows in a row per block, us per iteration of Algorithm 9: 48^3
 // 22.2 -> 21.4, 96^3 74.7 -> 72.4, 256^3 CSR 1088 -> 1047, 200k random rows
 // 91.1 -> 82.1; FP32 stencil iterations of 64^3 26.0 -> 25.0, 110^3 68.0 ->
-// 58.7. The FP32 CSR sweeps lost 2 to 3 % (193x160x131 184 -> 190) and keep
-// whole blocks of rows.
+// 58.7. The FP32 CSR sweeps of 7-point rows lost 2 to 3 % (193x160x131 184 ->
+// 190) and keep whole blocks of rows.
 __device__ __forceinline__ int grid_lo() {
     return (int)(((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32u + (threadIdx.x & 31u)) - (int)threadIdx.x;
 }
@@ -1126,6 +1126,7 @@ struct MixedArgs {
     double inner_rtol;
     int inner_maxit;
     int inner_fixed;     // > 0: every inner solve runs exactly this many iterations
+    int dealt;           // CSR: rows in runs of 32 to all blocks in turn (grid_lo)
     int stall_steps;     // steps in a row without a new best residual that stop the loop
 };
 
@@ -1140,7 +1141,7 @@ __global__ void __launch_bounds__(kMixedTPB, 4)
     __shared__ Exchange<kMixedTPB> X;
     if (threadIdx.x == 0) X.ok = 1;   // read only after the first exchange's barrier
     GridSync g{m.ctl, m.partials, 0u, 0, (int)(gridDim.x * blockDim.x)};
-    const int lo = HasGroups<Op32>::value ? grid_lo() : (int)(blockIdx.x * blockDim.x), hi = m.n;
+    const int lo = HasGroups<Op32>::value || m.dealt ? grid_lo() : (int)(blockIdx.x * blockDim.x), hi = m.n;
     int outer = 0, inner_total = 0, status = PBCG_NOT_CONVERGED, spmvs = 0, stalls = 0;
     double nr0 = 0.0, tol = 0.0, bound = 0.0, last = 0.0;
     double best = 0.0;        // smallest squared FP64 residual so far (valid when have_best)

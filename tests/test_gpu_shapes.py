@@ -197,6 +197,25 @@ def test_fp32_sweeps_of_x_lines_of_one_node(dims):
         assert iters == out[0][1]
 
 
+@pytest.mark.parametrize("values", ["f32", "bf16"])
+@pytest.mark.parametrize("n", [2, 33, 64, 257, 5001, 90001])
+def test_fp32_sweeps_of_long_rows(n, values):
+    """Rows dealt to the blocks in runs: odd numbers of pairs, blocks without a row, several rounds."""
+    import torch
+    A = P.random_sparse(n, seed=n, nnz_lo=min(9, n), nnz_hi=min(21, n))
+    b = oracle.spmv(A, P.splitmix64_uniform(2, n))
+    s = native.Solver.from_csr(A)
+    low = torch.from_numpy(A.val).cuda().to(torch.float32 if values == "f32" else torch.bfloat16)
+    kind = native.PBCG_VALUES_F32 if values == "f32" else native.PBCG_VALUES_BF16
+    for grid in (0, 3, 608):
+        solve = lambda: s.solve_mixed(dev(b), low, lowp_type=kind, rtol=1e-12, inner_rtol=1e-2, grid=grid)   # noqa: E731
+        x, info = solve()
+        assert info["status"] == native.PBCG_OK
+        assert np.linalg.norm(b - oracle.spmv(A, x.cpu().numpy())) <= 1e-11 * np.linalg.norm(b)
+        np.testing.assert_array_equal(x.cpu().numpy(), solve()[0].cpu().numpy())
+    s.close()
+
+
 @pytest.mark.parametrize("n", [0, 1, 4094, 4095, 4096, 12289])
 def test_transpose_row_pointers_at_the_tiles_of_the_scan(n):
     import torch
