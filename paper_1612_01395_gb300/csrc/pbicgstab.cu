@@ -257,6 +257,14 @@ pbcg_status launch_solver(pbicgstab_s *h, const Op &op, bool pipelined, const pb
 // throughput decides; the bound is kept where the interface states it.
 constexpr long long kClusterMaxEntries = 24576;
 
+// Stencil SpMVs of up to this many rows load a row's values where they are
+// used, larger ones ahead of the sum. While x and y stay in L2 (129 MB) the
+// loads are short and the extra registers cost more. Loads in place / ahead, us
+// back to back: 128^3 33.6 / 35.1, 160^3 61.7 / 65.8, 500x500x20 76.3 / 79.7,
+// 176^3 87.2 / 86.5, 192^3 110.7 / 111.6, 208^3 147 / 140, 256^3 295 / 246; 1024^2
+// 15.5 / 16.6, 2048^2 49.4 / 51.4, 4096^2 219 / 191.
+constexpr int kLeanRows = 5000000;
+
 // The launch of a cluster kernel: `size` CTAs of one cluster.
 struct ClusterLaunch {
     cudaLaunchConfig_t cfg = {};
@@ -622,7 +630,7 @@ pbcg_status pbicgstab_spmv(pbicgstab_t h, const double *d_x, double *d_y) {
         pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(chunked(h->csr), d_x, d_y);
     else if (h->kind == 0)
         pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(h->csr, d_x, d_y);
-    else if (h->st.nz == 1)   // loads ahead: 1024^2 16.8 against 15.4 us, 256^3 249 against 291
+    else if (h->n <= kLeanRows)
         pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(lean(h->st), d_x, d_y);
     else
         pbcg::spmv_kernel<<<blocks, pbcg::kTPB, 0, h->stream>>>(h->st, d_x, d_y);

@@ -216,6 +216,17 @@ def test_fp32_sweeps_of_long_rows(n, values):
     s.close()
 
 
+@pytest.mark.parametrize("dims", [(3, 2, 1), (37, 41, 5), (2500, 2000, 1), (2501, 2000, 1), (171, 171, 171)])
+def test_stencil_spmv_on_both_sides_of_its_line(dims):
+    """5,000,000 rows (the last with loads in place), 5,002,000 and 5,000,211: the bits of the assembled matrix."""
+    st = grid_stencil(*dims)
+    x = dev(P.splitmix64_uniform(5, st.n))
+    s, c = native.Solver.from_stencil(st), native.Solver.from_csr(P.stencil_to_csr(st))
+    np.testing.assert_array_equal(s.spmv(x).cpu().numpy(), c.spmv(x).cpu().numpy())
+    s.close()
+    c.close()
+
+
 @pytest.mark.parametrize("n", [0, 1, 4094, 4095, 4096, 12289])
 def test_transpose_row_pointers_at_the_tiles_of_the_scan(n):
     import torch
