@@ -300,18 +300,24 @@ bool cluster_fits(const void *fn, int size, int block, size_t bytes) {
     return clusters >= 1;
 }
 
-// Largest clusters (16, else 8, else none) of the two cluster solvers.
+// Largest clusters (16, else 8, else none) of the two cluster solvers. A CTA of
+// cluster_solve_kernel needs less of an SM than one of onchip_solve_kernel, so
+// what holds a cluster of the latter holds one of the former; each query takes
+// about 2 us of a handle's 60.
 template <class Op>
 void cluster_limits(pbicgstab_s *h) {
     h->cluster_max = h->onchip_max = 0;
     for (int size = 16; size >= 8; size /= 2) {
-        if (!h->cluster_max && cluster_fits((const void *)pbcg::cluster_solve_kernel<Op, true>, size, pbcg::kTPB, 0) &&
-            cluster_fits((const void *)pbcg::cluster_solve_kernel<Op, false>, size, pbcg::kTPB, 0))
-            h->cluster_max = size;
         if (!h->onchip_max &&
             cluster_fits((const void *)pbcg::onchip_solve_kernel<Op, true>, size, pbcg::kOnChipTPB, pbcg::kOnChipMaxBytes) &&
             cluster_fits((const void *)pbcg::onchip_solve_kernel<Op, false>, size, pbcg::kOnChipTPB, pbcg::kOnChipMaxBytes))
             h->onchip_max = size;
+        if (!h->cluster_max &&
+            (h->onchip_max == size ||
+             (cluster_fits((const void *)pbcg::cluster_solve_kernel<Op, true>, size, pbcg::kTPB, 0) &&
+              cluster_fits((const void *)pbcg::cluster_solve_kernel<Op, false>, size, pbcg::kTPB, 0))))
+            h->cluster_max = size;
+        if (h->cluster_max && h->onchip_max) return;
     }
 }
 
@@ -345,6 +351,9 @@ pbcg_status launch_cluster(pbicgstab_s *h, const Op &op, bool pipelined, const p
         return PBCG_OK;
     }
     *block = pbcg::kTPB;
+    const void *fn = pipelined ? (const void *)pbcg::cluster_solve_kernel<Op, true>
+                               : (const void *)pbcg::cluster_solve_kernel<Op, false>;
+    if (size > 8) PBCG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     ClusterLaunch l(size, *block, 0, h->stream);
     if (pipelined)
         PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::cluster_solve_kernel<Op, true>, op, args));
