@@ -1100,12 +1100,17 @@ extern "C" pbcg_status pbicgstab_csr_transpose(int32_t n, int32_t nnz, const int
     const int blocks = 4 * sms;
     PBCG_CUDA(cudaMemsetAsync(d_trowptr, 0, (size_t)(n + 1) * sizeof(int), st));
     if (nnz > 0) pbcg::transpose_count_kernel<<<blocks, 256, 0, st>>>(nnz, d_col, d_trowptr);
-    // the tile sums live in the cursors' array, which is cleared after the scan
+    // The tile sums live in the cursors' array, which is cleared after the scan; a single tile has
+    // the sum 0 before it (two launches less: n = 100, 60.5 -> 53.9 us).
     const int m = n + 1, tiles = (int)(((long long)m + pbcg::kScanTile - 1) / pbcg::kScanTile);
-    pbcg::scan_tiles_kernel<<<tiles, pbcg::kScanThreads, 0, st>>>(m, d_trowptr, cursor);
-    pbcg::scan_sums_kernel<<<1, pbcg::kScanThreads, 0, st>>>(tiles, cursor);
+    if (tiles > 1) {
+        pbcg::scan_tiles_kernel<<<tiles, pbcg::kScanThreads, 0, st>>>(m, d_trowptr, cursor);
+        pbcg::scan_sums_kernel<<<1, pbcg::kScanThreads, 0, st>>>(tiles, cursor);
+    } else {
+        PBCG_CUDA(cudaMemsetAsync(cursor, 0, (size_t)m * sizeof(int), st));
+    }
     pbcg::scan_apply_kernel<<<tiles, pbcg::kScanThreads, 0, st>>>(m, d_trowptr, cursor);
-    PBCG_CUDA(cudaMemsetAsync(cursor, 0, (size_t)(n + 1) * sizeof(int), st));
+    if (tiles > 1) PBCG_CUDA(cudaMemsetAsync(cursor, 0, (size_t)m * sizeof(int), st));
     if (n > 0) {
         pbcg::transpose_scatter_kernel<<<blocks, 256, 0, st>>>(n, d_rowptr, d_col, d_val, d_trowptr, cursor, d_tcol,
                                                                d_tval);
