@@ -5,7 +5,8 @@ CSR operator forms), both methods, the Jacobi-preconditioned methods
 (Algorithms 10 and 11), the mixed-precision solve (stencil with even and odd
 nx, CSR with FP32 and BF16 values), the SpMV entry point, the
 allocation-free entry point, the adjoint transpose and value gradient, and a
-small batch. No index may be reported out of range, and
+small batch; and, in a test of their own, the kernels that take over above a
+size. No index may be reported out of range, and
 the results must equal the default build's bit for bit: the checks only guard
 indices, they change no arithmetic.
 """
@@ -105,6 +106,57 @@ def test_checked_build_reports_no_fault_and_matches_default(libs):
     use(checked)
     assert native.pbicgstab_check_faults() == 0
     got = run_all()
+    assert native.pbicgstab_check_faults() == 0
+    use(default)
+    for key, x in ref.items():
+        assert np.all(np.isfinite(x)), key
+        np.testing.assert_array_equal(got[key], x, err_msg=str(key))
+
+
+def run_above_the_lines():
+    """Kernels that take over above a size: the wide sums (plain and Jacobi, both
+    forms and methods, with replacement), SpMV with loads ahead, rows dealt to
+    the blocks, x-lines of one node."""
+    import torch
+    out = {}
+    st = P.cd3d_trig(90)
+    A = P.stencil_to_csr(st)
+    b = torch.from_numpy(P.splitmix64_uniform(3, A.n)).cuda()
+    for prec in (native.PBCG_PREC_NONE, native.PBCG_PREC_JACOBI):
+        for form in ("stencil", "csr"):
+            s = native.Solver.from_stencil(st, prec=prec) if form == "stencil" else native.Solver.from_csr(A, prec=prec)
+            for method in ("pipelined", "standard"):
+                x, info = s.solve(b, rtol=0.0, maxit=6, fixed_iters=6, replace_period=4, method=method)
+                assert info["block"] == 512
+                out[(prec, form, method)] = x.cpu().numpy()
+            s.close()
+    st = P.cd2d_constant(2300, (10.0, 4.0))
+    s = native.Solver.from_stencil(st)
+    out["spmv"] = s.spmv(torch.from_numpy(P.splitmix64_uniform(3, st.n)).cuda()).cpu().numpy()
+    s.close()
+    R = P.random_sparse(3001, seed=5)
+    s = native.Solver.from_csr(R)
+    b = torch.from_numpy(P.splitmix64_uniform(1, R.n)).cuda()
+    v32 = torch.from_numpy(R.val).cuda().to(torch.float32)
+    out["mixed_long_rows"] = s.solve_mixed(b, v32, rtol=1e-10, inner_rtol=1e-3)[0].cpu().numpy()
+    s.close()
+    st = P.constant_stencil_2d(37, 4.5, -1.1, -0.9, -1.2, -0.8)
+    line = P.Stencil(nx=1, ny=37, nz=37, coefs=[st.coefs[P.C], P.Coef(), P.Coef(), st.coefs[P.W], st.coefs[P.E],
+                                                st.coefs[P.S], st.coefs[P.N]])
+    s = native.Solver.from_stencil(line)
+    b = torch.from_numpy(P.splitmix64_uniform(1, line.n)).cuda()
+    out["mixed_one_node"] = s.solve_mixed(b, None, rtol=1e-10, inner_rtol=1e-3)[0].cpu().numpy()
+    s.close()
+    return out
+
+
+def test_checked_build_above_the_lines(libs):
+    default, checked = libs
+    use(default)
+    ref = run_above_the_lines()
+    use(checked)
+    native.pbicgstab_check_faults()
+    got = run_above_the_lines()
     assert native.pbicgstab_check_faults() == 0
     use(default)
     for key, x in ref.items():

@@ -115,6 +115,49 @@ def test_wide_sums_above_their_line(dims, form, method):
     s.close()
 
 
+@pytest.fixture(scope="module")
+def wide_reference():
+    """The oracle's first iterations on a system of `dims`, once per method and options."""
+    done = {}
+
+    def get(dims, method, prec, replace):
+        st = grid_stencil(*dims)
+        if dims not in done:
+            A = P.stencil_to_csr(st)
+            x = P.splitmix64_uniform(3, A.n)
+            x[: A.n // 2] = 0.0
+            done[dims] = A, oracle.spmv(A, x)
+        A, b = done[dims]
+        key = dims, method, prec, replace
+        if key not in done:
+            args = dict(rtol=0.0, maxit=K, fixed_iters=K)
+            if method == "pipelined":
+                args["replace_period"] = replace
+            run = getattr(oracle, ("p" if method == "pipelined" else "") + "bicgstab" + ("_prec" if prec else ""))
+            done[key] = run(A, oracle.jacobi_minv(A), b, **args) if prec else run(A, b, **args)
+        return st, A, b, done[key]
+    return get
+
+
+@pytest.mark.parametrize("method,replace", [("pipelined", 0), ("pipelined", 4), ("standard", 0)])
+@pytest.mark.parametrize("prec", [native.PBCG_PREC_JACOBI, native.PBCG_PREC_NONE])
+@pytest.mark.parametrize("form", ["csr", "stencil"])
+@pytest.mark.parametrize("dims", [(83, 89, 95), (839, 837, 1)])
+def test_wide_sums_of_preconditioned_and_replaced_iterations(wide_reference, dims, form, prec, method, replace):
+    """Algorithms 10 and 11, and residual replacement, with the dot products in integers.
+    The Jacobi 2-D system falls by 12 orders in these iterations, where the two methods'
+    oracles differ by 1e-4 of the last norms: besides 1e-8 of itself, a norm may differ by
+    1e-13 of the first, a few hundred roundings of vectors of that size."""
+    st, A, b, ref = wide_reference(dims, method, prec, replace)
+    s = native.Solver.from_csr(A, prec=prec) if form == "csr" else native.Solver.from_stencil(st, prec=prec)
+    x, info, hist = s.solve(dev(b), rtol=0.0, maxit=K, fixed_iters=K, method=method, replace_period=replace, history=True)
+    assert info["block"] == 512 and info["n_replacements"] == (K // replace if replace else 0)
+    h = hist.cpu().numpy()
+    assert np.all(np.abs(h - ref.hist[:K + 1]) <= 1e-8 * ref.hist[:K + 1] + 1e-13 * ref.hist[0])
+    assert np.linalg.norm(x.cpu().numpy() - ref.x) <= 1e-9 * np.linalg.norm(ref.x)
+    s.close()
+
+
 def test_wide_sums_report_non_finite_values():
     st = grid_stencil(100, 100, 71)
     s = native.Solver.from_stencil(st)
