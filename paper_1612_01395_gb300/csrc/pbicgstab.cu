@@ -5,6 +5,8 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <type_traits>
+#include <utility>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -60,6 +62,14 @@ pbcg::StencilOpLean lean(const pbcg::StencilOp &a) {
     return o;
 }
 pbcg::CsrOpShort shortrows(const pbcg::CsrOpScalar &a) { return pbcg::CsrOpShort{a.n, a.rowptr, a.col, a.val, a.nnz}; }
+// The operator that the on-chip solver takes its entries from: one form of CSR, as it reads the arrays alone.
+template <class Op>
+const Op &onchip_source(const Op &a) { return a; }
+pbcg::CsrOpScalar onchip_source(const pbcg::CsrOpChunked &a) {
+    return pbcg::CsrOpScalar{a.n, a.rowptr, a.col, a.val, a.nnz};
+}
+template <class Op>
+using OnChipSource = std::decay_t<decltype(onchip_source(std::declval<const Op &>()))>;
 pbcg::CsrOpChunked chunked(const pbcg::CsrOpScalar &a) { return pbcg::CsrOpChunked{a.n, a.rowptr, a.col, a.val, a.nnz}; }
 
 }  // namespace
@@ -306,11 +316,12 @@ bool cluster_fits(const void *fn, int size, int block, size_t bytes) {
 // about 2 us of a handle's 60.
 template <class Op>
 void cluster_limits(pbicgstab_s *h) {
+    using Src = OnChipSource<Op>;
     h->cluster_max = h->onchip_max = 0;
     for (int size = 16; size >= 8; size /= 2) {
         if (!h->onchip_max &&
-            cluster_fits((const void *)pbcg::onchip_solve_kernel<Op, true>, size, pbcg::kOnChipTPB, pbcg::kOnChipMaxBytes) &&
-            cluster_fits((const void *)pbcg::onchip_solve_kernel<Op, false>, size, pbcg::kOnChipTPB, pbcg::kOnChipMaxBytes))
+            cluster_fits((const void *)pbcg::onchip_solve_kernel<Src, true>, size, pbcg::kOnChipTPB, pbcg::kOnChipMaxBytes) &&
+            cluster_fits((const void *)pbcg::onchip_solve_kernel<Src, false>, size, pbcg::kOnChipTPB, pbcg::kOnChipMaxBytes))
             h->onchip_max = size;
         if (!h->cluster_max &&
             (h->onchip_max == size ||
@@ -333,6 +344,7 @@ int onchip_cap(const pbicgstab_s *h, int size, int m) {
 template <class Op>
 pbcg_status launch_cluster(pbicgstab_s *h, const Op &op, bool pipelined, const pbcg::SolveArgs &args, int size,
                            bool any_variant, int *block) {
+    using Src = OnChipSource<Op>;
     const int m = (int)(((long long)h->n + size - 1) / size), cap = onchip_cap(h, size, m);
     const size_t bytes = pbcg::onchip_bytes(m, cap);
     if (size <= h->onchip_max && bytes <= pbcg::kOnChipMaxBytes) {
@@ -345,9 +357,9 @@ pbcg_status launch_cluster(pbicgstab_s *h, const Op &op, bool pipelined, const p
         if (any_variant) a.variant = 5;
         ClusterLaunch l(size, *block, bytes, h->stream);
         if (pipelined)
-            PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::onchip_solve_kernel<Op, true>, op, a, m, dm, cap));
+            PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::onchip_solve_kernel<Src, true>, onchip_source(op), a, m, dm, cap));
         else
-            PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::onchip_solve_kernel<Op, false>, op, a, m, dm, cap));
+            PBCG_CUDA(cudaLaunchKernelEx(&l.cfg, pbcg::onchip_solve_kernel<Src, false>, onchip_source(op), a, m, dm, cap));
         return PBCG_OK;
     }
     *block = pbcg::kTPB;
