@@ -42,8 +42,8 @@ __device__ __forceinline__ int block_scan(int v, int *warps) {
 }
 
 // In-place inclusive prefix sum of a[0..m) in tiles of 4096 elements, which turns
-// counts into row pointers. Three passes: the sum of each tile (kSums), the
-// tile sums scanned by one block, and each tile scanned from its offset. One
+// counts into row pointers. Three passes: the sum of each tile, the tile sums
+// scanned by one block, and each tile scanned from its offset. One
 // block walking 1024 uncoalesced chunks took 787 us for 1M counts; these take
 // about 10.
 constexpr int kScanTile = 4096, kScanThreads = 1024;

@@ -292,7 +292,7 @@ __device__ __forceinline__ bool wait_until(GridSync &g, const unsigned *word, un
 // Barrier without data.
 template <int T>
 __device__ __forceinline__ bool grid_sync(GridSync &g, Exchange<T> &X) {
-    __syncthreads();   // every thread's stores of this phase precede thread 0's fence
+    __syncthreads();   // every thread's stores of this phase precede thread 0's arrival
     if (threadIdx.x == 0) {
         red_release_inc(&g.ctl->arrivals);
         if (!wait_until(g, &g.ctl->arrivals, (g.epoch + 1u) * gridDim.x)) X.ok = 0;
@@ -355,7 +355,7 @@ __device__ __forceinline__ bool exchange(GridSync &g, double (&v)[K], Exchange<T
     if (!by_last) {
         sum_slots(g, buf, v, X);
         if (wid == 0) f(X.s, v);
-    } else if (X.last) {   // every slot is visible: all blocks fenced before arriving
+    } else if (X.last) {   // every slot is visible: all blocks arrived with release
         sum_slots(g, buf, v, X);
         if (wid == 0) {
             f(X.s, v);
@@ -441,11 +441,6 @@ __device__ __forceinline__ uint32_t cluster_map(const void *p, unsigned rank) {
 }
 __device__ __forceinline__ void st_cluster_f64(uint32_t addr, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
-}
-__device__ __forceinline__ double ld_cluster_f64(uint32_t addr) {
-    double v;
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
-    return v;
 }
 __device__ __forceinline__ void st_cluster_s32(uint32_t addr, int v) {
     asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");

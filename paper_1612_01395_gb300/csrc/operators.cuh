@@ -202,8 +202,9 @@ struct StencilOpT {
     // whose chain (about 140 cycles a step, and a loop per second table that
     // loads are not moved across) would otherwise wait for one load after
     // another. Algorithm 9 per iteration: 32^3 18.9 -> 16.6 us, 48^3 29.4 ->
-    // 27.0, 128^3 179 -> 174. The mixed-precision kernel, with 56 registers for
-    // its FP32 sweeps, spills more with it and loads one neighbour at a time.
+    // 27.0, 128^3 179 -> 174. The mixed-precision kernel, with 64 registers for
+    // its FP32 sweeps, spills more with it and loads one neighbour at a time, as
+    // does the SpMV of systems that stay in L2.
     template <class L>
     __device__ __forceinline__ auto row(int r, const L &u) const -> decltype(u(0)) {
         using T = decltype(u(0));
@@ -336,7 +337,7 @@ struct StencilOpT {
     }
 };
 using StencilOp = StencilOpT<double>;
-using StencilOpLean = StencilOpT<double, false>;   // mixed-precision kernel, FP64 residual
+using StencilOpLean = StencilOpT<double, false>;   // FP64 residual of the mixed-precision kernel, SpMV in L2
 
 // Operators whose fused sweeps load their vectors through L2 only.
 template <class Op>

@@ -214,10 +214,13 @@ long long max_index(const int64_t st[3], int nx, int ny, int nz) {
 //    490k, 5 entries       54 / 53     45 / 44     43 / 42
 //    885k, 7 points        84 / 79     75 / 67     69 / 62
 //    1.05M, 5 entries      174 / 161   108 / 102   81 / 75
-// Long rows (21 random entries) are bound by their gathers, which the wide
-// sums do not shorten and their shared memory takes L1 from: 200k 91 / 90 at 2
-// x 256 against 126 / 128, 500k 212 / 208 against 264 / 251. Systems of less
-// than a 128-row block per SM take blocks of 128, to use more SMs.
+// Long rows (21 random entries, Jacobi) are bound by their gathers, which the
+// wide sums do not shorten and their shared memory takes L1 from: 200k 82 / 80
+// at 2 x 256 against 93 / 93 wide, 500k 209 / 195 against 230 / 216, 1M 357 / 346
+// at 4 x 256 against 409 / 388. Above 700k rows they take all resident blocks:
+// 4 x 256 against 2 x 256, 700k 262 / 258 and 272 / 253, 1M 357 / 346 and 378 /
+// 349. Systems of less than a 128-row block per SM take blocks of 128, to use
+// more SMs. The wide kernel's sums have room for kWideThreadRows rows a thread.
 constexpr long long kOneBlockRows = 180000, kWideRows = 700000, kLongRow = 8;
 struct Shape {
     bool wide;

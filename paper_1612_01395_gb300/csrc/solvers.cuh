@@ -421,9 +421,10 @@ __device__ __forceinline__ void group_product(const Op &A, int gi, int hi, const
 // i-1; s := A p, z := A s after p_i; for i mod k == 0).
 // ===========================================================================
 // T is the vector and sweep arithmetic type: double for the FP64 solver,
-// float for the inner solves of the mixed-precision refinement. Dot products
-// are summed per thread in T (DotAccFor) and across threads in double, and
-// alpha, beta, omega, rho are doubles; a sweep uses them rounded to T.
+// float for the inner solves of the mixed-precision refinement. The dot
+// products of a thread's rows are summed by DotsFor (FP64 FMAs, compensated
+// FP32, or the integers of a Wide kernel) and those of the threads in double;
+// alpha, beta, omega, rho are doubles, and a sweep uses them rounded to T.
 template <class Op, typename T, int B, class Sync = GridSync, bool Wide = false>
 __device__ __forceinline__ bool pipelined_loop(const Op &A, const SolveArgsT<T> &a, Sync &g, Exchange<B> &X,
                                                int lo, int hi, Outcome &o, int &spmvs, WideSlot *wide) {
