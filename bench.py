@@ -121,6 +121,13 @@ def flops_per_launch(n, info):
     return info["spmvs"] * 2.0 * nnz_of(n) + info["iters"] * 2.0 * (13 + 8) * N
 
 
+def integer_pipe_flops(n, info):
+    """The part of flops_per_launch that the kernel does not run on the FP64
+    pipe: with blocks of 512 threads the 8 dot products of an iteration are
+    summed in integers."""
+    return info["iters"] * 2.0 * 8 * n ** 3 if info["block"] == 512 else 0.0
+
+
 def batched_flops(sizes, nnz, iters, n_repl):
     """Algorithmic FP64 flops of one batched launch. Per system: 2 flops per
     stored entry per SpMV (r_0 = b - A x_0 and w_0 = A r_0, two per iteration,
@@ -749,7 +756,8 @@ def run_ours(args):
     # roofline of the solver kernel (one cooperative launch per solve)
     kern_s = main["kernel_ms"] / 1e3
     fl = flops_per_launch(n, infos[0])
-    achieved_tf = fl / kern_s / 1e12
+    fp64_fl = fl - integer_pipe_flops(n, infos[0])
+    achieved_tf = fp64_fl / kern_s / 1e12
     peaks = json.load(open(MEASURED_PEAKS)) if os.path.exists(MEASURED_PEAKS) else {}
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     hbm_src = "measured" if "hbm_gbs" in peaks else "fallback"
@@ -764,8 +772,10 @@ def run_ours(args):
                 "frac": achieved_tf / FP64_PEAK_TFLOPS, "traffic": traffic,
                 "kernel": "pbicgstab_kernel<StencilOp>",
                 "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk/SM x 2 flop x 2.07 GHz",
-                "flops_per_launch": fl,
-                "note": "the dot products' flops count although the kernel forms them on the integer pipes",
+                "flops_per_launch": fp64_fl,
+                "note": "flops of the FP64 pipe; the dot products of the iterations run on the integer pipes",
+                "with_dot_products": {"flops_per_launch": fl, "achieved": fl / kern_s / 1e12,
+                                      "frac": fl / kern_s / 1e12 / FP64_PEAK_TFLOPS},
                 "hbm": {"achieved_gbs": gbs, "peak_gbs": hbm_peak, "frac": gbs / hbm_peak,
                         "peak_source": hbm_src, "bytes_per_iter": bpi}}
 

@@ -25,3 +25,9 @@ def test_batched_flops_of_an_unconverged_empty_batch():
     assert bench.batched_flops([], [], [], []) == 0.0
     # a system stopped before its first iteration still pays setup and residual
     assert bench.batched_flops(np.array([4]), np.array([10]), np.array([0]), np.array([0])) == 3 * 2 * 10
+
+
+def test_dot_products_on_the_integer_pipes_are_not_fp64_flops():
+    # 10^3 unknowns, 4 iterations: 8 dot products of 2 flops a row and iteration where the blocks have 512 threads
+    assert bench.integer_pipe_flops(10, {"iters": 4, "block": 512}) == 4 * 16 * 1000
+    assert bench.integer_pipe_flops(10, {"iters": 4, "block": 256}) == 0.0
