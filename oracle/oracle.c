@@ -113,12 +113,28 @@ static void spmv(const o_csr *A, const double *x, double *y, o_count *c)
     if (c) c->spmvs += 1;
 }
 
-/* (a, b) summed left to right */
+/* (a, b) summed left to right; the OpenMP build adds the threads' sums in thread
+ * order, so that a solve repeats (a reduction clause adds them as they come) */
 static double dot(int32_t n, const double *a, const double *b, o_count *c)
 {
     double acc = 0.0;
-#pragma omp parallel for schedule(static) reduction(+ : acc)
+#ifdef _OPENMP
+    enum { MOST = 1024 };
+    double part[MOST][8];   /* a line of its own for each thread's sum */
+    int threads = 1;
+#pragma omp parallel num_threads(omp_get_max_threads() < MOST ? omp_get_max_threads() : MOST)
+    {
+        double sum = 0.0;
+#pragma omp single
+        threads = omp_get_num_threads();
+#pragma omp for schedule(static) nowait
+        for (int32_t i = 0; i < n; i++) sum = sum + a[i] * b[i];
+        part[omp_get_thread_num()][0] = sum;
+    }
+    for (int t = 0; t < threads; t++) acc = acc + part[t][0];
+#else
     for (int32_t i = 0; i < n; i++) acc = acc + a[i] * b[i];
+#endif
     if (c) c->flops += 2.0 * n;
     return acc;
 }
